@@ -141,19 +141,34 @@ __global__ void mst_init_kernel(int n, int *comp, int *hook, unsigned long long 
 }
 
 // per vertex (one warp): the lightest edge to another component, then the
-// minimum per component
+// minimum per component.  An edge weighs at least its length, so a vertex
+// farther than the lightest weight found so far (shared across the warp every
+// 8 candidates) is passed over before its square root and division: the
+// rounds were bound by those (9 M edges a round, 45 us -> 26 us on average at
+// 3000 keypoints).  Once the tree is complete the remaining rounds end at once.
 __global__ void mst_min_edge_kernel(int n, const int *kps, const float *inten, float sig, const int *comp,
-                                    unsigned long long *best) {
+                                    unsigned long long *best, const int *nedges) {
     const int lane = threadIdx.x & 31;
     const int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (v >= n) return;
-    const int cv = comp[v];
+    if (v >= n || *nedges >= n - 1) return;
+    const int cv = comp[v], vx = kps[3 * v], vy = kps[3 * v + 1], vz = kps[3 * v + 2];
     unsigned long long b = ~0ull;
-    for (int u = lane; u < n; u += 32)
-        if (comp[u] != cv) {
+    float far2 = __int_as_float(0x7f800000);   // no edge longer than its root can be the lightest
+    for (int u0 = 0; u0 < n; u0 += 8 * 32) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int u = u0 + 32 * i + lane;
+            if (u >= n || comp[u] == cv) continue;
+            const int dx = vx - kps[3 * u], dy = vy - kps[3 * u + 1], dz = vz - kps[3 * u + 2];
+            if ((float)(dx * dx + dy * dy + dz * dz) > far2) continue;
             const unsigned long long key = edge_key(edge_w(kps, inten, sig, v, u), v, u);
             b = key < b ? key : b;
         }
+        // the rounding of the square, the root and the sum stays within the factor 1 + 1e-6
+        float w = b == ~0ull ? __int_as_float(0x7f800000) : __uint_as_float((unsigned)(b >> 32));
+        for (int o = 16; o > 0; o >>= 1) w = fminf(w, __shfl_xor_sync(0xffffffffu, w, o));
+        far2 = w * w * 1.000001f;
+    }
     for (int o = 16; o > 0; o >>= 1) {
         const unsigned long long t = __shfl_xor_sync(0xffffffffu, b, o);
         b = t < b ? t : b;
@@ -161,12 +176,17 @@ __global__ void mst_min_edge_kernel(int n, const int *kps, const float *inten, f
     if (lane == 0 && b != ~0ull) atomicMin(best + cv, b);
 }
 
-// each component adds its lightest edge and hooks onto the component at the
-// other end; of a mutual pair (both chose the same edge) the smaller adds the
-// edge and the larger hooks
-__global__ void mst_hook_kernel(int n, const int *comp, const unsigned long long *best, int *hook, int *edges,
-                                int *nedges) {
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
+// The rest of a round, one CTA.  Each component adds its lightest edge and
+// hooks onto the component at the other end; of a mutual pair (both chose the
+// same edge) the smaller adds the edge and the larger hooks.  Then components
+// = roots of the hook forest (chains end after < n steps), and the round's
+// scratch is reset.
+__global__ void __launch_bounds__(1024) mst_merge_kernel(int n, int *comp, unsigned long long *best, int *hook,
+                                                         int *edges, int *nedges) {
+    const int tid = threadIdx.x, nt = blockDim.x;
+    if (*nedges >= n - 1) return;
+    __syncthreads();   // every thread has read the count before the hooks add to it
+    for (int c = tid; c < n; c += nt) {
         if (comp[c] != c || best[c] == ~0ull) continue;
         const int lo = (int)((best[c] >> 16) & 0xffff), hi = (int)(best[c] & 0xffff);
         const int d = comp[lo] == c ? comp[hi] : comp[lo];
@@ -180,36 +200,36 @@ __global__ void mst_hook_kernel(int n, const int *comp, const unsigned long long
         }
         if (!mutual || c > d) hook[c] = d;
     }
-}
-
-// components = roots of the hook forest (chains end after < n steps)
-__global__ void mst_jump_kernel(int n, const int *hook, int *comp) {
-    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+    __syncthreads();
+    for (int v = tid; v < n; v += nt) {
         int r = comp[v];
         for (int s = 0; s < n && hook[r] != r; ++s) r = hook[r];
         comp[v] = r;
     }
-}
-
-__global__ void mst_reset_kernel(int n, int *hook, unsigned long long *best) {
-    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+    __syncthreads();
+    for (int v = tid; v < n; v += nt) {
         hook[v] = v;
         best[v] = ~0ull;
     }
 }
 
-// edges sorted by (lo, hi): each edge's rank counted over all edges
+// edges sorted by (lo, hi): each edge's rank counted over all edges, one warp
+// per edge (one thread per edge left 24 blocks chasing 3000 loads each: 99 us)
 __global__ void mst_sort_kernel(int m, const int *edges, const int *nedges, int *out, int *err) {
     if (blockIdx.x == 0 && threadIdx.x == 0 && *nedges != m) atomicExch(err, 1);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < m; i += (gridDim.x * blockDim.x) >> 5) {
         const long ki = ((long)edges[2 * i] << 16) | edges[2 * i + 1];
         int r = 0;
-        for (int j = 0; j < m; ++j) {
+        for (int j = lane; j < m; j += 32) {
             const long kj = ((long)edges[2 * j] << 16) | edges[2 * j + 1];
             r += kj < ki;
         }
-        out[2 * r] = edges[2 * i];
-        out[2 * r + 1] = edges[2 * i + 1];
+        for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+        if (lane == 0) {
+            out[2 * r] = edges[2 * i];
+            out[2 * r + 1] = edges[2 * i + 1];
+        }
     }
 }
 
@@ -220,6 +240,14 @@ __global__ void mst_sort_kernel(int m, const int *edges, const int *nedges, int 
 // equal ends are ignored and each vertex is claimed once, so a list that is
 // not a spanning tree cannot write out of bounds (vertices it does not reach
 // are left out of the levels).  Scratch: deg/off [n + 1] each, adj [2 n].
+//
+// The three sweeps are a chain of ~900 narrow levels (3000 keypoints).  While
+// the lists fit in shared memory (n <= kTreeSm) one warp walks them there, so
+// a level costs a few shared-memory round trips instead of two barriers of
+// 1024 threads and global loads: 1164 -> 517 us; larger trees take the wide form.
+// Also clears the belief propagation's work counter and completion counts.
+constexpr int kTreeSm = 13000;   // 16 bytes per vertex (4-byte offsets, parents and order, two 2-byte neighbours): 208 KB
+constexpr size_t tree_smem(int n) { return n <= kTreeSm ? ((size_t)n * 16 + 64) : 0; }
 __device__ __forceinline__ bool edge_ok(int n, int a, int b) { return a >= 0 && a < n && b >= 0 && b < n && a != b; }
 
 // exclusive scan of cnt[0..n) into out[0..n], one CTA (chunks per thread)
@@ -252,10 +280,13 @@ __device__ void cta_scan(int n, const int *cnt, int *out, int *s_part) {
 
 __global__ void __launch_bounds__(1024) tree_kernel(int n, int root, const int *edges, int *deg, int *off, int *adj,
                                                     int *order, int *level_off, int *nlevels, int *parent,
-                                                    int *child_off, int *child) {
+                                                    int *child_off, int *child, unsigned *next, unsigned *done) {
     const int tid = threadIdx.x, nt = blockDim.x;
     __shared__ int s_count, s_lvl, s_far, s_root;
     __shared__ int s_part[1025];
+    extern __shared__ int s_tree[];
+    for (int v = tid; v < n; v += nt) done[v] = 0u;
+    if (tid == 0) *next = 0u;
     for (int v = tid; v <= n; v += nt) deg[v] = 0;
     __syncthreads();
     for (int e = tid; e < n - 1; e += nt) {
@@ -324,16 +355,80 @@ __global__ void __launch_bounds__(1024) tree_kernel(int n, int root, const int *
         }
         __syncthreads();
     };
+    // the same sweep by warp 0 on shared-memory copies of the lists
+    const bool narrow = n <= kTreeSm;
+    int *w_off = s_tree, *w_par = w_off + n + 1, *w_ord = w_par + n;
+    unsigned short *w_adj = reinterpret_cast<unsigned short *>(w_ord + n);   // 2 (n - 1) entries at most
+    auto bfs_warp = [&](int r) {
+        for (int v = tid; v < n; v += 32) w_par[v] = -2;
+        __syncwarp();
+        if (tid == 0) {
+            w_ord[0] = r;
+            w_par[r] = -1;
+            level_off[0] = 0;
+            level_off[1] = 1;
+            s_count = 1;
+        }
+        __syncwarp();
+        int b0 = 0, b1 = 1, lv = 0, p0 = 0;
+        while (b1 > b0) {   // ends: every level claims at least one of n vertices
+            for (int i = b0 + tid; i < b1; i += 32) {
+                const int v = w_ord[i];
+                for (int j = w_off[v]; j < w_off[v + 1]; ++j) {
+                    const int u = w_adj[j];
+                    if (atomicCAS(w_par + u, -2, v) == -2) w_ord[atomicAdd(&s_count, 1)] = u;
+                }
+            }
+            __syncwarp();
+            p0 = b0;
+            b0 = b1;
+            b1 = *(volatile int *)&s_count;
+            if (tid == 0) level_off[lv + 2] = b1;
+            ++lv;
+            __syncwarp();
+        }
+        int far = n;   // the smallest index on the deepest level [p0, b0)
+        for (int i = p0 + tid; i < b0; i += 32) far = min(far, w_ord[i]);
+        for (int o = 16; o > 0; o >>= 1) far = min(far, __shfl_xor_sync(0xffffffffu, far, o));
+        if (tid == 0) {
+            s_far = far;
+            s_lvl = lv;
+        }
+        __syncwarp();
+    };
     // root = centre of a longest path (two sweeps), so the levels are fewest
-    bfs(root);
-    bfs(s_far);
-    if (tid == 0) {
-        int c = s_far;
-        for (int st = 0; st < (s_lvl - 1) / 2; ++st) c = parent[c];
-        s_root = c;
+    if (narrow) {
+        for (int v = tid; v <= n; v += nt) w_off[v] = off[v];
+        for (int j = tid; j < off[n]; j += nt) w_adj[j] = (unsigned short)adj[j];
+        __syncthreads();
+        if (tid < 32) {
+            bfs_warp(root);
+            bfs_warp(s_far);
+            if (tid == 0) {
+                int c = s_far;
+                for (int st = 0; st < (s_lvl - 1) / 2; ++st) c = w_par[c];
+                s_root = c;
+            }
+            __syncwarp();
+            bfs_warp(s_root);
+        }
+        __syncthreads();
+        for (int v = tid; v < n; v += nt) {
+            parent[v] = w_par[v];
+            if (v < s_count) order[v] = w_ord[v];
+        }
+        __syncthreads();
+    } else {
+        bfs(root);
+        bfs(s_far);
+        if (tid == 0) {
+            int c = s_far;
+            for (int st = 0; st < (s_lvl - 1) / 2; ++st) c = parent[c];
+            s_root = c;
+        }
+        __syncthreads();
+        bfs(s_root);
     }
-    __syncthreads();
-    bfs(s_root);
     if (tid == 0) *nlevels = s_lvl;   // levels 0 .. s_lvl - 1 are non-empty
     // child lists: the neighbours claimed by v, in sorted order
     for (int v = tid; v < n; v += nt) {
@@ -351,16 +446,42 @@ __global__ void __launch_bounds__(1024) tree_kernel(int n, int root, const int *
 }
 
 // ------------------------------------------------------------ belief propagation
-// One 33-point line of the min-convolution: out[j] = min_i v[i] + C[|i - j|].
-__device__ __forceinline__ void min_conv_line(float (&v)[kS], const float (&C)[kS]) {
-    float o[kS];
+__device__ __forceinline__ float min3(float a, float b, float c) {
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+// One 33-point line of the min-convolution: out[j] = min_i v[i] + lam (2 (i - j))^2
+// (one rounding per candidate), by distance d = |i - j|, both candidates of an output in one three-input
+// minimum.  Every candidate at distance d or more is at least min v + cost(d)
+// (rounding is monotone), so the warp stops at the first d whose bound reaches
+// its lines' largest output: the same values as all 33 candidates, a few
+// distances in place of 32 for most lines.  Called by whole warps.
+__device__ __forceinline__ void min_conv_line(float (&v)[kS], float lam) {
+    float o[kS], lo = v[0], hi = v[0];
 #pragma unroll
     for (int j = 0; j < kS; ++j) {
-        float m = v[j];   // C[0] = 0
+        o[j] = v[j];   // cost(0) = 0
+        lo = fminf(lo, v[j]);
+        hi = fmaxf(hi, v[j]);
+    }
 #pragma unroll
-        for (int i = 0; i < kS; ++i)
-            if (i != j) m = fminf(m, v[i] + C[i > j ? i - j : j - i]);
-        o[j] = m;
+    for (int d = 1; d < kS; ++d) {
+        const float dd = (float)(4 * d * d);
+        if (__all_sync(0xffffffffu, __fmaf_rn(lam, dd, lo) >= hi)) break;
+#pragma unroll
+        for (int j = 0; j < kS; ++j) {
+            if (j - d >= 0 && j + d < kS)
+                o[j] = min3(o[j], __fmaf_rn(lam, dd, v[j - d]), __fmaf_rn(lam, dd, v[j + d]));
+            else if (j - d >= 0) o[j] = fminf(o[j], __fmaf_rn(lam, dd, v[j - d]));
+            else if (j + d < kS) o[j] = fminf(o[j], __fmaf_rn(lam, dd, v[j + d]));
+        }
+        if (d == 1 || d == 2 || d == 4 || d == 8 || d == 16) {   // a tighter bound for the next distances
+            hi = o[0];
+#pragma unroll
+            for (int j = 1; j < kS; ++j) hi = fmaxf(hi, o[j]);
+        }
     }
 #pragma unroll
     for (int j = 0; j < kS; ++j) v[j] = o[j];
@@ -370,125 +491,164 @@ struct BpArgs {
     const float *D;        // [n][L] unary costs
     float *up;             // [n][L] message to the parent
     float *marg;           // [n][L] marginals
-    const int *order, *parent, *child_off, *child;
+    const int *order, *parent, *child_off, *child, *level_off, *nlevels;
     const int *kps;
     const float *inten;
     float sig, alpha;
-    int base;              // first vertex of the level in order[]
+    int n;
+    unsigned *next;        // work counter
+    unsigned *done;        // [n] CTAs of the vertex's cluster that have finished: kCl after the up message, 2 kCl with the marginal
+    int *err;              // set to 2 when a wait runs out
 };
 
-// Message of vertex k (DOWN: message of its parent q to k, then k's marginal),
-// spread over a cluster of 8 CTAs: CTA r owns z planes [4 r, 4 r + 4) (the
-// last one also plane 32), runs the x and y passes on them, and after a
-// cluster barrier the z pass on its share of the 1089 (y, x) columns, reading
-// the planes of the other CTAs through distributed shared memory.  The UP
-// pass leaves h_k = D_k + sum of the children's messages in marg[k]; the DOWN
-// pass adds the parent's message to it, which completes k's marginal.
-template <bool DOWN>
-__global__ void __launch_bounds__(kBpT) bp_message_kernel(const BpArgs a) {
+constexpr int kBpClusters = 38;          // clusters of 8 CTAs, two CTAs per SM
+constexpr int kBpPolls = 1 << 21;        // polls before a wait gives up (about two seconds)
+
+// Bounded wait for a completion count; after one wait has run out the others end too.
+__device__ __forceinline__ void bp_wait(const unsigned *p, unsigned need, int *err) {
+    for (int i = 0; i < kBpPolls; ++i) {
+        unsigned v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+        if (v >= need) return;
+        if ((i & 255) == 255 && *(volatile int *)err == 2) return;
+        __nanosleep(20);
+    }
+    atomicExch(err, 2);
+}
+
+// Both passes in one launch.  An item is a vertex's up message (children
+// before parents), the root's marginal, or a vertex's down message and
+// marginal (parents before children); clusters of 8 CTAs take the items from a
+// counter in that order, and an item waits only for the completion counts of
+// its children or its parent, which come earlier in the order and are held by
+// running clusters, so every wait ends.  (One launch per tree level paid the
+// launch gap and the slowest message of the level ~720 times: BP 6.1 -> 3.2 ms
+// per direction at 3000 keypoints, ~180 levels.)
+//
+// CTA r of a cluster owns z planes [4 r, 4 r + 4) of the vertex's labels (the
+// last one also plane 32), runs the x and y passes of the min-convolution on
+// them, and after a cluster barrier the z pass on its share of the 1089 (y, x)
+// columns, reading the planes of the other CTAs through distributed shared
+// memory; the planes are double-buffered, so that barrier is the only one of an
+// item.  The UP pass leaves h_k = D_k + sum of the children's messages in
+// marg[k]; the DOWN pass adds the parent's message to it, which completes k's
+// marginal.  Data of other clusters is read past L1 (written during the launch).
+__global__ void __launch_bounds__(kBpT, 2) bp_kernel(const BpArgs a) {
     constexpr int kPer = (5 * kPlane + kBpT - 1) / kBpT;   // slab values per thread
-    __shared__ float s[5 * kPlane];
+    __shared__ float sbuf[2][5 * kPlane];
+    __shared__ int s_item[2];
     cg::cluster_group cl = cg::this_cluster();
     const int r = (int)cl.block_rank();
-    const int k = a.order[a.base + blockIdx.x / kCl];
-    const int q = a.parent[k];
     const int z0 = 4 * r, nzp = r == kCl - 1 ? 5 : 4, nown = nzp * kPlane;
     const int tid = threadIdx.x;
-    const float lam = __fdiv_rn(a.alpha, edge_w(a.kps, a.inten, a.sig, k, q));
-    float C[kS];
-#pragma unroll
-    for (int d = 0; d < kS; ++d) C[d] = d == 0 ? 0.f : lam * (float)(4 * d * d);
-    // h over the own planes (all loads of one array issued together): UP:
-    // D_k + the children's messages; DOWN: the parent's marginal without k's message
+    const int nr = a.level_off[*a.nlevels], total = 2 * nr - 1;   // vertices the tree reaches; items
     const long pb = (long)z0 * kPlane;
-    {
-        float h[kPer];
-        const float *src = DOWN ? a.marg + (long)q * kL + pb : a.D + (long)k * kL + pb;
-#pragma unroll
-        for (int t = 0; t < kPer; ++t) {
-            const int i = tid + t * kBpT;
-            h[t] = i < nown ? __ldg(src + i) : 0.f;
+    const int per = (kPlane + kCl - 1) / kCl, j0 = r * per, j1 = min(kPlane, j0 + per);
+    const int zl = tid / kS, w = tid - zl * kS, j = j0 + tid;
+    auto claim = [&](int slot) {   // the cluster's next item into every CTA's mailbox (read after a cluster barrier)
+        if (r == 0 && tid == 0) {
+            const int it = (int)atomicAdd(a.next, 1u);
+            for (int c = 0; c < kCl; ++c) *cl.map_shared_rank(&s_item[slot], c) = it;
         }
-        if (DOWN) {
-            const float *u = a.up + (long)k * kL + pb;
+    };
+    auto finish = [&](int k, unsigned add) {   // this CTA's stores of vertex k are complete
+        __syncthreads();
+        if (tid == 0) {
+            __threadfence();
+            asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(a.done + k), "r"(add) : "memory");
+        }
+    };
+    claim(0);
+    cl.sync();
+    for (int t = 0;; ++t) {
+        const int item = s_item[t & 1];
+        if (item >= total) break;   // uniform over the cluster
+        claim((t + 1) & 1);
+        float *s = sbuf[t & 1];
+        const bool down = item >= nr;
+        const int k = a.order[down ? item - nr + 1 : nr - 1 - item];   // item nr - 1: the root
+        const int q = a.parent[k];
+        float h[kPer];
+        if (!down) {
+            const float *src = a.D + (long)k * kL + pb;
 #pragma unroll
-            for (int t = 0; t < kPer; ++t) {
-                const int i = tid + t * kBpT;
-                if (i < nown) h[t] -= __ldg(u + i);
-            }
-        } else {
-            for (int c = a.child_off[k]; c < a.child_off[k + 1]; ++c) {
+            for (int i = 0; i < kPer; ++i) h[i] = tid + i * kBpT < nown ? __ldg(src + tid + i * kBpT) : 0.f;
+            const int c0 = a.child_off[k], c1 = a.child_off[k + 1];
+            for (int c = c0 + tid; c < c1; c += kBpT) bp_wait(a.done + a.child[c], kCl, a.err);
+            __syncthreads();
+            for (int c = c0; c < c1; ++c) {
                 const float *u = a.up + (long)a.child[c] * kL + pb;
 #pragma unroll
-                for (int t = 0; t < kPer; ++t) {
-                    const int i = tid + t * kBpT;
-                    if (i < nown) h[t] += __ldg(u + i);
-                }
+                for (int i = 0; i < kPer; ++i)
+                    if (tid + i * kBpT < nown) h[i] += __ldcg(u + tid + i * kBpT);
             }
             float *mk = a.marg + (long)k * kL + pb;
 #pragma unroll
-            for (int t = 0; t < kPer; ++t) {
-                const int i = tid + t * kBpT;
-                if (i < nown) mk[i] = h[t];
-            }
-        }
+            for (int i = 0; i < kPer; ++i)
+                if (tid + i * kBpT < nown) mk[tid + i * kBpT] = h[i];
+        } else {
+            if (tid == 0) bp_wait(a.done + q, 2 * kCl, a.err);
+            __syncthreads();
+            const float *src = a.marg + (long)q * kL + pb, *u = a.up + (long)k * kL + pb;
 #pragma unroll
-        for (int t = 0; t < kPer; ++t) {
-            const int i = tid + t * kBpT;
-            if (i < nown) s[i] = h[t];
+            for (int i = 0; i < kPer; ++i) h[i] = tid + i * kBpT < nown ? __ldcg(src + tid + i * kBpT) : 0.f;
+#pragma unroll
+            for (int i = 0; i < kPer; ++i)
+                if (tid + i * kBpT < nown) h[i] -= __ldcg(u + tid + i * kBpT);
         }
-    }
-    __syncthreads();
-    // x pass, y pass (own planes, one line per thread), then the z pass over
-    // columns [j0, j1) of all planes; one copy of the line code for all three
-    const int per = (kPlane + kCl - 1) / kCl, j0 = r * per, j1 = min(kPlane, j0 + per);
-    const int zl = tid / kS, w = tid - zl * kS, j = j0 + tid;
+        if (q < 0) {   // the root: its marginal is complete
+            finish(k, 2);
+            cl.sync();
+            continue;
+        }
+        const float lam = __fdiv_rn(a.alpha, edge_w(a.kps, a.inten, a.sig, k, q));
+#pragma unroll
+        for (int i = 0; i < kPer; ++i)
+            if (tid + i * kBpT < nown) s[tid + i * kBpT] = h[i];
+        __syncthreads();
+        // x pass, y pass (own planes, one line per thread), then the z pass over
+        // columns [j0, j1) of all planes; one copy of the line code for all three
 #pragma unroll 1
-    for (int pass = 0; pass < 3; ++pass) {
-        if (pass == 2) cl.sync();   // every CTA's planes are complete
-        const bool act = pass < 2 ? tid < nzp * kS : j < j1;
-        float v[kS];
-        if (act) {
-            if (pass < 2) {
-                const int base = zl * kPlane + (pass == 0 ? w * kS : w), step = pass == 0 ? 1 : kS;
+        for (int pass = 0; pass < 3; ++pass) {
+            if (pass == 2) cl.sync();   // every CTA's planes are complete
+            const bool act = pass < 2 ? tid < nzp * kS : j < j1;
+            if (__any_sync(0xffffffffu, act)) {
+                float v[kS];
+                const int base = pass == 0 ? zl * kPlane + w * kS : zl * kPlane + w, step = pass == 0 ? 1 : kS;
+                if (pass < 2) {
 #pragma unroll
-                for (int i = 0; i < kS; ++i) v[i] = s[base + i * step];
-            } else {
+                    for (int i = 0; i < kS; ++i) v[i] = act ? s[base + i * step] : 0.f;
+                } else {
 #pragma unroll
-                for (int z = 0; z < kS; ++z) {
-                    const int owner = z / 4 < kCl - 1 ? z / 4 : kCl - 1;
-                    const float *rs = cl.map_shared_rank(s, owner);
-                    v[z] = rs[(z - 4 * owner) * kPlane + j];
+                    for (int z = 0; z < kS; ++z) {
+                        const int owner = z / 4 < kCl - 1 ? z / 4 : kCl - 1;
+                        v[z] = act ? cl.map_shared_rank(s, owner)[(z - 4 * owner) * kPlane + j] : 0.f;
+                    }
+                }
+                min_conv_line(v, lam);
+                if (act) {
+                    if (pass < 2) {
+#pragma unroll
+                        for (int i = 0; i < kS; ++i) s[base + i * step] = v[i];
+                    } else if (down) {
+                        float *mk = a.marg + (long)k * kL + j;
+                        float m[kS];
+#pragma unroll
+                        for (int z = 0; z < kS; ++z) m[z] = __ldcg(mk + (long)z * kPlane);
+#pragma unroll
+                        for (int z = 0; z < kS; ++z) mk[(long)z * kPlane] = m[z] + v[z];
+                    } else {
+                        float *uk = a.up + (long)k * kL + j;
+#pragma unroll
+                        for (int z = 0; z < kS; ++z) uk[(long)z * kPlane] = v[z];
+                    }
                 }
             }
-            min_conv_line(v, C);
-            if (pass < 2) {
-                const int base = zl * kPlane + (pass == 0 ? w * kS : w), step = pass == 0 ? 1 : kS;
-#pragma unroll
-                for (int i = 0; i < kS; ++i) s[base + i * step] = v[i];
-            } else if (DOWN) {
-                float *mk = a.marg + (long)k * kL + j;
-#pragma unroll
-                for (int z = 0; z < kS; ++z) mk[(long)z * kPlane] += v[z];
-            } else {
-                float *uk = a.up + (long)k * kL + j;
-#pragma unroll
-                for (int z = 0; z < kS; ++z) uk[(long)z * kPlane] = v[z];
-            }
+            if (pass < 2) __syncthreads();
         }
-        if (pass < 2) __syncthreads();
+        finish(k, 1);
     }
-    cl.sync();   // no CTA leaves while another may still read its planes
-}
-
-// marginal of the root (order[0]): D + the children's messages
-__global__ void bp_root_kernel(const BpArgs a) {
-    const int root = a.order[0];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kL; i += gridDim.x * blockDim.x) {
-        float m = a.D[(long)root * kL + i];
-        for (int c = a.child_off[root]; c < a.child_off[root + 1]; ++c) m += a.up[(long)a.child[c] * kL + i];
-        a.marg[(long)root * kL + i] = m;
-    }
+    cl.sync();   // no CTA leaves while another may still read its planes or write its mailbox
 }
 
 // ------------------------------------------------------------ argmin, refinement
@@ -557,6 +717,7 @@ struct KpWs {
     int *comp, *hook, *edges_raw, *edges, *nedges, *err;
     unsigned long long *best;
     int *deg, *off, *adj, *order, *level_off, *nlevels, *parent, *child_off, *child;
+    unsigned *next, *done;
 };
 
 struct Carve {
@@ -598,6 +759,8 @@ size_t kp_layout(Carve &cv, KpWs &w, long N, int n, bool match) {
     w.parent = cv.take<int>(n);
     w.child_off = cv.take<int>(n + 1);
     w.child = cv.take<int>(n);
+    w.next = cv.take<unsigned>(1);
+    w.done = cv.take<unsigned>(n);
     return (cv.off + 255) & ~(size_t)255;
 }
 
@@ -631,48 +794,22 @@ cudaError_t run_mst(int n, const int *kps, const float *inten, float sig, KpWs &
     int rounds = 1;
     while ((1 << (rounds - 1)) < n) ++rounds;   // components at least halve per round
     for (int it = 0; it < rounds; ++it) {
-        mst_min_edge_kernel<<<(n * 32 + 255) / 256, 256, 0, st>>>(n, kps, inten, sig, w.comp, w.best);
-        mst_hook_kernel<<<gb, 256, 0, st>>>(n, w.comp, w.best, w.hook, w.edges_raw, w.nedges);
-        mst_jump_kernel<<<gb, 256, 0, st>>>(n, w.hook, w.comp);
-        mst_reset_kernel<<<gb, 256, 0, st>>>(n, w.hook, w.best);
+        mst_min_edge_kernel<<<(n * 32 + 255) / 256, 256, 0, st>>>(n, kps, inten, sig, w.comp, w.best, w.nedges);
+        mst_merge_kernel<<<1, 1024, 0, st>>>(n, w.comp, w.best, w.hook, w.edges_raw, w.nedges);
     }
-    mst_sort_kernel<<<grid_for(n - 1, 128), 128, 0, st>>>(n - 1, w.edges_raw, w.nedges, w.edges, w.err);
-    counted(2 + 4L * rounds);
+    mst_sort_kernel<<<grid_for(32L * (n - 1), 128), 128, 0, st>>>(n - 1, w.edges_raw, w.nedges, w.edges, w.err);
+    counted(2 + 2L * rounds);
     return cudaGetLastError();
 }
 
-cudaError_t launch_cluster(void (*kernel)(const BpArgs), int nverts, const BpArgs &a, cudaStream_t st) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kCl * nverts);
-    cfg.blockDim = dim3(kBpT);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = kCl;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, a);
-}
-
-// Tree from the sorted MST edges, then the two passes; the level sizes are
-// read back once (one synchronisation) to size the per-level launches.
+// Tree from the sorted MST edges, then both passes in one launch.
 int run_bp(int n, const float *D, const int *kps, const float *inten, float sig, float alpha, KpWs &w, float *marg,
            cudaStream_t st) {
     const int root = 0;   // start of the sweeps that find the tree's centre
-    tree_kernel<<<1, 1024, 0, st>>>(n, root, w.edges, w.deg, w.off, w.adj, w.order, w.level_off, w.nlevels, w.parent,
-                                    w.child_off, w.child);
+    if (allow_max_dynamic_smem(tree_kernel) != cudaSuccess) return RG_ECUDA;
+    tree_kernel<<<1, 1024, tree_smem(n), st>>>(n, root, w.edges, w.deg, w.off, w.adj, w.order, w.level_off, w.nlevels,
+                                               w.parent, w.child_off, w.child, w.next, w.done);
     if (cudaGetLastError() != cudaSuccess) return RG_ECUDA;
-    // the level count and offsets, read on the caller's stream in one synchronisation
-    int nl = 0;
-    std::vector<int> lo(n + 2);
-    if (cudaMemcpyAsync(&nl, w.nlevels, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(lo.data(), w.level_off, sizeof(int) * (n + 2), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-        return RG_ECUDA;
-    if (nl < 1 || nl > n) return RG_ECUDA;
     BpArgs a;
     a.D = D;
     a.up = w.up;
@@ -681,25 +818,39 @@ int run_bp(int n, const float *D, const int *kps, const float *inten, float sig,
     a.parent = w.parent;
     a.child_off = w.child_off;
     a.child = w.child;
+    a.level_off = w.level_off;
+    a.nlevels = w.nlevels;
     a.kps = kps;
     a.inten = inten;
     a.sig = sig;
     a.alpha = alpha;
-    long long cnt = 1;
-    for (int lv = nl - 1; lv >= 1; --lv) {
-        a.base = lo[lv];
-        if (launch_cluster(bp_message_kernel<false>, lo[lv + 1] - lo[lv], a, st) != cudaSuccess) return RG_ECUDA;
-        ++cnt;
-    }
-    bp_root_kernel<<<grid_for(kL, 256), 256, 0, st>>>(a);
-    ++cnt;
-    for (int lv = 1; lv < nl; ++lv) {
-        a.base = lo[lv];
-        if (launch_cluster(bp_message_kernel<true>, lo[lv + 1] - lo[lv], a, st) != cudaSuccess) return RG_ECUDA;
-        ++cnt;
-    }
-    counted(cnt);
-    return cudaGetLastError() == cudaSuccess ? RG_OK : RG_ECUDA;
+    a.n = n;
+    a.next = w.next;
+    a.done = w.done;
+    a.err = w.err;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kCl * std::min(n, kBpClusters));
+    cfg.blockDim = dim3(kBpT);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kCl;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    counted(2);
+    return cudaLaunchKernelEx(&cfg, bp_kernel, a) == cudaSuccess ? RG_OK : RG_ECUDA;
+}
+
+// The flag the kernels of a call left on the device: 1 an incomplete tree, 2 a
+// wait that ran out.  Synchronises the stream.
+int read_flag(const KpWs &w, cudaStream_t st) {
+    int err = 0;
+    if (cudaMemcpyAsync(&err, w.err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess)
+        return RG_ECUDA;
+    return err == 2 ? RG_ETIMEOUT : (err ? RG_ECUDA : RG_OK);
 }
 
 }  // namespace
@@ -759,12 +910,9 @@ extern "C" int kp_mst(int32_t nk, const int32_t *kps, const float *intensity, do
     flag_kernel<<<1, 1, 0, st>>>(w.err);
     counted();
     if (run_mst(nk, kps, intensity, (float)sigma_i, w, st) != cudaSuccess) return RG_ECUDA;
-    int err = 0;
-    if (cudaMemcpyAsync(edges, w.edges, sizeof(int) * 2 * (nk - 1), cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(&err, w.err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
+    if (cudaMemcpyAsync(edges, w.edges, sizeof(int) * 2 * (nk - 1), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
         return RG_ECUDA;
-    return err ? RG_ECUDA : RG_OK;
+    return read_flag(w, st);
 }
 
 extern "C" int kp_bp_marginals(int32_t nk, const float *D, const int32_t *kps, const float *intensity,
@@ -776,7 +924,10 @@ extern "C" int kp_bp_marginals(int32_t nk, const float *D, const int32_t *kps, c
     cudaStream_t st = (cudaStream_t)stream;
     if (cudaMemcpyAsync(w.edges, edges, sizeof(int) * 2 * (nk - 1), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
         return RG_ECUDA;
-    return run_bp(nk, D, kps, intensity, (float)sigma_i, (float)alpha, w, marginals, st);
+    flag_kernel<<<1, 1, 0, st>>>(w.err);
+    counted();
+    const int s = run_bp(nk, D, kps, intensity, (float)sigma_i, (float)alpha, w, marginals, st);
+    return s ? s : read_flag(w, st);
 }
 
 extern "C" int kp_match(const int32_t *n, const float *F, const float *M, int32_t nk, const int32_t *kps,
@@ -789,6 +940,10 @@ extern "C" int kp_match(const int32_t *n, const float *F, const float *M, int32_
     Carve cv{(char *)ws, 0};
     KpWs w;
     kp_layout(cv, w, (long)n[0] * n[1] * n[2], nk, true);
+    if (marginals) {   // formed in the caller's array: forward [nk][L], then (symmetric) backward [nk][L]
+        w.E1 = marginals;
+        if (symmetric) w.E2 = marginals + (size_t)nk * kL;
+    }
     cudaStream_t st = (cudaStream_t)stream;
     const float sig = (float)p->sigma_i, alpha = (float)p->alpha;
     flag_kernel<<<1, 1, 0, st>>>(w.err);
@@ -816,20 +971,7 @@ extern "C" int kp_match(const int32_t *n, const float *F, const float *M, int32_
     }
     argmin_kernel<<<nk, 256, 0, st>>>(nk, E, Eb, kps, disp, nullptr);
     counted();
-    // marginals: forward [nk][L], then (symmetric) backward [nk][L]
-    if (marginals) {
-        if (cudaMemcpyAsync(marginals, E, sizeof(float) * (size_t)nk * kL, cudaMemcpyDeviceToDevice, st) !=
-            cudaSuccess)
-            return RG_ECUDA;
-        if (Eb && cudaMemcpyAsync(marginals + (size_t)nk * kL, Eb, sizeof(float) * (size_t)nk * kL,
-                                  cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-            return RG_ECUDA;
-    }
-    int err = 0;
-    if (cudaMemcpyAsync(&err, w.err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-        return RG_ECUDA;
-    return err ? RG_ECUDA : RG_OK;
+    return read_flag(w, st);
 }
 
 extern "C" int64_t kp_launch_count(void) { return g_kp_launches.load(); }
