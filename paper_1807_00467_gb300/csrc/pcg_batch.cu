@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(kNT, 1) pcg_batch_kernel(const __grid_constant
                 for (int bid = (r - A.vccOff[p]) * kVccPer + v, e = min(bid - v + kVccPer, P.nvcc); bid < e;
                      bid += kVccRun) {
                     const VBlock b = warp_block(tid % vcck::NC, bid, nb[0], nb[1], nb[2], 1 + v, vcck::NC);
-                    vcck::vcc_cell_body<1>(P.b.vcc, b, reinterpret_cast<vcck::VccSmem *>(smem)[v]);
+                    vcck::vcc_cell_body<1, float>(P.b.vcc, b, reinterpret_cast<vcck::VccSmem<float> *>(smem)[v]);
                 }
             } else {
                 const int v = tid / nodek::NT;
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(kNT, 1) pcg_batch_kernel(const __grid_constant
 
 size_t batch_smem(const KArgs &A) {
     size_t s = std::max(sizeof(pcgk::PcgSmem),
-                        std::max(kVccRun * sizeof(vcck::VccSmem), kNodeRun * sizeof(nodek::NodeSmem)));
+                        std::max(kVccRun * sizeof(vcck::VccSmem<float>), kNodeRun * sizeof(nodek::NodeSmem)));
     for (int p = 0; p < A.npairs; ++p) s = std::max(s, sizeof(float) * (size_t)gnpk::pc_smem(A.p[p].b.col.g).total);
     return s;
 }

@@ -1,9 +1,8 @@
 // Volume change control, Eqs. (7)-(9): gradient (and energy) of
 // sum_cells sum_{a,b,c} psi(d_abc), its Gauss-Newton product
 // sum psi''(d) (grad d . v) grad d and the diagonal of that product,
-// sum psi''(d) (d d / d u_{k,c})^2, one thread per grid cell: the body of the
-// kernels of vcc.cu, shared with the persistent batched PCG kernel
-// (pcg_batch.cu).
+// sum psi''(d) (d d / d u_{k,c})^2: the body of the kernels of vcc.cu, shared
+// with the persistent batched PCG kernel (pcg_batch.cu).
 //
 // In a cell the 64 bounds are d_abc = det[e1_a, e2_b, e3_c] = e1_a . X_bc with
 // the four x-, y- and z-edges e1_a, e2_b, e3_c (identity plus the scaled node
@@ -17,6 +16,20 @@
 // and +-(e1_a x e2_b) / g_z at the ends of e3_c (summed where two of these
 // edges share a corner).  Bounds with d <= 0 are folds: weight 0 here,
 // counted for the energy pass (the objective is then +inf).
+//
+// Bound by FP32 arithmetic: about 1700 multiply-adds a cell for the GN product
+// (60 us for 129 x 129 x 65 nodes at the ~97 three-operand FMA a clock and SM
+// that this part sustains).  The instructions around them are kept few: the
+// y-edges are taken one at a time in a rolled loop (their gradients parked in
+// shared memory), cells add to the box's nodes in place, one corner at a time
+// over the block, instead of through per-cell slots and an indexed gather, and
+// a fold is read from the least bound.  On large grids a thread holds two
+// cells, one per half of the packed f32x2 registers (TZ / 2 planes apart, their
+// nodes staged side by side), every operation serving both.  Gradient 137 ->
+// 81 us, GN product 107 -> 98 us at 129 x 129 x 65.  The one-cell form (F =
+// float: small grids, and the persistent kernel, whose block leaves fewer
+// registers) runs the same operations, each rounded by an explicit intrinsic,
+// so both give the same bits.
 #pragma once
 
 #include "common.cuh"
@@ -30,22 +43,90 @@ constexpr int TX = kVccTile[0], TY = kVccTile[1], TZ = kVccTile[2], NC = TX * TY
 constexpr int BX = TX + 1, BY = TY + 1, BZ = TZ + 1, NB = BX * BY * BZ;
 constexpr unsigned FULL = 0xffffffffu;
 
-struct V3 {
-    float x, y, z;
-};
-__device__ __forceinline__ V3 cross(const V3 &a, const V3 &b) {
-    return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
+// One cell (float) or two (float2, packed) per thread: every operation rounded once.
+__device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float add_(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub_(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float neg_(float a) { return -a; }
+__device__ __forceinline__ float2 fma_(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 mul_(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 add_(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub_(float2 a, float2 b) {
+    unsigned long long r;
+    asm("sub.rn.f32x2 %0, %1, %2;"
+        : "=l"(r)
+        : "l"(*reinterpret_cast<unsigned long long *>(&a)), "l"(*reinterpret_cast<unsigned long long *>(&b)));
+    return *reinterpret_cast<float2 *>(&r);
 }
-__device__ __forceinline__ float dot(const V3 &a, const V3 &b) { return fmaf(a.z, b.z, fmaf(a.y, b.y, a.x * b.x)); }
-__device__ __forceinline__ void axpy(float w, const V3 &x, V3 &y) {
-    y.x = fmaf(w, x.x, y.x); y.y = fmaf(w, x.y, y.y); y.z = fmaf(w, x.z, y.z);
-}
-__device__ __forceinline__ void add(const V3 &x, V3 &y) { y.x += x.x; y.y += x.y; y.z += x.z; }
+__device__ __forceinline__ float2 neg_(float2 a) { return make_float2(-a.x, -a.y); }
+template <typename F>
+__device__ __forceinline__ F bc_(float a);
+template <>
+__device__ __forceinline__ float bc_<float>(float a) { return a; }
+template <>
+__device__ __forceinline__ float2 bc_<float2>(float a) { return make_float2(a, a); }
+// f per lane
+template <typename Op>
+__device__ __forceinline__ float lanes(Op f, float a) { return f(a); }
+template <typename Op>
+__device__ __forceinline__ float2 lanes(Op f, float2 a) { return make_float2(f(a.x), f(a.y)); }
+template <typename Op>
+__device__ __forceinline__ float lanes(Op f, float a, float b) { return f(a, b); }
+template <typename Op>
+__device__ __forceinline__ float2 lanes(Op f, float2 a, float2 b) { return make_float2(f(a.x, b.x), f(a.y, b.y)); }
 
-// Packed FP32 (two lanes of f32x2: the bounds of two x-edges a = 2p, 2p + 1)
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 bc2(float a) { return make_float2(a, a); }
+template <typename F>
+struct Vec {
+    F x, y, z;
+};
+template <typename F>
+__device__ __forceinline__ Vec<F> neg_(const Vec<F> &a) { return {neg_(a.x), neg_(a.y), neg_(a.z)}; }
+// a x b, given -a
+template <typename F>
+__device__ __forceinline__ Vec<F> cross(const Vec<F> &a, const Vec<F> &na, const Vec<F> &b) {
+    return {fma_(a.y, b.z, mul_(na.z, b.y)), fma_(a.z, b.x, mul_(na.x, b.z)), fma_(a.x, b.y, mul_(na.y, b.x))};
+}
+// acc + a x b, given -a
+template <typename F>
+__device__ __forceinline__ Vec<F> cross_add(const Vec<F> &a, const Vec<F> &na, const Vec<F> &b, const Vec<F> &acc) {
+    return {fma_(a.y, b.z, fma_(na.z, b.y, acc.x)), fma_(a.z, b.x, fma_(na.x, b.z, acc.y)),
+            fma_(a.x, b.y, fma_(na.y, b.x, acc.z))};
+}
+// acc + a x b, given -b
+template <typename F>
+__device__ __forceinline__ Vec<F> cross_add_r(const Vec<F> &a, const Vec<F> &b, const Vec<F> &nb, const Vec<F> &acc) {
+    return {fma_(a.y, b.z, fma_(a.z, nb.y, acc.x)), fma_(a.z, b.x, fma_(a.x, nb.z, acc.y)),
+            fma_(a.x, b.y, fma_(a.y, nb.x, acc.z))};
+}
+template <typename F>
+__device__ __forceinline__ F dot(const Vec<F> &a, const Vec<F> &b) { return fma_(a.z, b.z, fma_(a.y, b.y, mul_(a.x, b.x))); }
+template <typename F>
+__device__ __forceinline__ F dot_add(const Vec<F> &a, const Vec<F> &b, F c) {
+    return fma_(a.z, b.z, fma_(a.y, b.y, fma_(a.x, b.x, c)));
+}
+template <typename F>
+__device__ __forceinline__ void axpy(F w, const Vec<F> &x, Vec<F> &y) {
+    y.x = fma_(w, x.x, y.x); y.y = fma_(w, x.y, y.y); y.z = fma_(w, x.z, y.z);
+}
+template <typename F>
+__device__ __forceinline__ Vec<F> scaled(const Vec<F> &a, float s) {
+    const F f = bc_<F>(s);
+    return {mul_(a.x, f), mul_(a.y, f), mul_(a.z, f)};
+}
+// 1 / d where d > 0, else 0 (a fold has weight 0)
+__device__ __forceinline__ float rcp_pos(float d) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    return d > 0.f ? r : 0.f;
+}
+
+// the smaller, NaN when either is (a NaN bound counts as a fold)
+__device__ __forceinline__ float min_nan(float a, float b) {
+    float r;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
 
 // corner offset (ox + 2 oy + 4 oz) of edge e = p + 2 q of axis `ax` at end `hi`;
 // p, q are the offsets along the other two axes in increasing axis order
@@ -53,21 +134,17 @@ __host__ __device__ constexpr int corner_of(int ax, int e, int hi) {
     return ax == 0 ? hi + 2 * (e & 1) + 4 * (e >> 1) : ax == 1 ? (e & 1) + 2 * hi + 4 * (e >> 1) : (e & 1) + 2 * (e >> 1) + 4 * hi;
 }
 
-struct Kahan32 {
-    float s = 0.f, c = 0.f;
-    __device__ __forceinline__ void add(float x) {
-        const float y = x - c;
-        const float t = s + y;
-        c = (t - s) - y;
-        s = t;
-    }
-};
-
-// shared scratch of one block of cells
+// shared scratch of one block of cells: the staged nodes (F = float2: nodes of
+// planes z and z + TZ / 2 side by side, so that a thread's two cells load
+// together), the box sums and the threads' y-edge gradients
+template <typename F>
 struct VccSmem {
-    float su[3][NB];
-    float sv[3][NB];
-    float scell[8 * 3][NC];
+    static constexpr int kLanes = (int)sizeof(F) / 4;
+    static constexpr int kPlanes = kLanes == 2 ? TZ / 2 + 1 : BZ;
+    F su[3][BX * BY * kPlanes];
+    F sv[3][BX * BY * kPlanes];
+    F g2[12][NC / kLanes];
+    float box[3][NB];
     double red[NC / 32];
     int sfold[NC / 32];
     float wmn[NC / 32], wmx[NC / 32];
@@ -75,86 +152,111 @@ struct VccSmem {
 
 // VM = 0: gradient of sum psi(d) (+ energy, folds, min / max d);
 // VM = 1: GN product along v; VM = 2: diagonal of the GN matrix.
-template <int VM>
-__device__ __forceinline__ void vcc_cell_body(const VccArgs &a, const VBlock &vb, VccSmem &sm) {
+// F = float: a block of NC threads, one cell each; F = float2: NC / 2 threads,
+// thread t the cells t and t + NC / 2.
+template <int VM, typename F>
+__device__ __forceinline__ void vcc_cell_body(const VccArgs &a, const VBlock &vb, VccSmem<F> &sm) {
     constexpr bool GN = VM == 1, DG = VM == 2;
-    float (&su)[3][NB] = sm.su;
-    float (&sv)[3][NB] = sm.sv;
-    float (&scell)[8 * 3][NC] = sm.scell;
+    constexpr int CPT = VccSmem<F>::kLanes, NTH = NC / CPT;   // cells per thread, threads
     const int tid = vb.tid;
     const int mx = a.m[0], my = a.m[1], mz = a.m[2];
     const long mxy = (long)mx * my, M = mxy * mz;
     const int cx0 = vb.x * TX, cy0 = vb.y * TY, cz0 = vb.z * TZ;
-    for (int i = tid; i < NB; i += NC) {
+    for (int i = tid; i < BX * BY * VccSmem<F>::kPlanes; i += NTH) {
         const int lz = i / (BX * BY), r = i - lz * BX * BY, ly = r / BX, lx = r - ly * BX;
         const int gx = cx0 + lx, gy = cy0 + ly, gz = cz0 + lz;
-        const bool ok = gx < mx && gy < my && gz < mz;
-        const long k = (long)gz * mxy + (long)gy * mx + gx;
+        const long k = (long)gz * mxy + (long)gy * mx + gx, k2 = k + TZ / 2 * mxy;
+        const bool okxy = gx < mx && gy < my, ok = okxy && gz < mz, ok2 = okxy && gz + TZ / 2 < mz;
+        auto ld = [&](const float *f, int c) -> F {
+            if constexpr (CPT == 2) return make_float2(ok ? f[c * M + k] : 0.f, ok2 ? f[c * M + k2] : 0.f);
+            else return ok ? f[c * M + k] : 0.f;
+        };
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            su[c][i] = ok ? a.u[c * M + k] : 0.f;
-            if (GN) sv[c][i] = ok ? a.v[c * M + k] : 0.f;
+            sm.su[c][i] = ld(a.u, c);
+            if (GN) sm.sv[c][i] = ld(a.v, c);
         }
     }
+    for (int i = tid; i < 3 * NB; i += NTH) (&sm.box[0][0])[i] = 0.f;
     vb.sync();
     const int lx = tid % TX, ly = (tid / TX) % TY, lz = tid / (TX * TY);
-    const bool valid = cx0 + lx < mx - 1 && cy0 + ly < my - 1 && cz0 + lz < mz - 1;
+    const bool validxy = cx0 + lx < mx - 1 && cy0 + ly < my - 1;
+    const bool valid0 = validxy && cz0 + lz < mz - 1, valid1 = validxy && cz0 + lz + TZ / 2 < mz - 1;
     const int base = (lz * BY + ly) * BX + lx;
     const float ig0 = a.ig[0], ig1 = a.ig[1], ig2 = a.ig[2];
-    auto at = [&](const auto &s, int o) {
+    auto corner = [&](const F (&s)[3][BX * BY * VccSmem<F>::kPlanes], int o) -> Vec<F> {
         const int i = base + (o & 1) + ((o >> 1) & 1) * BX + (o >> 2) * BX * BY;
-        return V3{s[0][i], s[1][i], s[2][i]};
+        return {s[0][i], s[1][i], s[2][i]};
     };
-    // edges (identity plus scaled differences) of u, and of v for the GN product
-    V3 E1[4], E2[4], E3[4], D1[GN ? 4 : 1], D2[GN ? 4 : 1], D3[GN ? 4 : 1];
-    {
-        V3 cu[8], cv[GN ? 8 : 1];
-#pragma unroll
-        for (int o = 0; o < 8; ++o) {
-            cu[o] = at(su, o);
-            if constexpr (GN) cv[o] = at(sv, o);
+    // the edge of axis ax between two corners: scaled difference (plus the identity for u)
+    auto edge = [&](const Vec<F> &p0, const Vec<F> &p1, int ax, bool unit) -> Vec<F> {
+        const F g = bc_<F>(ax == 0 ? ig0 : ax == 1 ? ig1 : ig2), one = bc_<F>(1.f);
+        const F x = sub_(p1.x, p0.x), y = sub_(p1.y, p0.y), z = sub_(p1.z, p0.z);
+        return {unit && ax == 0 ? fma_(x, g, one) : mul_(x, g), unit && ax == 1 ? fma_(y, g, one) : mul_(y, g),
+                unit && ax == 2 ? fma_(z, g, one) : mul_(z, g)};
+    };
+    auto y_edge = [&](const F (&s)[3][BX * BY * VccSmem<F>::kPlanes], int b, bool unit) -> Vec<F> {
+        return edge(corner(s, corner_of(1, b, 0)), corner(s, corner_of(1, b, 1)), 1, unit);
+    };
+    // corner o's contributions of the thread's cells onto the box: one corner at a
+    // time over the block, so that no two threads meet at a node and every
+    // node sums its cells in the order of o
+    auto scatter = [&](int o, F x, F y, F z) {
+        float *p = &sm.box[0][base + (o & 1) + ((o >> 1) & 1) * BX + (o >> 2) * BX * BY];
+        if (o > 0) vb.sync();
+        if constexpr (CPT == 2) {
+            constexpr int D = TZ / 2 * BX * BY;
+            p[0] += valid0 ? x.x : 0.f;
+            p[D] += valid1 ? x.y : 0.f;
+            p[NB] += valid0 ? y.x : 0.f;
+            p[NB + D] += valid1 ? y.y : 0.f;
+            p[2 * NB] += valid0 ? z.x : 0.f;
+            p[2 * NB + D] += valid1 ? z.y : 0.f;
+        } else {
+            p[0] += valid0 ? x : 0.f;
+            p[NB] += valid0 ? y : 0.f;
+            p[2 * NB] += valid0 ? z : 0.f;
         }
+    };
+    const F zero = bc_<F>(0.f);
+    Vec<F> E1[4], E3[4], D1[GN ? 4 : 1], D3[GN ? 4 : 1];
+    {
+        Vec<F> p[8];
+#pragma unroll
+        for (int o = 0; o < 8; ++o) p[o] = corner(sm.su, o);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const V3 &x0 = cu[corner_of(0, e, 0)], &x1 = cu[corner_of(0, e, 1)];
-            const V3 &y0 = cu[corner_of(1, e, 0)], &y1 = cu[corner_of(1, e, 1)];
-            const V3 &z0 = cu[corner_of(2, e, 0)], &z1 = cu[corner_of(2, e, 1)];
-            E1[e] = {fmaf(x1.x - x0.x, ig0, 1.f), (x1.y - x0.y) * ig0, (x1.z - x0.z) * ig0};
-            E2[e] = {(y1.x - y0.x) * ig1, fmaf(y1.y - y0.y, ig1, 1.f), (y1.z - y0.z) * ig1};
-            E3[e] = {(z1.x - z0.x) * ig2, (z1.y - z0.y) * ig2, fmaf(z1.z - z0.z, ig2, 1.f)};
-            if (GN) {
-                const V3 &p0 = cv[corner_of(0, e, 0)], &p1 = cv[corner_of(0, e, 1)];
-                const V3 &q0 = cv[corner_of(1, e, 0)], &q1 = cv[corner_of(1, e, 1)];
-                const V3 &r0 = cv[corner_of(2, e, 0)], &r1 = cv[corner_of(2, e, 1)];
-                D1[e] = {(p1.x - p0.x) * ig0, (p1.y - p0.y) * ig0, (p1.z - p0.z) * ig0};
-                D2[e] = {(q1.x - q0.x) * ig1, (q1.y - q0.y) * ig1, (q1.z - q0.z) * ig1};
-                D3[e] = {(r1.x - r0.x) * ig2, (r1.y - r0.y) * ig2, (r1.z - r0.z) * ig2};
+            E1[e] = edge(p[corner_of(0, e, 0)], p[corner_of(0, e, 1)], 0, true);
+            E3[e] = edge(p[corner_of(2, e, 0)], p[corner_of(2, e, 1)], 2, true);
+        }
+        if constexpr (GN) {
+#pragma unroll
+            for (int o = 0; o < 8; ++o) p[o] = corner(sm.sv, o);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                D1[e] = edge(p[corner_of(0, e, 0)], p[corner_of(0, e, 1)], 0, false);
+                D3[e] = edge(p[corner_of(2, e, 0)], p[corner_of(2, e, 1)], 2, false);
             }
         }
     }
-    V3 G1[4], G2[4], G3[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) G1[e] = G2[e] = G3[e] = V3{0.f, 0.f, 0.f};
-    int fold = 0;
-    float dmn = 3.4e38f, dmx = -3.4e38f;
-    Kahan32 en;
-    float out[8][3];
-#pragma unroll
-    for (int o = 0; o < 8; ++o) out[o][0] = out[o][1] = out[o][2] = 0.f;
+    F en = zero, en_c = zero;                       // Kahan sum of psi(d)
+    F dmn = bc_<F>(3.4e38f), dmx = bc_<F>(-3.4e38f);
     if constexpr (DG) {
+        F out[8][3];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int o = 0; o < 8; ++o) out[o][0] = out[o][1] = out[o][2] = zero;
 #pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const V3 X = cross(E2[b], E3[c]);
-                const V3 gx{X.x * ig0, X.y * ig0, X.z * ig0};
+        for (int b = 0; b < 4; ++b) {
+            const Vec<F> E2 = y_edge(sm.su, b, true), nE2 = neg_(E2);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const Vec<F> X = cross(E2, nE2, E3[c]), gx = scaled(X, ig0), nE3 = neg_(E3[c]);
 #pragma unroll
                 for (int aa = 0; aa < 4; ++aa) {
-                    const float d = dot(E1[aa], X);
-                    const float rd = __fdividef(1.f, d);
-                    const float w = d > 0.f ? 2.f * rd * rd * rd : 0.f;   // psi''(d)
-                    const V3 Y = cross(E3[c], E1[aa]), Z = cross(E1[aa], E2[b]);
-                    const V3 gy{Y.x * ig1, Y.y * ig1, Y.z * ig1}, gz{Z.x * ig2, Z.y * ig2, Z.z * ig2};
+                    const F rd = lanes(rcp_pos, dot(E1[aa], X));
+                    const F w = mul_(mul_(rd, rd), rd);   // psi''(d) / 2
+                    const Vec<F> nE1 = neg_(E1[aa]);
+                    const Vec<F> gy = scaled(cross(E3[c], nE3, E1[aa]), ig1), gz = scaled(cross(E1[aa], nE1, E2), ig2);
                     // corners and signs are compile-time once the loops are unrolled
 #pragma unroll
                     for (int o = 0; o < 8; ++o) {
@@ -162,173 +264,150 @@ __device__ __forceinline__ void vcc_cell_body(const VccArgs &a, const VBlock &vb
                         const int sy = (o == corner_of(1, b, 1)) - (o == corner_of(1, b, 0));
                         const int sz = (o == corner_of(2, c, 1)) - (o == corner_of(2, c, 0));
                         if (sx == 0 && sy == 0 && sz == 0) continue;
-                        V3 g{0.f, 0.f, 0.f};
+                        // the square of +-gx +- gy +- gz does not depend on a common sign
+                        const int s0 = sx ? sx : sy ? sy : sz;
+                        Vec<F> g{zero, zero, zero};
                         bool first = true;
-                        auto term = [&](int sg, const V3 &t) {
+                        auto term = [&](int sg, const Vec<F> &t) {
                             if (sg == 0) return;
-                            const V3 st = sg > 0 ? t : V3{-t.x, -t.y, -t.z};
-                            if (first) g = st;
-                            else add(st, g);
+                            if (first) g = t;
+                            else if (sg == s0) g = {add_(g.x, t.x), add_(g.y, t.y), add_(g.z, t.z)};
+                            else g = {sub_(g.x, t.x), sub_(g.y, t.y), sub_(g.z, t.z)};
                             first = false;
                         };
                         term(sx, gx);
                         term(sy, gy);
                         term(sz, gz);
-                        out[o][0] = fmaf(w * g.x, g.x, out[o][0]);
-                        out[o][1] = fmaf(w * g.y, g.y, out[o][1]);
-                        out[o][2] = fmaf(w * g.z, g.z, out[o][2]);
+                        out[o][0] = fma_(mul_(w, g.x), g.x, out[o][0]);
+                        out[o][1] = fma_(mul_(w, g.y), g.y, out[o][1]);
+                        out[o][2] = fma_(mul_(w, g.z), g.z, out[o][2]);
                     }
                 }
             }
         }
-    } else if constexpr (GN) {
-        // the x-edges in pairs (a = 2p, 2p + 1), one f32x2 lane each
-        float2 e1x[2], e1y[2], e1z[2], d1x[2], d1y[2], d1z[2], g1x[2], g1y[2], g1z[2];
 #pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            e1x[p] = make_float2(E1[2 * p].x, E1[2 * p + 1].x);
-            e1y[p] = make_float2(E1[2 * p].y, E1[2 * p + 1].y);
-            e1z[p] = make_float2(E1[2 * p].z, E1[2 * p + 1].z);
-            d1x[p] = make_float2(D1[2 * p].x, D1[2 * p + 1].x);
-            d1y[p] = make_float2(D1[2 * p].y, D1[2 * p + 1].y);
-            d1z[p] = make_float2(D1[2 * p].z, D1[2 * p + 1].z);
-            g1x[p] = g1y[p] = g1z[p] = make_float2(0.f, 0.f);
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const V3 X = cross(E2[b], E3[c]);
-                V3 Y = cross(D2[b], E3[c]);
-                add(cross(E2[b], D3[c]), Y);
-                const float2 Xx = bc2(X.x), Xy = bc2(X.y), Xz = bc2(X.z);
-                float2 wx = make_float2(0.f, 0.f), wy = wx, wz = wx;   // W = sum_a w e1_a, per lane
-#pragma unroll
-                for (int p = 0; p < 2; ++p) {
-                    const float2 d = fma2(e1z[p], Xz, fma2(e1y[p], Xy, mul2(e1x[p], Xx)));
-                    // grad d . v = d1_a . X + e1_a . Y
-                    const float2 dd = fma2(e1z[p], bc2(Y.z), fma2(e1y[p], bc2(Y.y), fma2(e1x[p], bc2(Y.x),
-                                      fma2(d1z[p], Xz, fma2(d1y[p], Xy, mul2(d1x[p], Xx))))));
-                    const float r0 = __fdividef(1.f, d.x), r1 = __fdividef(1.f, d.y);
-                    const float2 r = make_float2(r0, r1);
-                    float2 w = mul2(mul2(mul2(r, r), mul2(r, bc2(2.f))), dd);   // psi''(d) (grad d . v)
-                    w.x = d.x > 0.f ? w.x : 0.f;
-                    w.y = d.y > 0.f ? w.y : 0.f;
-                    g1x[p] = fma2(w, Xx, g1x[p]);
-                    g1y[p] = fma2(w, Xy, g1y[p]);
-                    g1z[p] = fma2(w, Xz, g1z[p]);
-                    wx = fma2(w, e1x[p], wx);
-                    wy = fma2(w, e1y[p], wy);
-                    wz = fma2(w, e1z[p], wz);
-                }
-                const V3 W{wx.x + wx.y, wy.x + wy.y, wz.x + wz.y};
-                add(cross(E3[c], W), G2[b]);
-                add(cross(W, E2[b]), G3[c]);
-            }
-        }
-#pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            G1[2 * p] = V3{g1x[p].x, g1y[p].x, g1z[p].x};
-            G1[2 * p + 1] = V3{g1x[p].y, g1y[p].y, g1z[p].y};
-        }
+        for (int o = 0; o < 8; ++o) scatter(o, out[o][0], out[o][1], out[o][2]);
     } else {
+        Vec<F> G1[4], G3[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const V3 X = cross(E2[b], E3[c]);
-                V3 W{0.f, 0.f, 0.f};
-#pragma unroll
-                for (int aa = 0; aa < 4; ++aa) {
-                    const float d = dot(E1[aa], X);
-                    const bool pos = d > 0.f;
-                    dmn = fminf(dmn, d);
-                    dmx = fmaxf(dmx, d);
-                    fold += pos ? 0 : 1;
-                    const float rd = __frcp_rn(d);
-                    const float dm = d - 1.f;
-                    en.add(pos ? dm * dm * rd : 0.f);               // psi(d) = (d - 1)^2 / d
-                    const float w = pos ? dm * (d + 1.f) * rd * rd : 0.f;   // psi'(d) = 1 - 1/d^2
-                    axpy(w, X, G1[aa]);
-                    axpy(w, E1[aa], W);
-                }
-                add(cross(E3[c], W), G2[b]);
-                add(cross(W, E2[b]), G3[c]);
+        for (int e = 0; e < 4; ++e) G1[e] = G3[e] = Vec<F>{zero, zero, zero};
+#pragma unroll 1
+        for (int b = 0; b < 4; ++b) {
+            const Vec<F> E2 = y_edge(sm.su, b, true), nE2 = neg_(E2);
+            Vec<F> D2, nD2, G2{zero, zero, zero};
+            if constexpr (GN) {
+                D2 = y_edge(sm.sv, b, false);
+                nD2 = neg_(D2);
             }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const Vec<F> X = cross(E2, nE2, E3[c]);
+                Vec<F> W{zero, zero, zero};   // sum_a w e1_a
+                if constexpr (GN) {
+                    const Vec<F> Y = cross_add(D2, nD2, E3[c], cross(E2, nE2, D3[c]));
+#pragma unroll
+                    for (int aa = 0; aa < 4; ++aa) {
+                        const F rd = lanes(rcp_pos, dot(E1[aa], X));
+                        const F dd = dot_add(E1[aa], Y, dot(D1[aa], X));   // grad d . v
+                        const F w = mul_(mul_(rd, rd), mul_(rd, dd));     // psi''(d) (grad d . v) / 2
+                        axpy(w, X, G1[aa]);
+                        axpy(w, E1[aa], W);
+                    }
+                } else {
+                    F ps = zero;
+#pragma unroll
+                    for (int aa = 0; aa < 4; ++aa) {
+                        const F d = dot(E1[aa], X), one = bc_<F>(1.f);
+                        dmn = lanes(min_nan, dmn, d);
+                        dmx = lanes([](float p, float q) { return fmaxf(p, q); }, dmx, d);
+                        // 1 / d, refined to half an ulp; psi = (d - 1)^2 / d and psi' = 1 - 1 / d^2
+                        // vanish with it on a fold
+                        const F r0 = lanes(rcp_pos, d);
+                        const F rd = fma_(r0, fma_(d, neg_(r0), one), r0);
+                        const F dm = sub_(d, one), q = mul_(dm, rd);
+                        ps = fma_(dm, q, ps);
+                        const F w = mul_(q, mul_(add_(d, one), rd));
+                        axpy(w, X, G1[aa]);
+                        axpy(w, E1[aa], W);
+                    }
+                    const F y = sub_(ps, en_c), t = add_(en, y);
+                    en_c = sub_(sub_(t, en), y);
+                    en = t;
+                }
+                const Vec<F> nW = neg_(W);
+                G2 = cross_add_r(E3[c], W, nW, G2);
+                G3[c] = cross_add_r(W, E2, nE2, G3[c]);
+            }
+            sm.g2[b * 3][tid] = G2.x;
+            sm.g2[b * 3 + 1][tid] = G2.y;
+            sm.g2[b * 3 + 2][tid] = G2.z;
         }
-    }
-    // edge gradients onto the cell's corners (scaled by 1/g of the edge's axis)
+        // edge gradients onto the cell's corners, scaled by +-1/g of the edge's axis
+        // (times 2 for the GN product's halved weights): corner o is an end of one edge per axis
+        const float h = GN ? 2.f : 1.f, h0 = ig0 * h, h1 = ig1 * h, h2 = ig2 * h;
+        Vec<F> G2[4];
 #pragma unroll
-    for (int e = 0; e < 4 && !DG; ++e) {
-        const V3 g1{G1[e].x * ig0, G1[e].y * ig0, G1[e].z * ig0};
-        const V3 g2{G2[e].x * ig1, G2[e].y * ig1, G2[e].z * ig1};
-        const V3 g3{G3[e].x * ig2, G3[e].y * ig2, G3[e].z * ig2};
-        const int x1 = corner_of(0, e, 1), x0 = corner_of(0, e, 0);
-        const int y1 = corner_of(1, e, 1), y0 = corner_of(1, e, 0);
-        const int z1 = corner_of(2, e, 1), z0 = corner_of(2, e, 0);
-        out[x1][0] += g1.x; out[x1][1] += g1.y; out[x1][2] += g1.z;
-        out[x0][0] -= g1.x; out[x0][1] -= g1.y; out[x0][2] -= g1.z;
-        out[y1][0] += g2.x; out[y1][1] += g2.y; out[y1][2] += g2.z;
-        out[y0][0] -= g2.x; out[y0][1] -= g2.y; out[y0][2] -= g2.z;
-        out[z1][0] += g3.x; out[z1][1] += g3.y; out[z1][2] += g3.z;
-        out[z0][0] -= g3.x; out[z0][1] -= g3.y; out[z0][2] -= g3.z;
-    }
-#pragma unroll
-    for (int o = 0; o < 8; ++o)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) scell[o * 3 + k][tid] = valid ? out[o][k] : 0.f;
-    vb.sync();
-    // gather per node of the box from the (up to) 8 cells of this tile
-    const int cta = vb.bid;
-    float *dst = a.boxes + (long)cta * 3 * a.box;
-    for (int i = tid; i < NB; i += NC) {
-        const int bz = i / (BX * BY), r = i - bz * BX * BY, by = r / BX, bx = r - by * BX;
-        float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+        for (int e = 0; e < 4; ++e) G2[e] = Vec<F>{sm.g2[e * 3][tid], sm.g2[e * 3 + 1][tid], sm.g2[e * 3 + 2][tid]};
 #pragma unroll
         for (int o = 0; o < 8; ++o) {
-            const int qx = bx - (o & 1), qy = by - ((o >> 1) & 1), qz = bz - (o >> 2);
-            if (qx < 0 || qy < 0 || qz < 0 || qx >= TX || qy >= TY || qz >= TZ) continue;
-            const int c = (qz * TY + qy) * TX + qx;
-            s0 += scell[o * 3][c];
-            s1 += scell[o * 3 + 1][c];
-            s2 += scell[o * 3 + 2][c];
+            const int e1 = o >> 1, e2 = (o & 1) + 2 * (o >> 2), e3 = o & 3;
+            const F sx = bc_<F>((o & 1) ? h0 : -h0), sy = bc_<F>((o & 2) ? h1 : -h1), sz = bc_<F>((o & 4) ? h2 : -h2);
+            scatter(o, fma_(G3[e3].x, sz, fma_(G2[e2].x, sy, mul_(G1[e1].x, sx))),
+                    fma_(G3[e3].y, sz, fma_(G2[e2].y, sy, mul_(G1[e1].y, sx))),
+                    fma_(G3[e3].z, sz, fma_(G2[e2].z, sy, mul_(G1[e1].z, sx))));
         }
-        dst[i] = s0 * a.wscale;
-        dst[a.box + i] = s1 * a.wscale;
-        dst[2 * a.box + i] = s2 * a.wscale;
+    }
+    vb.sync();
+    const int cta = vb.bid;
+    const float wscale = DG ? 2.f * a.wscale : a.wscale;
+    float *dst = a.boxes + (long)cta * 3 * a.box;
+    for (int i = tid; i < NB; i += NTH) {
+        dst[i] = sm.box[0][i] * wscale;
+        dst[a.box + i] = sm.box[1][i] * wscale;
+        dst[2 * a.box + i] = sm.box[2][i] * wscale;
     }
     if (VM == 0) {
-        // energy, fold count and min / max d of the block
+        // energy, folds and min / max d of the block
         double (&red)[NC / 32] = sm.red;
         int (&sfold)[NC / 32] = sm.sfold;
         float (&wmn)[NC / 32] = sm.wmn;
         float (&wmx)[NC / 32] = sm.wmx;
-        double e = valid ? (double)en.s - (double)en.c : 0.0;
-        int f = valid ? fold : 0;
-        if (!valid) { dmn = 3.4e38f; dmx = -3.4e38f; }
+        double e;
+        float mn, mxv;
+        if constexpr (CPT == 2) {
+            e = (valid0 ? (double)en.x - (double)en_c.x : 0.0) + (valid1 ? (double)en.y - (double)en_c.y : 0.0);
+            mn = min_nan(valid0 ? dmn.x : 3.4e38f, valid1 ? dmn.y : 3.4e38f);
+            mxv = fmaxf(valid0 ? dmx.x : -3.4e38f, valid1 ? dmx.y : -3.4e38f);
+        } else {
+            e = valid0 ? (double)en - (double)en_c : 0.0;
+            mn = valid0 ? dmn : 3.4e38f;
+            mxv = valid0 ? dmx : -3.4e38f;
+        }
+        // a fold is a bound that is not positive: the least one decides
+        int f = mn > 0.f ? 0 : 1;
         for (int off = 16; off > 0; off >>= 1) {
             e += __shfl_xor_sync(FULL, e, off);
             f += __shfl_xor_sync(FULL, f, off);
-            dmn = fminf(dmn, __shfl_xor_sync(FULL, dmn, off));
-            dmx = fmaxf(dmx, __shfl_xor_sync(FULL, dmx, off));
+            mn = fminf(mn, __shfl_xor_sync(FULL, mn, off));
+            mxv = fmaxf(mxv, __shfl_xor_sync(FULL, mxv, off));
         }
         const int w = tid >> 5;
-        if ((tid & 31) == 0) { red[w] = e; sfold[w] = f; wmn[w] = dmn; wmx[w] = dmx; }
+        if ((tid & 31) == 0) { red[w] = e; sfold[w] = f; wmn[w] = mn; wmx[w] = mxv; }
         vb.sync();
         if (tid == 0) {
             double t = 0.0;
             int ft = 0;
-            float mn = 3.4e38f, mxv = -3.4e38f;
-            for (int i = 0; i < NC / 32; ++i) {
+            float tn = 3.4e38f, tx = -3.4e38f;
+            for (int i = 0; i < NTH / 32; ++i) {
                 t += red[i];
                 ft += sfold[i];
-                mn = fminf(mn, wmn[i]);
-                mxv = fmaxf(mxv, wmx[i]);
+                tn = fminf(tn, wmn[i]);
+                tx = fmaxf(tx, wmx[i]);
             }
             a.epart[cta] = t;
             a.fold[cta] = ft;
-            a.dmin[cta] = mn;
-            a.dmax[cta] = mxv;
+            a.dmin[cta] = tn;
+            a.dmax[cta] = tx;
         }
     }
 }
