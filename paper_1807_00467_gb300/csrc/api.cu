@@ -960,6 +960,10 @@ static int pcg(rg_ctx *c, const float *g, float *p, int iters, double *stats) {
         int napart = 0;   // d.q partials: from the node pass, else from the alpha kernel
         if ((st = matvec(c, c->d, c->q, c->apart, &napart))) return st;
         if (!napart) LAUNCH(9, launch_pcg_alpha(a, c->q, &napart, c->st));
+        if (pcg_fused_ok(a.n)) {
+            LAUNCH(9, launch_pcg_fused(a, c->q, napart, p, k, c->st));
+            continue;
+        }
         LAUNCH(9, launch_pcg_step(a, c->q, napart, k, c->st));
         LAUNCH(9, launch_pcg_reorth(a, k, c->st));
         LAUNCH(9, launch_pcg_dir(a, p, k, c->st));

@@ -172,6 +172,10 @@ cudaError_t launch_pcg_alpha(const PcgArgs &a, const float *q, int *napart, cuda
 // napart: the d.q partials in a.apart (from launch_pcg_alpha or the node pass)
 cudaError_t launch_pcg_step(const PcgArgs &a, const float *q, int napart, int k, cudaStream_t st);
 cudaError_t launch_pcg_reorth(const PcgArgs &a, int k, cudaStream_t st);
+// The three together in one launch of one thread-block cluster, where the
+// partition has at most that many blocks (pcg_fused_ok).
+bool pcg_fused_ok(long n);
+cudaError_t launch_pcg_fused(const PcgArgs &a, const float *q, int napart, float *s, int k, cudaStream_t st);
 cudaError_t launch_pcg_dir(const PcgArgs &a, float *s, int k, cudaStream_t st);
 cudaError_t launch_axpy_copy(long n, float t, const float *x, const float *p, float *y, cudaStream_t st,
                              const int *skip = nullptr);

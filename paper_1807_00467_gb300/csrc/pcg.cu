@@ -22,6 +22,8 @@
 //
 // The preconditioner is diagonal, so z_j = M^-1 r_j is not stored: the
 // Gram-Schmidt coefficients use r . z_j = (M^-1 r) . r_j.
+#include <cooperative_groups.h>
+
 #include "pcg_body.cuh"
 
 namespace ngf {
@@ -100,18 +102,20 @@ __global__ void __launch_bounds__(kVT, 2) pcg_alpha_kernel(Part P, const float *
 
 // ---------------------------------------------------------------------------
 // step, reorthogonalisation and direction: the bodies of pcg_body.cuh
+template <int Q>
 __global__ void __launch_bounds__(kVT, 2) pcg_step_kernel(Part P, PcgScalars *sc, const double *apart, int napart,
                                                        const float *q, const float *minv, float *Rh, long stride,
                                                        int k, double *part) {
     __shared__ PcgSmem sm;
-    pcg_step_body(P, sc, apart, napart, q, minv, Rh, stride, k, part, cuda_block_1d(), sm);
+    pcg_step_body<Q>(P, sc, apart, napart, q, minv, Rh, stride, k, part, cuda_block_1d(), sm);
 }
 
+template <int Q>
 __global__ void __launch_bounds__(kVT, 2) pcg_reorth_kernel(Part P, const PcgScalars *sc, const float *minv, float *Rh,
                                                          long stride, int k, const double *rzh, const double *cpart,
                                                          double *rzpart) {
     __shared__ PcgSmem sm;
-    pcg_reorth_body(P, sc, minv, Rh, stride, k, rzh, cpart, rzpart, cuda_block_1d(), sm);
+    pcg_reorth_body<Q>(P, sc, minv, Rh, stride, k, rzh, cpart, rzpart, cuda_block_1d(), sm);
 }
 
 __global__ void __launch_bounds__(kVT, 2) pcg_dir_kernel(Part P, PcgScalars *sc, const float *minv, const float *r,
@@ -120,12 +124,59 @@ __global__ void __launch_bounds__(kVT, 2) pcg_dir_kernel(Part P, PcgScalars *sc,
     pcg_dir_body(P, sc, minv, r, d, s, k, rzh, rzpart, cuda_block_1d(), sm);
 }
 
+// The three bodies one after the other in one launch: the blocks of a short
+// vector's partition as one thread-block cluster, whose barrier takes the place
+// of the kernel boundaries (same partition and sums: same bits).  Three
+// launches of 6 blocks spent much of their ~30 us on launch, drain and
+// re-reading r, M^-1 and the scalars: 24 us fused at 11 k floats.  Up to 16
+// blocks: longer vectors need more than a cluster's SMs for their history.
+template <int Q>
+__global__ void __launch_bounds__(kVT) pcg_fused_kernel(Part P, PcgScalars *sc, const double *apart, int napart,
+                                                     const float *q, const float *minv, float *Rh, long stride, int k,
+                                                     double *part, double *rzh, double *rzpart, float *d, float *s) {
+    __shared__ PcgSmem sm;
+    const VBlock b = cuda_block_1d();
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    pcg_step_body<Q>(P, sc, apart, napart, q, minv, Rh, stride, k, part, b, sm);
+    cl.sync();
+    pcg_reorth_body<Q>(P, sc, minv, Rh, stride, k, rzh, part, rzpart, b, sm);
+    cl.sync();
+    pcg_dir_body(P, sc, minv, Rh + (long)(k + 1) * stride, d, s, k, rzh, rzpart, b, sm);
+}
+
+constexpr int kFuseMax = 16;   // blocks of a cluster (opt-in size)
+
 }  // namespace
 
 int pcg_blocks(long n) {
     int nb;
     make_part(n, &nb);
     return nb;
+}
+
+bool pcg_fused_ok(long n) { return pcg_blocks(n) <= kFuseMax; }
+
+cudaError_t launch_pcg_fused(const PcgArgs &a, const float *q, int napart, float *s, int k, cudaStream_t st) {
+    if (k < 0 || k + 1 >= kHist || napart < 1 || !pcg_fused_ok(a.n)) return cudaErrorInvalidValue;
+    int nb;
+    const Part P = make_part(a.n, &nb);
+    auto kernel = pcg_fused_kernel<1>;   // at most kFuseMax blocks: one quad per thread
+    static const cudaError_t big =
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (big != cudaSuccess) return big;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nb);
+    cfg.blockDim = dim3(kVT);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = nb;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P, a.sc, (const double *)a.apart, napart, q, a.minv, a.Rh, a.stride, k,
+                              a.part, a.rzh, a.rzpart, a.d, s);
 }
 
 long pcg_stride(long n) { return (n + 63) / 64 * 64; }
@@ -149,7 +200,15 @@ cudaError_t launch_pcg_step(const PcgArgs &a, const float *q, int napart, int k,
     if (k < 0 || k + 1 >= kHist || napart < 1) return cudaErrorInvalidValue;
     int nb;
     const Part P = make_part(a.n, &nb);
-    pcg_step_kernel<<<nb, kVT, 0, st>>>(P, a.sc, a.apart, napart, q, a.minv, a.Rh, a.stride, k, a.part);
+    auto run = [&](auto kernel) {
+        kernel<<<nb, kVT, 0, st>>>(P, a.sc, a.apart, napart, q, a.minv, a.Rh, a.stride, k, a.part);
+    };
+    switch (P.qpt) {
+        case 1: run(pcg_step_kernel<1>); break;
+        case 2: run(pcg_step_kernel<2>); break;
+        case 3: run(pcg_step_kernel<3>); break;
+        default: run(pcg_step_kernel<0>);
+    }
     return cudaGetLastError();
 }
 
@@ -157,7 +216,15 @@ cudaError_t launch_pcg_reorth(const PcgArgs &a, int k, cudaStream_t st) {
     if (k < 0 || k + 1 >= kHist) return cudaErrorInvalidValue;
     int nb;
     const Part P = make_part(a.n, &nb);
-    pcg_reorth_kernel<<<nb, kVT, 0, st>>>(P, a.sc, a.minv, a.Rh, a.stride, k, a.rzh, a.part, a.rzpart);
+    auto run = [&](auto kernel) {
+        kernel<<<nb, kVT, 0, st>>>(P, a.sc, a.minv, a.Rh, a.stride, k, a.rzh, a.part, a.rzpart);
+    };
+    switch (P.qpt) {
+        case 1: run(pcg_reorth_kernel<1>); break;
+        case 2: run(pcg_reorth_kernel<2>); break;
+        case 3: run(pcg_reorth_kernel<3>); break;
+        default: run(pcg_reorth_kernel<0>);
+    }
     return cudaGetLastError();
 }
 

@@ -35,18 +35,28 @@ __device__ __forceinline__ double block_total(float v, double *red, const VBlock
 }
 
 // Sum of the partials part[0..n) of the previous kernel by the whole block in
-// a fixed order (thread-strided, a fixed shuffle tree, the warps in order):
-// the same value in every block, valid in every thread.
+// a fixed order (strided over the threads, a fixed shuffle tree, the warps in
+// order): the same value in every block, valid in every thread.  FP64 runs at
+// two lanes a clock and SM here, so a short list is left to four warps and one
+// thread adds the warps' sums (all 16 warps, each adding all 16 sums, took 2-4
+// us a kernel: direction kernel 18.2 -> 15.5 us at 3.2 M floats, 12.2 -> 8.2 at
+// 418 k).
 __device__ __forceinline__ double block_sum_parts(const double *part, int n, double *red, const VBlock &b) {
-    double s = 0.0;
-    for (int i = b.tid; i < n; i += kVT) s += __ldcg(part + i);
-    s = lb_warp_sum(s);
-    if ((b.tid & 31) == 0) red[b.tid >> 5] = s;
+    const int nt = n > 1024 ? kVT : 128;
+    if (b.tid < nt) {
+        double s = 0.0;
+        for (int i = b.tid; i < n; i += nt) s += __ldcg(part + i);
+        s = lb_warp_sum(s);
+        if ((b.tid & 31) == 0) red[b.tid >> 5] = s;
+    }
     b.sync();
-    double t = 0.0;
-    for (int w = 0; w < kVW; ++w) t += red[w];
+    if (b.tid == 0) {
+        double t = red[0];
+        for (int w = 1; w < nt / 32; ++w) t += red[w];
+        red[kVW] = t;
+    }
     b.sync();
-    return t;
+    return red[kVW];
 }
 
 struct Part {
@@ -61,22 +71,55 @@ struct Part {
 __device__ __forceinline__ float4 ldg4(const float *p, long q) { return reinterpret_cast<const float4 *>(p)[q]; }
 __device__ __forceinline__ void st4(float *p, long q, float4 v) { reinterpret_cast<float4 *>(p)[q] = v; }
 
+// Whether this thread holds its i-th quad: Q > 0 is the partition's qpt known
+// at compile time, Q = 0 reads it from the partition.
+template <int Q>
+__device__ __forceinline__ bool has_quad(const Part &P, int i, long e) {
+    return (Q > 0 || i < P.qpt) && e < P.n4;
+}
+
+// Residuals of the history in flight at once per thread.  A long vector has up
+// to kQmax quads of one residual in flight per thread; a short one has a
+// single quad, and reading the history one residual at a time then costs a
+// memory latency each, up to 31 in a row.  So residuals are loaded in groups
+// that keep about 8 quads in flight: step and reorthogonalisation kernels 18.6
+// -> 11.7 and 15.7 -> 11.2 us at 11 k floats, 25.2 -> 20.0 and 21.2 -> 18.5 us
+// at 418 k.  The sums keep their order (same bits).
+template <int Q>
+__host__ __device__ constexpr int hist_group() {
+    return Q == 1 ? 8 : Q == 2 ? 4 : Q == 3 ? 2 : 1;
+}
+
 // shared scratch of one block of the step, reorthogonalisation and direction bodies
 struct PcgSmem {
     double wp[kHist][kVW];
-    double red[kVW];
+    double red[kVW + 1];
     float c[kHist];
 };
 
 // ---------------------------------------------------------------------------
 // alpha = r.z / d.q (stop on a non-positive curvature d.q or a vanishing r.z);
 // r_{k+1} = r_k - alpha q; then the partials of (M^-1 r_{k+1}) . r_j, j = 0..k
+template <int Q = 0>
 __device__ __forceinline__ void pcg_step_body(const Part &P, PcgScalars *sc, const double *apart, int napart,
                                               const float *q, const float *minv, float *Rh, long stride, int k,
                                               double *part, const VBlock &b, PcgSmem &sm) {
     double (&wp)[kHist][kVW] = sm.wp;
     double *red = sm.red;
     const int nb = b.nblk, lane = b.tid & 31, warp = b.tid >> 5;
+    constexpr int NQ = Q > 0 ? Q : kQmax, G = hist_group<Q>();
+    // a short vector's operands are loaded before the scalars are formed
+    float4 x[Q > 0 ? G : 1][NQ];
+    auto load_group = [&](int j0) {
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+#pragma unroll
+            for (int i = 0; i < NQ; ++i) {
+                const long e = P.quad(i, b);
+                if (e < P.n4 && j0 + g <= k) x[g][i] = ldg4(Rh + (long)(j0 + g) * stride, e);
+            }
+    };
+    if constexpr (Q > 0) load_group(0);
     // every block forms the same alpha; a block that reads the stop flag block 0
     // has just set takes the same decision (the flag only ever turns on)
     const double pq = block_sum_parts(apart, napart, red, b);
@@ -90,12 +133,12 @@ __device__ __forceinline__ void pcg_step_body(const Part &P, PcgScalars *sc, con
     const float al = (float)al64;
     const float *r = Rh + (long)k * stride;
     float *rn = Rh + (long)(k + 1) * stride;
-    float4 zn[kQmax];
+    float4 zn[NQ];
 #pragma unroll
-    for (int i = 0; i < kQmax; ++i) {
+    for (int i = 0; i < NQ; ++i) {
         const long e = P.quad(i, b);
         zn[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (i < P.qpt && e < P.n4) {
+        if (has_quad<Q>(P, i, e)) {
             const float4 qv = ldg4(q, e), rv = ldg4(r, e), m = ldg4(minv, e);
             const float4 nv = make_float4(fmaf(-al, qv.x, rv.x), fmaf(-al, qv.y, rv.y), fmaf(-al, qv.z, rv.z),
                                           fmaf(-al, qv.w, rv.w));
@@ -111,18 +154,37 @@ __device__ __forceinline__ void pcg_step_body(const Part &P, PcgScalars *sc, con
         rn[et] = nv;
         zt = minv[et] * nv;
     }
+    if constexpr (Q > 0) {
 #pragma unroll 1
-    for (int j = 0; j <= k; ++j) {
-        const float *rj = Rh + (long)j * stride;
-        float acc = 0.f;
+        for (int j0 = 0; j0 <= k; j0 += G) {
+            if (j0 > 0) load_group(j0);
 #pragma unroll
-        for (int i = 0; i < kQmax; ++i) {
-            const long e = P.quad(i, b);
-            if (i < P.qpt && e < P.n4) acc += dot4(zn[i], ldg4(rj, e));
+            for (int g = 0; g < G; ++g) {
+                const int j = j0 + g;
+                if (j > k) break;
+                float acc = 0.f;
+#pragma unroll
+                for (int i = 0; i < NQ; ++i)
+                    if (P.quad(i, b) < P.n4) acc += dot4(zn[i], x[g][i]);
+                if (tail) acc = fmaf(zt, Rh[(long)j * stride + et], acc);
+                acc = lb_warp_sum_f(acc);
+                if (lane == 0) wp[j][warp] = (double)acc;
+            }
         }
-        if (tail) acc = fmaf(zt, rj[et], acc);
-        acc = lb_warp_sum_f(acc);
-        if (lane == 0) wp[j][warp] = (double)acc;
+    } else {
+#pragma unroll 1
+        for (int j = 0; j <= k; ++j) {
+            const float *rj = Rh + (long)j * stride;
+            float acc = 0.f;
+#pragma unroll
+            for (int i = 0; i < kQmax; ++i) {
+                const long e = P.quad(i, b);
+                if (i < P.qpt && e < P.n4) acc += dot4(zn[i], ldg4(rj, e));
+            }
+            if (tail) acc = fmaf(zt, rj[et], acc);
+            acc = lb_warp_sum_f(acc);
+            if (lane == 0) wp[j][warp] = (double)acc;
+        }
     }
     b.sync();
     for (int j = b.tid; j <= k; j += kVT) {
@@ -135,6 +197,7 @@ __device__ __forceinline__ void pcg_step_body(const Part &P, PcgScalars *sc, con
 // ---------------------------------------------------------------------------
 // c_j = (M^-1 r_{k+1}) . r_j / (r_j . z_j);  r_{k+1} -= sum_j c_j r_j;  then the
 // partials of r.z with z = M^-1 r_{k+1}
+template <int Q = 0>
 __device__ __forceinline__ void pcg_reorth_body(const Part &P, const PcgScalars *sc, const float *minv, float *Rh,
                                                 long stride, int k, const double *rzh, const double *cpart,
                                                 double *rzpart, const VBlock &b, PcgSmem &sm) {
@@ -142,11 +205,22 @@ __device__ __forceinline__ void pcg_reorth_body(const Part &P, const PcgScalars 
     double *red = sm.red;
     const int nb = b.nblk, lane = b.tid & 31, warp = b.tid >> 5;
     float *r = Rh + (long)(k + 1) * stride;
-    float4 rv[kQmax];
+    constexpr int NQ = Q > 0 ? Q : kQmax, G = hist_group<Q>();
+    float4 x[Q > 0 ? G : 1][NQ];
+    auto load_group = [&](int j0) {
 #pragma unroll
-    for (int i = 0; i < kQmax; ++i) {
+        for (int g = 0; g < G; ++g)
+#pragma unroll
+            for (int i = 0; i < NQ; ++i) {
+                const long e = P.quad(i, b);
+                if (e < P.n4 && j0 - g >= 0) x[g][i] = ldg4(Rh + (long)(j0 - g) * stride, e);
+            }
+    };
+    float4 rv[NQ];
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {
         const long e = P.quad(i, b);
-        rv[i] = (i < P.qpt && e < P.n4) ? ldg4(r, e) : make_float4(0.f, 0.f, 0.f, 0.f);
+        rv[i] = has_quad<Q>(P, i, e) ? ldg4(r, e) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     const bool tail = b.bid == 0 && b.tid < P.tail;
     const long et = 4 * P.n4 + b.tid;
@@ -158,26 +232,46 @@ __device__ __forceinline__ void pcg_reorth_body(const Part &P, const PcgScalars 
         if (lane == 0) c[j] = (stop || rzh[j] == 0.0) ? 0.f : (float)(v / rzh[j]);
     }
     b.sync();
-#pragma unroll 2
-    for (int j = k; j >= 0; --j) {
-        const float *rj = Rh + (long)j * stride;
-        const float cj = c[j];
+    if constexpr (Q > 0) {
+#pragma unroll 1
+        for (int j0 = k; j0 >= 0; j0 -= G) {
+            load_group(j0);
 #pragma unroll
-        for (int i = 0; i < kQmax; ++i) {
-            const long e = P.quad(i, b);
-            if (i < P.qpt && e < P.n4) {
-                const float4 x = ldg4(rj, e);
-                rv[i].x = fmaf(-cj, x.x, rv[i].x); rv[i].y = fmaf(-cj, x.y, rv[i].y);
-                rv[i].z = fmaf(-cj, x.z, rv[i].z); rv[i].w = fmaf(-cj, x.w, rv[i].w);
+            for (int g = 0; g < G; ++g) {
+                const int j = j0 - g;
+                if (j < 0) break;
+                const float cj = c[j];
+#pragma unroll
+                for (int i = 0; i < NQ; ++i)
+                    if (P.quad(i, b) < P.n4) {
+                        rv[i].x = fmaf(-cj, x[g][i].x, rv[i].x); rv[i].y = fmaf(-cj, x[g][i].y, rv[i].y);
+                        rv[i].z = fmaf(-cj, x[g][i].z, rv[i].z); rv[i].w = fmaf(-cj, x[g][i].w, rv[i].w);
+                    }
+                if (tail) rt = fmaf(-cj, Rh[(long)j * stride + et], rt);
             }
         }
-        if (tail) rt = fmaf(-cj, rj[et], rt);
+    } else {
+#pragma unroll 2
+        for (int j = k; j >= 0; --j) {
+            const float *rj = Rh + (long)j * stride;
+            const float cj = c[j];
+#pragma unroll
+            for (int i = 0; i < kQmax; ++i) {
+                const long e = P.quad(i, b);
+                if (i < P.qpt && e < P.n4) {
+                    const float4 y = ldg4(rj, e);
+                    rv[i].x = fmaf(-cj, y.x, rv[i].x); rv[i].y = fmaf(-cj, y.y, rv[i].y);
+                    rv[i].z = fmaf(-cj, y.z, rv[i].z); rv[i].w = fmaf(-cj, y.w, rv[i].w);
+                }
+            }
+            if (tail) rt = fmaf(-cj, rj[et], rt);
+        }
     }
     float acc = 0.f;
 #pragma unroll
-    for (int i = 0; i < kQmax; ++i) {
+    for (int i = 0; i < NQ; ++i) {
         const long e = P.quad(i, b);
-        if (i < P.qpt && e < P.n4) {
+        if (has_quad<Q>(P, i, e)) {
             const float4 m = ldg4(minv, e);
             st4(r, e, rv[i]);
             acc += dot4(rv[i], make_float4(m.x * rv[i].x, m.y * rv[i].y, m.z * rv[i].z, m.w * rv[i].w));

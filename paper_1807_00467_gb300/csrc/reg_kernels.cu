@@ -216,53 +216,64 @@ __device__ double sum_parts(const double *p, int n) {
     return block_sum(s);
 }
 
-__global__ void terms_kernel(const TermsArgs a) {
+// The four sums run side by side, eight warps each, with four loads in flight
+// per thread (one after the other by the whole block: 24 us at 8192 + 5445 +
+// 288 partials, mostly load latency and FP64 at two lanes a clock).
+__global__ void __launch_bounds__(1024) terms_kernel(const TermsArgs a) {
     if (a.skip && *a.skip) return;   // uniform: every block reads the same flag
-    double D = a.dpart ? sum_parts(a.dpart, a.nd) * a.dscale : 0.0;
-    __syncthreads();
-    double R = a.rpart ? sum_parts(a.rpart, a.nr) * a.rscale : 0.0;
-    __syncthreads();
-    double V = a.vpart ? sum_parts(a.vpart, a.nv) * a.vscale : 0.0;
-    __syncthreads();
-    double K = a.kpart ? sum_parts(a.kpart, a.nkp) : 0.0;
-    __syncthreads();
-    __shared__ int sfold;
-    __shared__ float smn, smx;
-    if (threadIdx.x == 0) { sfold = 0; smn = 3.4e38f; smx = -3.4e38f; }
-    __syncthreads();
-    if (a.vpart) {
-        int f = 0;
-        float mn = 3.4e38f, mx = -3.4e38f;
-        for (int i = threadIdx.x; i < a.nv; i += blockDim.x) {
-            f += a.fold[i];
+    __shared__ double red[32];
+    __shared__ float wmn[32], wmx[32];
+    __shared__ int wf[32];
+    const int grp = threadIdx.x >> 8, t = threadIdx.x & 255, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double *p = grp == 0 ? a.dpart : grp == 1 ? a.rpart : grp == 2 ? a.vpart : a.kpart;
+    const int n = p ? (grp == 0 ? a.nd : grp == 1 ? a.nr : grp == 2 ? a.nv : a.nkp) : 0;
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int i = t; i < n; i += 1024)
+        for (int k = 0; k < 4; ++k)
+            if (i + 256 * k < n) s[k] += p[i + 256 * k];
+    double v = (s[0] + s[1]) + (s[2] + s[3]);
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    int f = 0;
+    float mn = 3.4e38f, mx = -3.4e38f;
+    if (a.vpart)
+        for (int i = threadIdx.x; i < a.nv; i += 1024) {
+            f |= a.fold[i];
             mn = fminf(mn, a.dmin[i]);
             mx = fmaxf(mx, a.dmax[i]);
         }
-        if (f) atomicAdd(&sfold, f);
-        // min/max via shared atomics on the float bit patterns is avoided: serialise per warp
-        for (int off = 16; off > 0; off >>= 1) {
-            mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, off));
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-        }
-        __shared__ float wmn[32], wmx[32];
-        if ((threadIdx.x & 31) == 0) { wmn[threadIdx.x >> 5] = mn; wmx[threadIdx.x >> 5] = mx; }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int i = 0; i < (int)(blockDim.x + 31) / 32; ++i) { smn = fminf(smn, wmn[i]); smx = fmaxf(smx, wmx[i]); }
-        }
+    f = __any_sync(0xffffffffu, f != 0);
+    for (int off = 16; off > 0; off >>= 1) {
+        mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, off));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
     }
+    if (lane == 0) { red[warp] = v; wmn[warp] = mn; wmx[warp] = mx; wf[warp] = f; }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (warp != 0) return;
+    double g = 0.0;   // lanes 0..3: the sum of their group's warps in order
+    if (lane < 4)
+        for (int i = 0; i < 8; ++i) g += red[8 * lane + i];
+    f = __any_sync(0xffffffffu, wf[lane] != 0);
+    mn = wmn[lane];
+    mx = wmx[lane];
+    for (int off = 16; off > 0; off >>= 1) {
+        mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, off));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+    }
+    const double sd = __shfl_sync(0xffffffffu, g, 0), sr = __shfl_sync(0xffffffffu, g, 1);
+    const double sv = __shfl_sync(0xffffffffu, g, 2), K = __shfl_sync(0xffffffffu, g, 3);
+    if (lane == 0) {
+        const double D = a.dpart ? sd * a.dscale : 0.0, R = a.rpart ? sr * a.rscale : 0.0;
+        double V = a.vpart ? sv * a.vscale : 0.0;
         double J = D + a.alpha * R + a.gamma * V + a.delta * K;
-        if (sfold) { J = INFINITY; V = INFINITY; }
+        if (f) { J = INFINITY; V = INFINITY; }
         else if (a.nonfinite && !isfinite(J)) atomicExch(a.nonfinite, 1);
         a.terms[0] = D; a.terms[1] = R; a.terms[2] = V; a.terms[3] = K; a.terms[4] = J;
-        if (a.dminmax) { a.dminmax[0] = a.vpart ? smn : 1.0; a.dminmax[1] = a.vpart ? smx : 1.0; }
+        if (a.dminmax) { a.dminmax[0] = a.vpart ? mn : 1.0; a.dminmax[1] = a.vpart ? mx : 1.0; }
     }
 }
 
 cudaError_t launch_terms(const TermsArgs &a, cudaStream_t st) {
-    terms_kernel<<<1, 512, 0, st>>>(a);
+    terms_kernel<<<1, 1024, 0, st>>>(a);
     return cudaGetLastError();
 }
 
