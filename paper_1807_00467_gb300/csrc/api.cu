@@ -51,9 +51,10 @@ struct rg_ctx {
                               // [2]: set by the terms kernel when an objective came out NaN (or +inf without a fold)
     bool err_zeroed;
     CUtensorMap map_dT, map_a;
-    ColGeom cg;               // column-marching GN-product kernel: geometry, tensor maps, node boxes
+    ColGeom cg, cp;           // column-marching passes: geometry of the objective / gradient pass, of the
+                              // GN product (z chunks), tensor maps, node boxes
     CUtensorMap map_col_dT, map_col_a;
-    BoxGeom bM;
+    BoxGeom bM, bP;
     const BoxGeom *bcur;      // node-box geometry of the last NGF tile launch (read by the node pass)
     int hook_no_tma, hook_poll;   // test hooks (rg_debug_hook)
     int pass_sel;                 // objective / gradient pass: 0 by size, 1 column-marching, 2 tile
@@ -206,10 +207,12 @@ static void tile_geom(const rg_image_geom *img, const rg_grid_geom *grid, TileGe
     if ((long)t.nzt * 3 * t.nxt * t.nyt > 12 * 1024) t.nzt = 0;
 }
 
-// Column geometry of the column-marching GN-product kernel: TXI x 16 voxel
-// columns in x-y (TXI = 60 less a remainder so that it is whole cells), every z
-// plane; node boxes [3][m3][C1 + 1][C0 + 1] per column.
-static void col_geom(const rg_image_geom *img, const rg_grid_geom *grid, ColGeom &c) {
+// Column geometry of the column-marching kernels: TXI x 16 voxel columns in x-y
+// (TXI = 60 less a remainder so that it is whole cells), every z plane or (fill)
+// chunks of them; node boxes [3][nodes][C1 + 1][C0 + 1] per column and chunk.
+// Chunks, by the rule of tile_geom, where the columns leave SMs idle (one CTA
+// per SM): multiples of 4 planes, so that CTAs can walk several of them.
+static void col_geom(const rg_image_geom *img, const rg_grid_geom *grid, ColGeom &c, bool fill) {
     for (int a = 0; a < 3; ++a) {
         c.n[a] = img->n[a];
         c.m[a] = grid->m[a];
@@ -226,7 +229,21 @@ static void col_geom(const rg_image_geom *img, const rg_grid_geom *grid, ColGeom
     // node columns of voxel columns x0 - 2 .. x0 + 61 (rows y0 - 2 .. y0 + 17) and the next node
     c.nxt = ((61 >> c.lrho[0]) + 1) - ((-2) >> c.lrho[0]) + 1;
     c.nyt = ((17 >> c.lrho[1]) + 1) - ((-2) >> c.lrho[1]) + 1;
-    c.box = (c.C0 + 1) * (c.C1 + 1) * c.m[2];
+    c.TZ = c.n[2];
+    if (fill) {
+        const int q = std::max(4, c.rho[2]);
+        const long nxy = (long)c.nb[0] * c.nb[1];
+        long best = (nxy + 151) / 152 * (c.n[2] + 8);
+        for (int z = c.n[2] / q * q; z >= q; z -= q) {
+            const long cost = (nxy * ((c.n[2] + z - 1) / z) + 151) / 152 * (z + 8);
+            if (cost < best) {
+                best = cost;
+                c.TZ = z;
+            }
+        }
+    }
+    c.nbz = (c.n[2] + c.TZ - 1) / c.TZ;
+    c.box = (c.C0 + 1) * (c.C1 + 1) * (c.TZ / c.rho[2] + 1);
     c.tma = 0;
 }
 
@@ -340,21 +357,20 @@ static void derive(rg_ctx *c) {
         if (n > c->nA_cap) c->nA_cap = n;
         if (n * 3 * t.box > c->boxA_cap) c->boxA_cap = n * 3 * t.box;
     }
-    col_geom(&c->img, &c->grid, c->cg);
-    {
-        const long n = (long)c->cg.nb[0] * c->cg.nb[1] * 3 * c->cg.box;
-        if (n > c->boxA_cap) c->boxA_cap = n;
+    for (int i = 0; i < 2; ++i) {
+        ColGeom &g = i ? c->cp : c->cg;
+        BoxGeom &b = i ? c->bP : c->bM;
+        col_geom(&c->img, &c->grid, g, i != 0);
+        c->boxA_cap = std::max(c->boxA_cap, (long)g.nb[0] * g.nb[1] * g.nbz * 3 * g.box);
+        for (int k = 0; k < 3; ++k) b.m[k] = c->grid.m[k];
+        b.nb[0] = g.nb[0];
+        b.nb[1] = g.nb[1];
+        b.nb[2] = g.nbz;
+        b.C[0] = g.C0;
+        b.C[1] = g.C1;
+        b.C[2] = g.TZ / g.rho[2];
+        b.box = g.box;
     }
-    c->bM.m[0] = c->grid.m[0];
-    c->bM.m[1] = c->grid.m[1];
-    c->bM.m[2] = c->grid.m[2];
-    c->bM.nb[0] = c->cg.nb[0];
-    c->bM.nb[1] = c->cg.nb[1];
-    c->bM.nb[2] = 1;
-    c->bM.C[0] = c->cg.C0;
-    c->bM.C[1] = c->cg.C1;
-    c->bM.C[2] = c->grid.m[2] - 1;
-    c->bM.box = c->cg.box;
     tile_geom(&c->img, &c->grid, c->tg, 16);
     c->nA = c->tg.nb[0] * c->tg.nb[1] * c->tg.nb[2];
     c->nD = c->nA;
@@ -424,6 +440,7 @@ extern "C" int rg_ctx_create(rg_ctx **out, const rg_image_geom *img, const rg_gr
                  encode_field_map(&c->map_col_a, c->cg.n, 16, c->lin_a, kColBoxX))
                     ? 1
                     : 0;
+    c->cp.tma = c->cg.tma;
     c->bcur = &c->bA;
     c->hook_poll = 1 << 20;
     c->ev_pool = new std::vector<cudaEvent_t>();
@@ -592,10 +609,10 @@ static int run_tile(rg_ctx *c, int mode, const float *field) {
     };
     const int pid = mode == MODE_MATVEC ? 0 : (mode == MODE_OBJ ? 2 : (mode == MODE_DIAG ? 10 : 1));
     c->bcur = &c->bA;
-    if ((mode == MODE_MATVEC || mode == MODE_DIAG) && !c->general_only && gn_product_supported(c->cg)) {
+    if ((mode == MODE_MATVEC || mode == MODE_DIAG) && !c->general_only && gn_product_supported(c->cp)) {
         // the column-marching kernel (node boxes per column of the volume)
         ColArgs a;
-        a.g = c->cg;
+        a.g = c->cp;
         a.v = field;
         a.boxes = c->boxA;
         a.map_dT = c->map_col_dT;
@@ -605,7 +622,7 @@ static int run_tile(rg_ctx *c, int mode, const float *field) {
         a.poll_limit = c->hook_poll;
         a.no_tma = c->hook_no_tma;
         LAUNCH(pid, launch_gn_product(a, mode == MODE_DIAG, c->st));
-        c->bcur = &c->bM;
+        c->bcur = &c->bP;
         return RG_OK;
     }
     if ((mode == MODE_MATVEC || mode == MODE_DIAG) && !c->general_only && gn_matvec_supported(c->tg)) {
@@ -974,14 +991,14 @@ static int pcg(rg_ctx *c, const float *g, float *p, int iters, double *stats) {
 // Whether the persistent batched PCG (pcg_batch.cu) can take this context's
 // PCG steps: the column GN-product kernel covers its volume and H has no
 // keypoint term (its node sums use atomics outside the node pass).
-static bool batch_pcg_ok(const rg_ctx *c) { return !c->general_only && c->nk <= 0 && pcg_batch_supported(c->cg); }
+static bool batch_pcg_ok(const rg_ctx *c) { return !c->general_only && c->nk <= 0 && pcg_batch_supported(c->cp); }
 
 // The operands of one PCG step of the context (the GN product H d into q as
 // matvec forms it, the vectors of pcg), with s the PCG iterate.
 static void batch_pair(rg_ctx *c, float *s, BatchPair &b) {
     ColArgs &a = b.col;
     a = ColArgs();
-    a.g = c->cg;
+    a.g = c->cp;
     a.v = c->d;
     a.boxes = c->boxA;
     a.map_dT = c->map_col_dT;
@@ -1015,7 +1032,7 @@ static void batch_pair(rg_ctx *c, float *s, BatchPair &b) {
         n.ig2[i] = (float)(1.0 / (c->g[i] * c->g[i]));
     }
     n.boxA = c->boxA;
-    n.gA = c->bM;
+    n.gA = c->bP;
     n.sA = (float)c->hbar;
     n.boxB = vcc ? c->boxB : nullptr;
     n.gB = c->bB;

@@ -117,7 +117,8 @@ struct ColGeom {
     int nb[2];         // tiles along x, y
     int C0, C1;        // cells per tile along x, y
     int nxt, nyt;      // node-plane extent read by a tile's prolongation
-    int box;           // floats per component of a column's node box: (C0 + 1)(C1 + 1) m3
+    int TZ, nbz;       // z planes per chunk (whole cells), chunks (1 but on small volumes)
+    int box;           // floats per component of a column's node box: (C0 + 1)(C1 + 1)(TZ / rho_z + 1)
     int tma;           // 1: tensor maps valid
 };
 

@@ -10,34 +10,40 @@
 // and the product is 2 hbar P^T z (the same three stages as the tile kernel
 // of ngf_matvec.cu).
 //
-// Layout:
+// Bound by instruction issue, then by HBM (24 bytes a voxel), so the layout is
+// the one with few instructions per voxel:
 //  - a CTA owns a column of the volume: TXI (60, or 56 when rho_x = 8) x 16
-//    voxels in x-y and every z plane.  Lane L holds the two adjacent x columns
-//    x0 - 2 + 2L and x0 - 1 + 2L (packed FP32: one f32x2 instruction serves
-//    both), warp w the row y0 - 2 + w; 20 warps cover the 16 rows and the
-//    2-row halos, 32 lanes the 60 columns and the 2-column halos;
-//  - the CTA marches z from plane -2 to n3 + 1, so every plane of the stored
-//    linearisation is read once per column (no z halo is re-read); each
-//    plane's dT/dy and a arrive by TMA (box 68 x 20 x 1 x 3, zero fill outside
-//    the volume) into a 4-stage ring, 3 planes ahead, and the plane sequence
-//    continues into the CTA's next column;
+//    voxels in x-y and a chunk of z planes (all of them on large volumes; 24 at
+//    256x256x64, whose 80 columns left half of the SMs idle: 59 -> 51 us).
+//    Lane L holds the two adjacent x columns x0 - 2 + 2L and x0 - 1 + 2L (packed
+//    FP32: one f32x2 instruction serves both), warp w the two rows
+//    y0 - 2 + 2w and y0 - 1 + 2w: 10 warps cover the 16 rows and the 2-row
+//    halos, 32 lanes the 60 columns and the 2-column halos.  The rows of a
+//    pair share a grid cell, so P v is interpolated along x once for both, and
+//    P^T sums them along y in registers before anything is reduced (one row per
+//    warp, with the rows parked in shared memory and reduced along x and y by
+//    passes of all warps: 151 M warp instructions and 219-222 us at 512x512x128,
+//    111 M and 207 us so).  10 warps at 160 registers leave the latency of one
+//    plane's chain exposed (issue 47%): the neighbour differences are formed at
+//    the top of a step, ahead of the TMA wait (219 -> 207 us);
+//  - the CTA marches z from plane z0 - 2 to z0 + nz + 1; step s takes plane
+//    s - 2 through W, the one before through C and the one before that through
+//    A.  dT/dy of plane s and a of plane s - 1 arrive by TMA (box 68 x 20 x 1 x 3,
+//    zero fill outside the volume), 3 steps ahead, into a ring of 6 planes of
+//    dT/dy (stage A reads it again two steps later) and 4 of a, so no register
+//    carries them; the sequence continues into the CTA's next column;
 //  - one barrier per plane; x neighbours by warp shuffles (the other column of
-//    a lane pair is local), y neighbours through double-buffered exchange
-//    rows, z neighbours in registers;
+//    a lane pair is local), y neighbours outside the pair through
+//    double-buffered exchange rows, z neighbours in registers;
 //  - P v: the node planes of v stream through a 4-slot ring in shared memory
-//    (each thread stages one node of a plane in registers two cells before it
-//    is needed); each lane pair interpolates bilinearly in x-y at cell starts
-//    and linearly in z per plane;
-//  - P^T: every lane accumulates its columns' two z-node planes in registers.
-//    When a node plane is complete, each lane of the interior warps parks its
-//    pair's hat-weighted parts for the cell's lower and upper node (plain
-//    stores, no shuffles); in the next plane all threads sum the parked lanes
-//    of each (row, node column) (the x reduction), and in the plane after
-//    that one thread per node of the column's box [3][m3][C1 + 1][C0 + 1]
-//    sums its rows with the y hat weights and writes it (the y reduction), so
-//    the reduction is spread over every warp and two barriers that the plane
-//    loop has anyway; a node-parallel pass sums the boxes of neighbouring
-//    columns (no atomics).
+//    by cp.async; at a cell's start a warp interpolates the pair's two node
+//    rows along x, per plane along z, per row along y;
+//  - P^T: every lane accumulates the row pair's two y-nodes on its cell's two
+//    z-node planes; a completed node plane is weighted along x, summed over
+//    the cell's lanes by shuffles and written once per node and row pair; in the next
+//    step one thread per node of the column's box adds the row pairs and stores
+//    it: node boxes [3][cells + 1][C1 + 1][C0 + 1] per column and chunk, summed
+//    by the node pass (no atomics).
 #pragma once
 
 #include "common.cuh"
@@ -48,30 +54,31 @@ namespace ngf {
 namespace gnpk {
 
 constexpr int kTY = 16;                   // owned voxel rows per column
-constexpr int kNW = kTY + 4;              // warps: rows incl. the 2-row halos
+constexpr int kNW = (kTY + 4) / 2;        // warps: row pairs incl. the 2-row halos
 constexpr int kNT = 32 * kNW;
-constexpr int kStages = 4;                // TMA ring depth (planes) = loop unroll
-constexpr int kAhead = 3;                 // planes in flight ahead of stage W
+constexpr int kStages = 4;                // TMA barriers (steps) = ring depth of a
+constexpr int kRingD = 6;                 // ring depth of dT/dy: 3 planes in use, 3 on the way
+constexpr int kAhead = 3;                 // steps issued ahead
+constexpr int kBoxRows = kTY + 4;
 constexpr int kBoxF = 4096;               // floats per field box (3 x 20 x 68 = 4080, 128-byte padded)
-constexpr int kStageF = 2 * kBoxF;        // dT/dy box, then a box
-constexpr int kComp = kNW * kColBoxX;     // floats between components in a box
-constexpr int kEx = kNW * 64;             // floats per exchange buffer (a float2 per lane and warp)
-constexpr uint32_t kPlaneBytes = 2u * kColBoxX * kNW * 3 * 4;
+constexpr int kComp = kBoxRows * kColBoxX;   // floats between components in a box
+constexpr int kEx = kNW * 2 * 64;         // floats per exchange buffer (a float2 per lane and row)
+constexpr uint32_t kPlaneBytes = 2u * kColBoxX * kBoxRows * 3 * 4;
+constexpr int kNodeMax = 2 * kNT;         // nodes of a staged plane at most
 constexpr unsigned FULL = 0xffffffffu;
 
 struct PcSmem {
-    int tma, ext, exc, nodes, park, xr, total;
+    int tma, ext, exc, nodes, xr, total;
 };
 
 __host__ __device__ inline PcSmem pc_smem(const ColGeom &g) {
     PcSmem s;
     int off = 0;
-    s.tma = off; off += kStages * kStageF + 32;            // + 128 bytes to align the base
+    s.tma = off; off += (kRingD + kStages) * kBoxF + 32;    // + 128 bytes to align the base
     s.ext = off; off += 2 * kEx;                            // t of plane C, double-buffered
     s.exc = off; off += 2 * kEx;                            // c'_y of plane A, double-buffered
     s.nodes = off; off += 4 * ((g.nyt * g.nxt + 31) & ~31) * 4;   // node planes of v, [slot][y][x][xyz_]
-    s.park = off; off += 2 * kTY * 32 * 6;                 // parked lane parts of 2 node planes, [slot][row][lane][3][lo, hi]
-    s.xr = off; off += 2 * kTY * (g.C0 + 1) * 3;           // x-reduced rows of 2 node planes, [slot][row][node][3]
+    s.xr = off; off += 2 * (kTY / 2) * 2 * (g.C0 + 1) * 3;  // x-reduced node planes, [slot][row pair][lo, hi][node][3]
     s.total = off;
     return s;
 }
@@ -88,36 +95,19 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 bc2(float a) { return make_float2(a, a); }
 
-// P^T along y for one node of a column box: node row jy receives the x-reduced
-// rows of its lower cell (rows jy ry + i, weight 1 - f_i) and of its upper
-// cell (rows (jy - 1) ry + i, weight f_i), f_i = (i + 1/2) / ry (squared
-// weights for the diagonal); src points at row 0 of the node's column (stride ss).
-template <int RY, bool SQ>
-__device__ __forceinline__ float y_node(const float *src, int ss, int jy, int C1) {
-    float acc = 0.f;
-#pragma unroll
-    for (int i = 0; i < RY; ++i) {
-        const float f = (i + 0.5f) / RY;
-        if (jy < C1) acc = fmaf(SQ ? (1.f - f) * (1.f - f) : 1.f - f, src[(jy * RY + i) * ss], acc);
-        if (jy > 0) acc = fmaf(SQ ? f * f : f, src[((jy - 1) * RY + i) * ss], acc);
-    }
-    return acc;
-}
-
-template <bool SQ>
-__device__ __forceinline__ float y_node_any(int ry, const float *src, int ss, int jy, int C1) {
-    switch (ry) {
-        case 1: return y_node<1, SQ>(src, ss, jy, C1);
-        case 2: return y_node<2, SQ>(src, ss, jy, C1);
-        case 4: return y_node<4, SQ>(src, ss, jy, C1);
-        default: return y_node<8, SQ>(src, ss, jy, C1);
-    }
-}
-
 // Bounded wait on a TMA barrier: one try (which suspends the thread for a
 // while in hardware) and, rarely, the polling loop that gives up.
 __device__ __forceinline__ void plane_wait(uint64_t *bar, uint32_t phase, int *err, int limit) {
     if (!mbar_try_wait(bar, phase)) mbar_wait_bounded(bar, phase, err, limit);
+}
+
+// Sum over the lanes of a cell (RX / 2 adjacent lanes, the first at 1 + c RX / 2),
+// valid in its first lane.
+template <int RX>
+__device__ __forceinline__ float cell_sum(float v) {
+    if (RX >= 4) v += __shfl_down_sync(FULL, v, 1);
+    if (RX >= 8) v += __shfl_down_sync(FULL, v, 2);
+    return v;
 }
 
 // DG = false: the GN product.  DG = true: the Jacobi diagonal of 2 hbar J^T J
@@ -125,398 +115,391 @@ __device__ __forceinline__ void plane_wait(uint64_t *bar, uint32_t phase, int *e
 // beta = sum_a (a'_a^2 at x - e_a and x + e_a) with a' = a / (2 h), times
 // (dT/dy)_k^2, onto the nodes with squared hat weights (stage C forms a'^2,
 // stage A sums instead of differencing, P v is not needed).
-// RZ: rho_z when it divides the ring depth (phases are constants), else 0.
-// CHAIN: a column's plane count is a whole number of ring cycles (no bound
-// checks inside a cycle), and CTAs walk several columns.
-// RXY: 4 when rho_x = rho_y = 4 (the x and y passes are then straight-line
-// code with constant extents), else 0 (extents from the geometry).
-// The kernel body: the CTA's columns t0, t0 + tstep, ... (CHAIN) or column t0
-// alone.  bars: the CTA's kStages TMA barriers, initialised here when
-// init_bars; pbits: the parity of each barrier's next phase (bit j for stage
-// j), carried from one call to the next when a CTA processes the columns of
-// several volumes (MULTI: the persistent batched kernel of pcg_batch.cu, whose
-// calls each end with no copy in flight).
-template <int RZ, bool DG, bool CHAIN, int RXY, bool MULTI = false>
+// RX: rho_x.  RZ: rho_z when it divides the unroll (phases are constants), else 0.
+// The kernel body: the CTA's columns t0, t0 + tstep, ... while chain (every
+// column's step count is a whole number of ring cycles), else column t0 alone.
+// bars: the CTA's kStages TMA barriers, initialised here when init_bars;
+// pbits: the parity of each barrier's next phase (bit j for barrier j), carried
+// from one call to the next when a CTA processes the columns of several
+// volumes (pcg_batch.cu; each call ends with no copy in flight).
+template <int RX, int RZ, bool DG>
 __device__ __forceinline__ void gn_product_body(const ColArgs &a, float *smem, uint64_t *bars, int t0, int tstep,
-                                                bool init_bars, uint32_t &pbits) {
+                                                bool chain, bool init_bars, uint32_t &pbits) {
     const ColGeom &g = a.g;
     const PcSmem S = pc_smem(g);
 
     const int tid = threadIdx.x, L = tid & 31, w = tid >> 5;
-    const int ncols = g.nb[0] * g.nb[1];
-    const int lrx = g.lrho[0], lry = g.lrho[1], lrz = g.lrho[2];
-    const int rx = g.rho[0], half = rx >> 1, rzm = g.rho[2] - 1;
+    const int ncols = g.nb[0] * g.nb[1] * g.nbz;
+    const int lry = g.lrho[1], lrz = g.lrho[2], rzm = g.rho[2] - 1;
     const float irz = g.irho[2];
-    const int n3 = g.n[2], nsteps = n3 + 4;
+    constexpr int LRX = RX == 2 ? 1 : RX == 4 ? 2 : 3, HX = RX / 2, C0 = (60 - 60 % RX) / RX, TXI = C0 * RX;
     const int nxt = g.nxt, nplane = nxt * g.nyt, npad = (nplane + 31) & ~31;
-    const int C0 = g.C0, C1 = g.C1, XR = (C0 + 1) * 3;
+    const int C1 = g.C1, np = (C1 + 1) * (C0 + 1);
     const long mxy = (long)g.m[0] * g.m[1], Mn = mxy * g.m[2];
 
-    float *tma_base = smem + S.tma + ((128u - (smem_u32(smem + S.tma) & 127u)) & 127u) / 4;
+    float *ring_d = smem + S.tma + ((128u - (smem_u32(smem + S.tma) & 127u)) & 127u) / 4;
+    float *ring_a = ring_d + kRingD * kBoxF;
     float4 *s_nodes = reinterpret_cast<float4 *>(smem + S.nodes);
-    float2 *park = reinterpret_cast<float2 *>(smem + S.park);   // [2 slots][16 rows][32 lanes][3] (lo, hi)
-    float *xr = smem + S.xr;                                     // [2 slots][16 rows][C0 + 1][3]
+    constexpr int XW = 2 * (C0 + 1) * 3, XS = (kTY / 2) * XW;   // floats per row pair, per slot
+    float *xr = smem + S.xr;
 
-    auto origin = [&](int t, int &x0, int &y0) {
-        x0 = (t % g.nb[0]) * g.TXI;
-        y0 = (t / g.nb[0]) * kTY;
+    auto origin = [&](int t, int &x0, int &y0, int &z0) {
+        const int q = t / g.nb[0];
+        x0 = (t - q * g.nb[0]) * TXI;
+        y0 = (q % g.nb[1]) * kTY;
+        z0 = (q / g.nb[1]) * g.TZ;
     };
-    // plane j (voxel plane j - 2) of column (x0, y0) into stage `st`; issued by
-    // lane 0 of the last warp (a halo row with the least other work; callers
-    // are warp-uniform)
-    auto issue_plane = [&](int x0, int y0, int j, int st) {
+    // step j's planes (dT/dy of voxel plane z0 + j - 2, a of the one before) into
+    // ring slots sd and sa; issued by lane 0 of the last warp (halo rows;
+    // callers are warp-uniform)
+    auto issue = [&](int x0, int y0, int z, int sd, int sa) {
         if (a.no_tma || L != 0) return;   // no_tma: test hook, the waits run out instead
-        float *dst = tma_base + st * kStageF;
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_expect_tx(&bars[st], kPlaneBytes);
-        tma_load_4d(dst, &a.map_dT, &bars[st], x0 - 4, y0 - 2, j - 2, 0);
-        tma_load_4d(dst + kBoxF, &a.map_a, &bars[st], x0 - 4, y0 - 2, j - 2, 0);
+        mbar_expect_tx(&bars[sa], kPlaneBytes);
+        tma_load_4d(ring_d + sd * kBoxF, &a.map_dT, &bars[sa], x0 - 4, y0 - 2, z, 0);
+        tma_load_4d(ring_a + sa * kBoxF, &a.map_a, &bars[sa], x0 - 4, y0 - 2, z - 1, 0);
     };
 
     int t = t0;
     if (t >= ncols) return;
     {
-        int x0, y0;
-        origin(t, x0, y0);
+        int x0, y0, z0;
+        origin(t, x0, y0, z0);
         if (init_bars && tid == kNT - 32) {
             for (int i = 0; i < kStages; ++i) mbar_init(&bars[i], 1);
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
         if (w == kNW - 1)
-            for (int j = 0; j < kAhead && j < nsteps; ++j) issue_plane(x0, y0, j, j);
+            for (int j = 0; j < kAhead; ++j) issue(x0, y0, z0 + j - 2, j, j);   // (a column has at least 5 steps)
     }
 
     // this lane's pair of columns: local x index i0 = 2L - 2 (even) and i0 + 1
     const int i0 = 2 * L - 2;
-    const bool interior_warp = w >= 2 && w < kTY + 2;
-    const bool owner = interior_warp && i0 >= 0 && i0 < g.TXI;   // tile-owned pair
-    const int ph = i0 & (rx - 1);   // x phase of the pair's first column in its cell (both share the cell)
-    const float2 *sbase = reinterpret_cast<const float2 *>(tma_base + w * kColBoxX + 2 * L + 2);
-    float2 *ex_t = reinterpret_cast<float2 *>(smem + S.ext) + w * 32 + L;
-    float2 *ex_c = reinterpret_cast<float2 *>(smem + S.exc) + w * 32 + L;
-    const int up = w > 0 ? -32 : 0, dn = w < kNW - 1 ? 32 : 0;   // in float2; the outer rows read themselves
-    constexpr int exh = kEx / 2;                                   // float2 per exchange buffer
-    const float2 *ex_t_up = ex_t + up, *ex_t_dn = ex_t + dn, *ex_c_up = ex_c + up, *ex_c_dn = ex_c + dn;
-    float2 *park_lane = park + ((w - 2) * 32 + L) * 3;   // this lane's parked parts in a slot (interior warps)
-    // the last warps (halo rows and the interior rows next to them) copy the node planes of v
-    const bool node_warp = (kNW - 1 - w) * 32 < npad;
-    const int ntid = tid - (kNT - npad);              // this thread's node of a plane (when node_warp)
-    // work items of the x and y passes go to the threads lane-major, so that
-    // every warp takes a share; quotients by the item extents from reciprocals
-    // (exact for the item counts and extents here: below 2^11)
-    const int lane_major = L * kNW + w;
-    const float invXR = 1.f / XR, invNP = 1.f / ((C1 + 1) * (C0 + 1)), invC0 = 1.f / (C0 + 1);
-    auto idiv = [](int a, float inv) { return __float2int_rz(((float)a + 0.5f) * inv); };
+    const bool own_rows = w >= 1 && w < kNW - 1;
+    const bool owner = own_rows && i0 >= 0 && i0 < TXI;   // tile-owned pair
+    const float fe = ((i0 & (RX - 1)) + 0.5f) / RX;       // x fractions of the pair in its cell: fe, fe + 1 / RX
+    const float2 fx2 = make_float2(fe, fe + 1.f / RX);
+    const bool node_lane = L >= 1 && ((L - 1) & (HX - 1)) == 0 && (L - 1) / HX <= C0;
+    const int jx_lane = (L - 1) / HX;
+    const float2 *lane_d = reinterpret_cast<const float2 *>(ring_d + 2 * w * kColBoxX + 2 * L + 2);
+    const float2 *lane_a = reinterpret_cast<const float2 *>(ring_a + 2 * w * kColBoxX + 2 * L + 2);
+    constexpr int kRow = kColBoxX / 2, kC2 = kComp / 2, kB2 = kBoxF / 2;   // in float2
+    // exchange rows [buffer][warp][row][lane]; the outer pairs read themselves
+    float2 *ex_t = reinterpret_cast<float2 *>(smem + S.ext) + w * 64 + L;
+    float2 *ex_c = reinterpret_cast<float2 *>(smem + S.exc) + w * 64 + L;
+    const int up = w > 0 ? -32 : 0, dn = w < kNW - 1 ? 64 : 32;   // the row above the pair, the row below
+    constexpr int exh = kEx / 2;
+    // the node reduction's items (component k, node row jy, node jx): this thread's first one
+    const int hy = g.rho[1] >> 1;   // row pairs per cell
+    struct Item {
+        int src, dst;      // in xr (lower node of the first row pair of cell jy), in a box component
+        bool lo, hi;       // the node has a cell above, below
+    };
+    auto item = [&](int it) {
+        const int k = it / np, r = it - k * np, jy = r / (C0 + 1), jx = r - jy * (C0 + 1);
+        return Item{jy * hy * XW + jx * 3 + k, k * g.box + r, jy < C1, jy > 0};
+    };
+    const Item item0 = item(tid);
 
-    uint32_t phase = 0;   // continues across the columns of this CTA (each has a multiple of kStages planes)
+    int sd = 0;   // ring slot of dT/dy of the current step
     for (;;) {
-        int x0, y0, xn = 0, yn = 0;
-        origin(t, x0, y0);
+        int x0, y0, z0, xn = 0, yn = 0, zn = 0;
+        origin(t, x0, y0, z0);
         const int tn = t + tstep;
-        const bool has_next = CHAIN && tn < ncols;
-        if (has_next) origin(tn, xn, yn);
-        const int kx_lo = (x0 - 2) >> lrx, ky_lo = (y0 - 2) >> lry;
+        const bool has_next = chain && tn < ncols;
+        if (has_next) origin(tn, xn, yn, zn);
+        const int nz = min(g.TZ, g.n[2] - z0), nsteps = nz + 4;
+        const int kx_lo = (x0 - 2) >> LRX, ky_lo = (y0 - 2) >> lry;
         float *box = a.boxes + (long)t * 3 * g.box;
 
-        // P v: this thread's node of every node plane (threads of the node warps
-        // beyond the plane fill padding), copied asynchronously into the ring
-        // (zero outside the grid)
-        int ngo = -1;   // offset of the node in a grid plane, -1 outside the grid or the plane
-        if (ntid >= 0 && ntid < nplane) {
-            const int ly = ntid / nxt, lx = ntid - ly * nxt;
-            const int ux = kx_lo + lx, uy = ky_lo + ly;
-            if (ux >= 0 && ux < g.m[0] && uy >= 0 && uy < g.m[1]) ngo = uy * g.m[0] + ux;
-        }
-        auto node_copy = [&](int kz) {   // node warps only (warp-uniform callers)
-            const bool in = ngo >= 0 && kz >= 0 && kz < g.m[2];
-            const float *p = in ? a.v + kz * mxy + ngo : a.v;
-            const uint32_t dst = smem_u32(s_nodes + (kz & 3) * npad + ntid);
-            const uint32_t n = in ? 4u : 0u;   // 0 source bytes: zero fill
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(p), "r"(n) : "memory");
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + 4), "l"(p + Mn), "r"(n) : "memory");
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + 8), "l"(p + 2 * Mn), "r"(n) : "memory");
+        // P v: this thread's nodes of every node plane (the last threads take the
+        // first), copied asynchronously into the ring (zero outside the grid)
+        const int nd0 = kNT - 1 - tid;
+        const bool node_thread = nd0 < nplane;
+        int ngo[2] = {-1, -1};   // offsets of the nodes in a grid plane, -1 outside the grid or the plane
+        if (!DG && node_thread)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int nd = nd0 + i * kNT, ly = nd / nxt, lx = nd - ly * nxt;
+                const int ux = kx_lo + lx, uy = ky_lo + ly;
+                if (nd < nplane && ux >= 0 && ux < g.m[0] && uy >= 0 && uy < g.m[1]) ngo[i] = uy * g.m[0] + ux;
+            }
+        auto node_copy = [&](int kz) {   // node threads only
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int nd = nd0 + i * kNT;
+                if (nd < nplane) {
+                    const bool in = ngo[i] >= 0 && kz >= 0 && kz < g.m[2];
+                    const float *p = in ? a.v + kz * mxy + ngo[i] : a.v;
+                    const uint32_t dst = smem_u32(s_nodes + (kz & 3) * npad + nd);
+                    const uint32_t n = in ? 4u : 0u;   // 0 source bytes: zero fill
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(p), "r"(n) : "memory");
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + 4), "l"(p + Mn), "r"(n) : "memory");
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + 8), "l"(p + 2 * Mn), "r"(n) : "memory");
+                }
+            }
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
-        const int cz0 = (-2) >> lrz;   // node plane of voxel plane -2
-        if (!DG && node_warp) {
+        const int cz0 = (z0 - 2) >> lrz;   // node plane of voxel plane z0 - 2
+        if (!DG && node_thread) {
             asm volatile("cp.async.wait_all;" ::: "memory");   // the last column's copies have landed
             for (int i = 0; i < 4; ++i) node_copy(cz0 + i);
             asm volatile("cp.async.wait_all;" ::: "memory");
         }
 
-        // this pair's bilinear position in a node plane
-        const int qoff = (((y0 - 2 + w) >> lry) - ky_lo) * nxt + (((x0 + i0) >> lrx) - kx_lo);
-        auto bilinear = [&](int kz, float2 *U) {
+        // the pair's node rows of a node plane, interpolated along x
+        const int yA = y0 - 2 + 2 * w;
+        const int qoff = ((yA >> lry) - ky_lo) * nxt + (((x0 + i0) >> LRX) - kx_lo);
+        const float fyA = ((yA & (g.rho[1] - 1)) + 0.5f) * g.irho[1], fyB = fyA + g.irho[1];
+        const float2 fA2 = bc2(fyA), fB2 = bc2(fyB);
+        auto x_lines = [&](int kz, float2 (&U)[2][3]) {
             const float4 *qp = s_nodes + (kz & 3) * npad + qoff;
-            const float4 n00 = qp[0], n10 = qp[1], n01 = qp[nxt], n11 = qp[nxt + 1];
-            const float2 fx2 = make_float2((ph + 0.5f) * g.irho[0], (ph + 1.5f) * g.irho[0]);
-            const float2 fy2 = bc2((((y0 - 2 + w) & (g.rho[1] - 1)) + 0.5f) * g.irho[1]);
-            float2 lo = fma2(fx2, bc2(n10.x - n00.x), bc2(n00.x)), hi = fma2(fx2, bc2(n11.x - n01.x), bc2(n01.x));
-            U[0] = fma2(fy2, sub2(hi, lo), lo);
-            lo = fma2(fx2, bc2(n10.y - n00.y), bc2(n00.y));
-            hi = fma2(fx2, bc2(n11.y - n01.y), bc2(n01.y));
-            U[1] = fma2(fy2, sub2(hi, lo), lo);
-            lo = fma2(fx2, bc2(n10.z - n00.z), bc2(n00.z));
-            hi = fma2(fx2, bc2(n11.z - n01.z), bc2(n01.z));
-            U[2] = fma2(fy2, sub2(hi, lo), lo);
-        };
-        // park a completed node plane (interior warps): the pair's parts for its
-        // cell's lower and upper node, hat weights 1 - f and f with f = fe and
-        // fe + 1 / rho_x (squared for the diagonal), zero outside the tile
-        auto park_plane = [&](const float2 *acc, int kz) {
-            if (!interior_warp) return;
-            float2 *dst = park_lane + (kz & 1) * (kTY * 32 * 3);
-            const float irx = g.irho[0], fe = (ph + 0.5f) * irx;
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const float ve = owner ? acc[k].x : 0.f, vo = owner ? acc[k].y : 0.f;
-                if (DG) {
-                    const float fo = fe + irx;
-                    dst[k] = make_float2(fmaf((1.f - fo) * (1.f - fo), vo, (1.f - fe) * (1.f - fe) * ve),
-                                         fmaf(fo * fo, vo, fe * fe * ve));
-                } else {
-                    const float sum = ve + vo, hi = fmaf(fe, sum, vo * irx);
-                    dst[k] = make_float2(sum - hi, hi);
-                }
+            for (int n = 0; n < 2; ++n) {
+                const float4 p = qp[n * nxt], q = qp[n * nxt + 1];
+                U[n][0] = fma2(fx2, bc2(q.x - p.x), bc2(p.x));
+                U[n][1] = fma2(fx2, bc2(q.y - p.y), bc2(p.y));
+                U[n][2] = fma2(fx2, bc2(q.z - p.z), bc2(p.z));
             }
         };
-        // x reduction of a parked node plane (all threads): item (row, node jx,
-        // component) sums the lower parts of the lanes of cell jx and the upper
-        // parts of the lanes of cell jx - 1 (the lanes of cell c are
-        // 1 + c rho_x / 2 .. + rho_x / 2 - 1; cell C0 lies outside the tile)
-        auto x_pass = [&](int kz) {
-            const float2 *src = park + (kz & 1) * (kTY * 32 * 3);
-            float *dst = xr + (kz & 1) * (kTY * XR);
-            if constexpr (RXY > 0) {   // consecutive threads take consecutive (row, node, component) items
-                constexpr int H = RXY / 2, C0c = (60 - 60 % RXY) / RXY, XRc = (C0c + 1) * 3, NX = kTY * XRc;
+        // a completed node plane of the row pair: hat weights along x (1 - f and f
+        // with f = fe and fe + 1 / rho_x, squared for the diagonal, zero outside the
+        // tile), summed over each cell's lanes; node jx takes the lower part of
+        // cell jx and the upper part of cell jx - 1
+        auto park = [&](const float2 (&acc)[2][3], int lk) {
+            if (!own_rows) return;
+            float *dst = xr + (lk & 1) * XS + (w - 1) * XW + jx_lane * 3;
 #pragma unroll
-                for (int i = 0; i < (NX + kNT - 1) / kNT; ++i) {
-                    const int it = tid + i * kNT;
-                    if (NX % kNT == 0 || it < NX) {
-                        const int row = it / XRc, r = it % XRc, jx = r / 3, k = r % 3;
-                        const float2 *p = src + (row * 32 + 1 + jx * H) * 3 + k;
-                        const float2 *pl = jx < C0c ? p : p - 3 * H, *ph = jx > 0 ? p : p + 3 * H;
-                        float lo = 0.f, hi = 0.f;
+            for (int n = 0; n < 2; ++n)
 #pragma unroll
-                        for (int q = 0; q < H; ++q) {
-                            lo += pl[3 * q].x;
-                            hi += ph[3 * (q - H)].y;
-                        }
-                        dst[it] = (jx < C0c ? lo : 0.f) + (jx > 0 ? hi : 0.f);
-                    }
-                }
-            } else {
-                for (int it = lane_major; it < kTY * XR; it += kNT) {
-                    const int row = idiv(it, invXR), r = it - row * XR, jx = (r * 43) >> 7, k = r - jx * 3;
-                    const float2 *p = src + (row * 32 + 1 + jx * half) * 3 + k;
-                    // the lanes of cell jx (lower parts, none for jx = C0) and of cell
-                    // jx - 1 (upper parts, none for jx = 0); a missing cell reads a
-                    // neighbouring one inside the row and is discarded
-                    const float2 *pl = jx < C0 ? p : p - 3 * half, *ph = jx > 0 ? p : p + 3 * half;
+                for (int k = 0; k < 3; ++k) {
+                    const float ve = owner ? acc[n][k].x : 0.f, vo = owner ? acc[n][k].y : 0.f;
                     float lo, hi;
-                    switch (half) {
-                        case 1: lo = pl[0].x; hi = ph[-3].y; break;
-                        case 2: lo = pl[0].x + pl[3].x; hi = ph[-6].y + ph[-3].y; break;
-                        default: lo = (pl[0].x + pl[3].x) + (pl[6].x + pl[9].x); hi = (ph[-12].y + ph[-9].y) + (ph[-6].y + ph[-3].y);
+                    if (DG) {
+                        const float fo = fe + 1.f / RX;
+                        lo = fmaf((1.f - fo) * (1.f - fo), vo, (1.f - fe) * (1.f - fe) * ve);
+                        hi = fmaf(fo * fo, vo, fe * fe * ve);
+                    } else {
+                        const float sum = ve + vo;
+                        hi = fmaf(fe, sum, vo * (1.f / RX));
+                        lo = sum - hi;
                     }
-                    dst[it] = (jx < C0 ? lo : 0.f) + (jx > 0 ? hi : 0.f);
+                    lo = cell_sum<RX>(lo);
+                    hi = cell_sum<RX>(hi);
+                    const float below = __shfl_up_sync(FULL, hi, HX);
+                    if (node_lane) dst[n * (C0 + 1) * 3 + k] = lo + (L > HX ? below : 0.f);
                 }
-            }
         };
-        // y reduction of an x-reduced node plane: one thread per node of the box
-        auto y_pass = [&](int kz) {
-            if constexpr (RXY > 0) {   // consecutive threads take consecutive nodes (coalesced stores)
-                constexpr int C0c = (60 - 60 % RXY) / RXY, C1c = kTY / RXY, XRc = (C0c + 1) * 3;
-                constexpr int NP = (C1c + 1) * (C0c + 1), NY = 3 * NP;
-                const float *src = xr + (kz & 1) * (kTY * XRc);
-                float *dst = box + (long)kz * NP;
-#pragma unroll
-                for (int i = 0; i < (NY + kNT - 1) / kNT; ++i) {
-                    const int it = (tid + kNT - 64) % kNT + i * kNT;   // from the third warp on
-                    if (it < NY) {
-                        const int k = it / NP, r = it % NP, jy = r / (C0c + 1), jx = r % (C0c + 1);
-                        const float v = y_node<RXY, DG>(src + jx * 3 + k, XRc, jy, C1c);
-                        dst[(long)k * g.box + r] = (DG ? 1.f : 2.f) * v;
-                    }
+        // one thread per node of the box: the row pairs of its lower cell (their
+        // lower node) and of its upper cell (their upper node)
+        auto y_pass = [&](int lk) {
+            const float *src = xr + (lk & 1) * XS;
+            float *dst = box + (long)lk * np;
+            auto one = [&](const Item &m) {
+                const float *p = src + m.src;
+                float v = 0.f;
+                for (int i = 0; i < hy; ++i) {
+                    if (m.lo) v += p[i * XW];
+                    if (m.hi) v += p[(i - hy) * XW + (C0 + 1) * 3];
                 }
-            } else {
-                const int np = (C1 + 1) * (C0 + 1);
-                for (int it = lane_major; it < 3 * np; it += kNT) {
-                    const int k = idiv(it, invNP), r = it - k * np;
-                    const int jy = idiv(r, invC0), jx = r - jy * (C0 + 1);
-                    const float v = y_node_any<DG>(g.rho[1], xr + (kz & 1) * (kTY * XR) + jx * 3 + k, XR, jy, C1);
-                    box[(long)k * g.box + (long)kz * np + r] = (DG ? 1.f : 2.f) * v;
-                }
-            }
+                dst[m.dst] = (DG ? 1.f : 2.f) * v;
+            };
+            if (tid < 3 * np) one(item0);
+            for (int it = tid + kNT; it < 3 * np; it += kNT) one(item(it));
         };
 
         // the exchange rows read before this column has written them (stages C and A
-        // of its first planes, which multiply them by zeros) must hold finite values
+        // of its first planes, whose results are dropped) must hold finite values
         {
             float *ex = smem + S.ext;
             for (int i = tid; i < 4 * kEx; i += kNT) ex[i] = 0.f;
         }
-        __syncthreads();   // node ring filled, exchange rows cleared; the previous column's sweeps are done with xr
+        __syncthreads();   // node ring filled, exchange rows cleared; the previous column's reduction is done with xr
 
-        // P v of the pair at node planes kz (U0) and kz + 1 (U0 + D) of the current cell
-        float2 U0[3], D[3];
-        if (!DG) {
-            float2 U1[3];
-            bilinear(cz0, U0);
-            bilinear(cz0 + 1, U1);
-            for (int k = 0; k < 3; ++k) D[k] = sub2(U1[k], U0[k]);
-        } else {
-            for (int k = 0; k < 3; ++k) U0[k] = D[k] = make_float2(0.f, 0.f);
-        }
         const float2 z2 = make_float2(0.f, 0.f);
-        float2 tm = z2, t0 = z2;                  // t at planes pC - 1, pC
-        float2 a1[3] = {z2, z2, z2};              // a' at plane pC
-        float2 d1[3] = {z2, z2, z2}, d2[3] = {z2, z2, z2};   // dT/dy at planes pC, pA
-        float2 cxp = z2;                          // c'_x at plane pA
-        float2 czm2 = z2, czm1 = z2;              // c'_z at planes pA - 1, pA
-        float2 acc0[3] = {z2, z2, z2}, acc1[3] = {z2, z2, z2};   // z-node planes of pA's cell
-        int xk = -1, yk = -1;                     // node planes due for the x pass, the y pass in this step
-
-        for (int s0 = 0; s0 < nsteps; s0 += kStages, phase ^= 1u) {
+        // x lines at node planes kz (U0) and kz + 1 (U0 + D) of the current cell
+        float2 U0[2][3], D[2][3];
+        if (!DG) {
+            float2 U1[2][3];
+            x_lines(cz0, U0);
+            x_lines(cz0 + 1, U1);
 #pragma unroll
-            for (int j = 0; j < kStages; ++j) {
-                const int s = s0 + j;
-                if (!CHAIN && s >= nsteps) break;
-                const int pW = s - 2;
-                // z phases of planes pW and pA = pW - 2 (s0 is a multiple of rho_z when RZ != 0)
-                const int phW = RZ ? ((j - 2) & (RZ - 1)) : (pW & rzm);
-                const int phA = RZ ? (j & (RZ - 1)) : ((pW - 2) & rzm);
+            for (int n = 0; n < 2; ++n)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) D[n][k] = sub2(U1[n][k], U0[n][k]);
+        }
+        float2 tm[2] = {z2, z2}, tc[2] = {z2, z2};        // t at planes pC - 1, pC
+        float2 cxp[2] = {z2, z2}, cyp[2] = {z2, z2};      // c'_x, c'_y at plane pA
+        float2 czm2[2] = {z2, z2}, czm1[2] = {z2, z2};    // c'_z at planes pA - 1, pA
+        float2 acc0[2][3], acc1[2][3];                    // z-node planes of pA's cell, [y node][component]
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) acc0[n][k] = acc1[n][k] = z2;
+        int yk = -1;                                       // node plane due for the y pass in this step
+
+        constexpr int U = RZ == 4 ? 4 : 2;   // unroll: whole cells where the phases are constants
+        for (int s0 = 0; s0 < nsteps; s0 += U) {
+#pragma unroll
+            for (int j = 0; j < U; ++j) {
+                const int s = s0 + j, sa = s & (kStages - 1);   // barrier and ring slot of a
+                if (s >= nsteps) break;
+                // z phases of planes pW = z0 + s - 2 and pA = pW - 2 (z0, and s0 when RZ != 0, are multiples of rho_z)
+                const int phW = RZ ? ((j - 2) & (RZ - 1)) : ((s - 2) & rzm);
+                const int phA = RZ ? (j & (RZ - 1)) : ((s - 4) & rzm);
                 const float fz = RZ ? (phW + 0.5f) / (float)(RZ ? RZ : 1) : (phW + 0.5f) * irz;
-                const float wz1 = RZ ? (phA + 0.5f) / (float)(RZ ? RZ : 1) : (phA + 0.5f) * irz;
+                const float wz = RZ ? (phA + 0.5f) / (float)(RZ ? RZ : 1) : (phA + 0.5f) * irz;
                 const bool cell_start = !DG && phW == 0 && s > 0;
+                const int sd2 = sd >= 2 ? sd - 2 : sd + kRingD - 2;   // slot of plane pA
 
                 // at a cell start, the node-plane copy issued two cells ago (the plane
                 // read in this step) lands before this barrier; the last one stays in flight
-                if (cell_start && node_warp) asm volatile("cp.async.wait_group 1;" ::: "memory");
-                // the stage of plane s - 1 and the buffers of the last plane were last read before this barrier
+                if (cell_start && node_thread) asm volatile("cp.async.wait_group 1;" ::: "memory");
+                // the slots issued below and the buffers of the last plane were last read before this barrier
                 __syncthreads();
                 if (w == kNW - 1) {
-                    // 3 planes ahead: of this column, then the first planes of the next one
-                    if (CHAIN ? s < nsteps - kAhead : s + kAhead < nsteps)
-                        issue_plane(x0, y0, s + kAhead, (j + kAhead) & (kStages - 1));
-                    else if (has_next)
-                        issue_plane(xn, yn, s + kAhead - nsteps, (j + kAhead) & (kStages - 1));
+                    // 3 steps ahead: of this column, then the first of the next one
+                    const int sd3 = sd >= kRingD - kAhead ? sd - (kRingD - kAhead) : sd + kAhead;
+                    const int sa3 = (s + kAhead) & (kStages - 1);
+                    if (s + kAhead < nsteps) issue(x0, y0, z0 + s + kAhead - 2, sd3, sa3);
+                    else if (has_next) issue(xn, yn, zn + s + kAhead - nsteps - 2, sd3, sa3);
                 }
-                // the node planes parked and x-reduced in the last steps move on
-                if (yk >= 0) y_pass(yk);
-                if (xk >= 0) x_pass(xk);
-                yk = xk;
-                xk = -1;
+                // the neighbour differences of the last planes, first: their shuffle and
+                // shared-memory latency overlaps what follows up to the TMA wait
+                const int bo = (j & 1) * exh;   // (U is even)
+                float2 dtx[2], dty[2], bxy[2];
+                if (!DG) {
+                    const float2 tu = ex_t[bo + up], td = ex_t[bo + dn];
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        const float sU = __shfl_up_sync(FULL, tc[r].y, 1), sD = __shfl_down_sync(FULL, tc[r].x, 1);
+                        dtx[r] = make_float2(tc[r].y - sU, sD - tc[r].x);
+                    }
+                    dty[0] = sub2(tc[1], tu);
+                    dty[1] = sub2(td, tc[0]);
+                }
+                {
+                    const float2 cu = ex_c[bo + up], cd = ex_c[bo + dn];
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        const float cxl = __shfl_up_sync(FULL, cxp[r].y, 1), cxr = __shfl_down_sync(FULL, cxp[r].x, 1);
+                        const float2 y0_ = r == 0 ? cu : cyp[0], y1_ = r == 0 ? cyp[1] : cd;
+                        if (DG) bxy[r] = add2(make_float2(cxl + cxp[r].y, cxp[r].x + cxr), add2(y0_, y1_));
+                        else bxy[r] = add2(make_float2(cxl - cxp[r].y, cxp[r].x - cxr), sub2(y0_, y1_));
+                    }
+                }
+                if (yk >= 0) y_pass(yk);   // the node plane completed in the last step
+                yk = -1;
 
                 // ------------------------------------------------ P v: the next node plane at a cell start
                 if (cell_start) {
-                    const int kz = pW >> lrz;
-                    float2 U1[3];
-                    bilinear(kz + 1, U1);
-                    for (int k = 0; k < 3; ++k) {
-                        U0[k] = add2(U0[k], D[k]);   // node plane kz (to one rounding)
-                        D[k] = sub2(U1[k], U0[k]);
-                    }
-                    if (node_warp) node_copy(kz + 3);   // read at the start of cell kz + 2
+                    const int kz = (z0 + s - 2) >> lrz;
+                    float2 U1[2][3];
+                    x_lines(kz + 1, U1);
+#pragma unroll
+                    for (int n = 0; n < 2; ++n)
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) {
+                            U0[n][k] = add2(U0[n][k], D[n][k]);   // node plane kz (to one rounding)
+                            D[n][k] = sub2(U1[n][k], U0[n][k]);
+                        }
+                    if (node_thread) node_copy(kz + 3);   // read at the start of the cell after the next
                 }
 
-                if constexpr (MULTI) {
-                    plane_wait(&bars[j], (pbits >> j) & 1u, a.err, a.poll_limit);
-                    pbits ^= 1u << j;
-                } else {
-                    plane_wait(&bars[j], phase, a.err, a.poll_limit);
-                }
+                plane_wait(&bars[sa], (pbits >> sa) & 1u, a.err, a.poll_limit);
+                pbits ^= 1u << sa;
                 // ------------------------------------------------ stage W: t at plane pW
-                const float2 *sW = sbase + j * (kStageF / 2);
-                const float2 dw0 = sW[0], dw1 = sW[kComp / 2], dw2 = sW[kComp];
-                // a' = a / (2 h), stored so by the linearisation
-                const float2 aw0 = sW[kBoxF / 2], aw1 = sW[(kBoxF + kComp) / 2], aw2 = sW[(kBoxF + 2 * kComp) / 2];
-                float2 tp;
+                float2 tp[2] = {z2, z2};
                 if (!DG) {
+                    const float2 *sW = lane_d + sd * kB2;
                     const float2 fz2 = bc2(fz);
-                    tp = mul2(dw0, fma2(fz2, D[0], U0[0]));
-                    tp = fma2(dw1, fma2(fz2, D[1], U0[1]), tp);
-                    tp = fma2(dw2, fma2(fz2, D[2], U0[2]), tp);
-                } else {
-                    tp = z2;
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        const float2 v0 = fma2(fz2, D[0][k], U0[0][k]), dv = sub2(fma2(fz2, D[1][k], U0[1][k]), v0);
+                        const float2 vA = fma2(fA2, dv, v0), vB = fma2(fB2, dv, v0);
+                        const float2 dA = sW[k * kC2], dB = sW[k * kC2 + kRow];
+                        tp[0] = k == 0 ? mul2(dA, vA) : fma2(dA, vA, tp[0]);
+                        tp[1] = k == 0 ? mul2(dB, vB) : fma2(dB, vB, tp[1]);
+                    }
                 }
 
                 // ------------------------------------------------ stage C: c' at plane pC = pW - 1
-                const int bo = (j & 1) * exh;
-                float2 c0, c1, c2;
-                if (DG) {
-                    c0 = mul2(a1[0], a1[0]); c1 = mul2(a1[1], a1[1]); c2 = mul2(a1[2], a1[2]);
-                } else {
-                    const float sU = __shfl_up_sync(FULL, t0.y, 1), sD = __shfl_down_sync(FULL, t0.x, 1);
-                    const float2 dtx = make_float2(t0.y - sU, sD - t0.x);
-                    const float2 dty = sub2(ex_t_dn[bo], ex_t_up[bo]);
-                    const float2 dr = fma2(a1[2], sub2(tp, tm), fma2(a1[1], dty, mul2(a1[0], dtx)));
-                    c0 = mul2(dr, a1[0]); c1 = mul2(dr, a1[1]); c2 = mul2(dr, a1[2]);
+                // (a' = a / (2 h), stored so by the linearisation)
+                float2 c0[2], c1[2], c2[2], dz[2];   // dz: c'_z at plane pA - 1 less that at pC
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const float2 *sA = lane_a + sa * kB2 + r * kRow;
+                    const float2 a0 = sA[0], a1 = sA[kC2], a2 = sA[2 * kC2];
+                    if (DG) {
+                        c0[r] = mul2(a0, a0); c1[r] = mul2(a1, a1); c2[r] = mul2(a2, a2);
+                        dz[r] = add2(czm2[r], c2[r]);
+                    } else {
+                        const float2 dr = fma2(a2, sub2(tp[r], tm[r]), fma2(a1, dty[r], mul2(a0, dtx[r])));
+                        c0[r] = mul2(dr, a0); c1[r] = mul2(dr, a1); c2[r] = mul2(dr, a2);
+                        dz[r] = fma2(make_float2(-dr.x, -dr.y), a2, czm2[r]);
+                    }
                 }
 
                 // ------------------------------------------------ stage A: G^T c at plane pA = pW - 2, times dT/dy
-                // (planes before the volume have dT/dy = 0 and add nothing)
-                {
-                    const float cxl = __shfl_up_sync(FULL, cxp.y, 1), cxr = __shfl_down_sync(FULL, cxp.x, 1);
-                    const float2 wz = bc2(wz1);
-                    if (DG) {
-                        const float2 bx = make_float2(cxl + cxp.y, cxp.x + cxr);
-                        const float2 beta = add2(add2(bx, add2(ex_c_up[bo], ex_c_dn[bo])), add2(czm2, c2));
-                        const float2 b1 = mul2(mul2(wz, wz), beta);
-                        const float2 b0 = mul2(bc2((1.f - wz1) * (1.f - wz1)), beta);
-                        for (int k = 0; k < 3; ++k) {
-                            const float2 qk2 = mul2(d2[k], d2[k]);
-                            acc0[k] = fma2(b0, qk2, acc0[k]);
-                            acc1[k] = fma2(b1, qk2, acc1[k]);
+                // (planes before the chunk, s < 4, only feed the hand-over)
+                if (s >= 4) {
+                    float2 b[2];
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) b[r] = add2(bxy[r], dz[r]);
+                    const float2 *sD = lane_d + sd2 * kB2;
+                    const float2 w1 = bc2(DG ? wz * wz : wz), w0 = bc2(DG ? (1.f - wz) * (1.f - wz) : 1.f - wz);
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        float2 dA = sD[k * kC2], dB = sD[k * kC2 + kRow];
+                        float2 ylo, yhi;   // the pair's sums onto its cell's lower and upper y node
+                        if (DG) {
+                            dA = mul2(b[0], mul2(dA, dA));
+                            dB = mul2(b[1], mul2(dB, dB));
+                            yhi = fma2(bc2(fyB * fyB), dB, mul2(bc2(fyA * fyA), dA));
+                            ylo = fma2(bc2((1.f - fyB) * (1.f - fyB)), dB, mul2(bc2((1.f - fyA) * (1.f - fyA)), dA));
+                        } else {
+                            dA = mul2(b[0], dA);
+                            const float2 sum = fma2(b[1], dB, dA);
+                            dB = mul2(b[1], dB);
+                            yhi = fma2(fB2, dB, mul2(fA2, dA));
+                            ylo = sub2(sum, yhi);
                         }
-                    } else {
-                        const float2 bx = make_float2(cxl - cxp.y, cxp.x - cxr);
-                        const float2 bsum = add2(add2(bx, sub2(ex_c_up[bo], ex_c_dn[bo])), sub2(czm2, c2));
-                        const float2 b1 = mul2(wz, bsum), b0 = sub2(bsum, b1);
-                        for (int k = 0; k < 3; ++k) {
-                            acc0[k] = fma2(b0, d2[k], acc0[k]);
-                            acc1[k] = fma2(b1, d2[k], acc1[k]);
-                        }
+                        // a cell's first plane: its lower node plane is the upper one of the cell below
+                        acc0[0][k] = fma2(w0, ylo, phA == 0 ? acc1[0][k] : acc0[0][k]);
+                        acc1[0][k] = phA == 0 ? mul2(w1, ylo) : fma2(w1, ylo, acc1[0][k]);
+                        acc0[1][k] = fma2(w0, yhi, phA == 0 ? acc1[1][k] : acc0[1][k]);
+                        acc1[1][k] = phA == 0 ? mul2(w1, yhi) : fma2(w1, yhi, acc1[1][k]);
                     }
-                    if (phA == (RZ ? RZ - 1 : rzm) && s0 > 0) {
-                        // node plane (pA >> lrz) is complete: park it (x pass next step, y pass after)
-                        const int kz = (s - 4) >> lrz;
-                        park_plane(acc0, kz);
-                        xk = kz;
-                        for (int k = 0; k < 3; ++k) {
-                            acc0[k] = acc1[k];
-                            acc1[k] = z2;
-                        }
+                    if (phA == (RZ ? RZ - 1 : rzm)) {
+                        // the cell's lower node plane is complete: park it (y pass in the next step)
+                        yk = (s - 4) >> lrz;
+                        park(acc0, yk);
                     }
                 }
                 // ------------------------------------------------ hand over to the next plane
-                ex_t[exh - bo] = tp;
-                ex_c[exh - bo] = c1;
-                tm = t0; t0 = tp;
-                czm2 = czm1; czm1 = c2;
-                cxp = c0;
-                for (int k = 0; k < 3; ++k) d2[k] = d1[k];
-                d1[0] = dw0; d1[1] = dw1; d1[2] = dw2;
-                a1[0] = aw0; a1[1] = aw1; a1[2] = aw2;
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    ex_t[exh - bo + 32 * r] = tp[r];
+                    ex_c[exh - bo + 32 * r] = c1[r];
+                    tm[r] = tc[r]; tc[r] = tp[r];
+                    czm2[r] = czm1[r]; czm1[r] = c2[r];
+                    cxp[r] = c0[r]; cyp[r] = c1[r];
+                }
+                sd = sd == kRingD - 1 ? 0 : sd + 1;
             }
         }
-        // the pending passes and the top node plane (above the last cell)
+        // the pending node plane and the top one (above the last cell)
+        const int top = nz >> lrz;
         __syncthreads();
         if (yk >= 0) y_pass(yk);
-        if (xk >= 0) x_pass(xk);
-        park_plane(acc0, g.m[2] - 1);
+        park(acc1, top);
         __syncthreads();
-        if (xk >= 0) y_pass(xk);
-        x_pass(g.m[2] - 1);
-        __syncthreads();
-        y_pass(g.m[2] - 1);
+        y_pass(top);
         if (!has_next) break;
         t = tn;
     }
-    if constexpr (MULTI) {   // the node-plane copies still in flight land before the CTA moves on
-        if (!DG && node_warp) asm volatile("cp.async.wait_all;" ::: "memory");
-        __syncthreads();
-    }
+    if (!DG) asm volatile("cp.async.wait_all;" ::: "memory");   // the node-plane copies still in flight
+    __syncthreads();   // a caller may reuse the shared memory
 }
 
 }  // namespace gnpk

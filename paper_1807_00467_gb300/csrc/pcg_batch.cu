@@ -41,12 +41,14 @@ namespace ngf {
 namespace {
 
 using gnpk::kNT;
-constexpr int kVccRun = kNT / vcck::NC;        // VCC cell blocks at once (5 x 128 threads)
-constexpr int kNodeRun = kNT / nodek::NT;      // node tiles at once (2 x 256 threads, 128 idle)
+constexpr int kVccT = vcck::NC / 2;            // threads of a VCC cell block (two cells each)
+constexpr int kVccRun = kNT / kVccT;           // VCC cell blocks at once (5 x 64 threads)
+constexpr int kNodeRun = kNT / nodek::NT;      // node tiles at once (256 threads, 64 idle)
+constexpr int kVecS = 2, kVecT = pcgk::kVT / kVecS;   // a PCG vector block's threads stand for two each
 // units per work item: the light phases take several rounds per item, so the
 // per-item cost (work counter, completion record) stays small
 constexpr int kVccPer = 4 * kVccRun, kNodePer = 8 * kNodeRun, kVecPer = 2;
-static_assert(pcgk::kVT <= kNT, "a PCG vector block fits in a CTA");
+static_assert(kVecT <= kNT, "a PCG vector block fits in a CTA");
 
 struct KPair {
     BatchPair b;
@@ -54,7 +56,6 @@ struct KPair {
     int nvec;              // vector blocks
     int ncols, nvcc, nnode;
     int nA, nB, nV;        // items of phase A (columns, VCC groups, curvature groups), B and each vector phase
-    int rz, rxy;           // GN-product specialisation: rho_z ring phases (0: generic), rho 4 x 4
 };
 
 struct KArgs {
@@ -154,14 +155,11 @@ __device__ __forceinline__ VBlock node_block(const KPair &P, int tid, int bid, i
 
 __device__ __forceinline__ void gn_column(const KPair &P, float *smem, uint64_t *bars, int t, uint32_t &pbits) {
     const ColArgs &a = P.b.col;
-    if (P.rxy == 4) {
-        switch (P.rz) {
-            case 2: gnpk::gn_product_body<2, false, false, 4, true>(a, smem, bars, t, 1, false, pbits); return;
-            case 4: gnpk::gn_product_body<4, false, false, 4, true>(a, smem, bars, t, 1, false, pbits); return;
-            default: gnpk::gn_product_body<0, false, false, 4, true>(a, smem, bars, t, 1, false, pbits); return;
-        }
+    switch (a.g.rho[0]) {
+        case 2: gnpk::gn_product_body<2, 0, false>(a, smem, bars, t, 1, false, false, pbits); return;
+        case 4: gnpk::gn_product_body<4, 0, false>(a, smem, bars, t, 1, false, false, pbits); return;
+        default: gnpk::gn_product_body<8, 0, false>(a, smem, bars, t, 1, false, false, pbits);
     }
-    gnpk::gn_product_body<0, false, false, 0, true>(a, smem, bars, t, 1, false, pbits);
 }
 
 __global__ void __launch_bounds__(kNT, 1) pcg_batch_kernel(const __grid_constant__ KArgs A) {
@@ -194,12 +192,12 @@ __global__ void __launch_bounds__(kNT, 1) pcg_batch_kernel(const __grid_constant
             if (r < A.colOff[np]) {
                 gn_column(P, smem, bars, r - A.colOff[p], pbits);
             } else if (r < A.vccOff[np]) {
-                const int v = tid / vcck::NC;
+                const int v = tid / kVccT;
                 const int *nb = P.b.vcc.nb;
                 for (int bid = (r - A.vccOff[p]) * kVccPer + v, e = min(bid - v + kVccPer, P.nvcc); bid < e;
                      bid += kVccRun) {
-                    const VBlock b = warp_block(tid % vcck::NC, bid, nb[0], nb[1], nb[2], 1 + v, vcck::NC);
-                    vcck::vcc_cell_body<1, float>(P.b.vcc, b, reinterpret_cast<vcck::VccSmem<float> *>(smem)[v]);
+                    const VBlock b = warp_block(tid % kVccT, bid, nb[0], nb[1], nb[2], 1 + v, kVccT);
+                    vcck::vcc_cell_body<1, float2>(P.b.vcc, b, reinterpret_cast<vcck::VccSmem<float2> *>(smem)[v]);
                 }
             } else {
                 const int v = tid / nodek::NT;
@@ -236,18 +234,18 @@ __global__ void __launch_bounds__(kNT, 1) pcg_batch_kernel(const __grid_constant
         const unsigned need = (unsigned)(k + 1) * (ph == 0 ? P.nB : P.nV);
         if (!wait_done(A, p, 1 + ph, need, &s_ok)) return;
         const int b0 = (r - A.vecOff[p]) * kVecPer;
-        for (int vb = b0; tid < pcgk::kVT && vb < min(b0 + kVecPer, P.nvec); ++vb) {
-            const VBlock b = warp_block(tid, vb, P.nvec, 1, 1, 1, pcgk::kVT);
+        for (int vb = b0; tid < kVecT && vb < min(b0 + kVecPer, P.nvec); ++vb) {
+            const VBlock b = warp_block(tid, vb, P.nvec, 1, 1, 1, kVecT);
             const PcgArgs &g = P.b.pcg;
             pcgk::PcgSmem &sm = *reinterpret_cast<pcgk::PcgSmem *>(smem);
             if (vb > b0) b.sync();   // the last block's reads of the shared scratch are done
             if (ph == 0)
-                pcgk::pcg_step_body(P.part, g.sc, g.apart, P.nnode, P.b.nodes.out, g.minv, g.Rh, g.stride, k, g.part,
+                pcgk::pcg_step_body<0, kVecS>(P.part, g.sc, g.apart, P.nnode, P.b.nodes.out, g.minv, g.Rh, g.stride, k, g.part,
                                     b, sm);
             else if (ph == 1)
-                pcgk::pcg_reorth_body(P.part, g.sc, g.minv, g.Rh, g.stride, k, g.rzh, g.part, g.rzpart, b, sm);
+                pcgk::pcg_reorth_body<0, kVecS>(P.part, g.sc, g.minv, g.Rh, g.stride, k, g.rzh, g.part, g.rzpart, b, sm);
             else
-                pcgk::pcg_dir_body(P.part, g.sc, g.minv, g.Rh + (long)(k + 1) * g.stride, g.d, P.b.s, k, g.rzh,
+                pcgk::pcg_dir_body<kVecS>(P.part, g.sc, g.minv, g.Rh + (long)(k + 1) * g.stride, g.d, P.b.s, k, g.rzh,
                                    g.rzpart, b, sm);
         }
         item_done(A, p, 2 + ph, it);
@@ -256,7 +254,7 @@ __global__ void __launch_bounds__(kNT, 1) pcg_batch_kernel(const __grid_constant
 
 size_t batch_smem(const KArgs &A) {
     size_t s = std::max(sizeof(pcgk::PcgSmem),
-                        std::max(kVccRun * sizeof(vcck::VccSmem<float>), kNodeRun * sizeof(nodek::NodeSmem)));
+                        std::max(kVccRun * sizeof(vcck::VccSmem<float2>), kNodeRun * sizeof(nodek::NodeSmem)));
     for (int p = 0; p < A.npairs; ++p) s = std::max(s, sizeof(float) * (size_t)gnpk::pc_smem(A.p[p].b.col.g).total);
     return s;
 }
@@ -288,11 +286,9 @@ cudaError_t launch_pcg_batch(const BatchPair *pairs, int npairs, int iters, unsi
         if (!pcg_batch_supported(g) || !P.b.s || P.b.pcg.n != 3L * g.m[0] * g.m[1] * g.m[2])
             return cudaErrorInvalidValue;
         P.part = pcgk::make_part(P.b.pcg.n, &P.nvec);
-        P.ncols = g.nb[0] * g.nb[1];
+        P.ncols = g.nb[0] * g.nb[1] * g.nbz;
         P.nvcc = P.b.vcc_on ? P.b.vcc.nb[0] * P.b.vcc.nb[1] * P.b.vcc.nb[2] : 0;
         P.nnode = node_blocks(g.m);
-        P.rz = (g.rho[2] == 2 || g.rho[2] == 4) ? g.rho[2] : 0;
-        P.rxy = (g.rho[0] == 4 && g.rho[1] == 4) ? 4 : 0;
         P.nB = (P.nnode + kNodePer - 1) / kNodePer;
         P.nA = P.ncols + (P.nvcc + kVccPer - 1) / kVccPer + P.nB;
         P.nV = (P.nvec + kVecPer - 1) / kVecPer;
