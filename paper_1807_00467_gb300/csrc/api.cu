@@ -357,6 +357,7 @@ static void derive(rg_ctx *c) {
         if (n > c->nA_cap) c->nA_cap = n;
         if (n * 3 * t.box > c->boxA_cap) c->boxA_cap = n * 3 * t.box;
     }
+    if (c->nA_cap < kGobjMax) c->nA_cap = kGobjMax;   // (also the D partials)
     for (int i = 0; i < 2; ++i) {
         ColGeom &g = i ? c->cp : c->cg;
         BoxGeom &b = i ? c->bP : c->bM;
@@ -634,43 +635,41 @@ static int run_tile(rg_ctx *c, int mode, const float *field) {
         return RG_OK;
     }
     c->nD = c->nA;
-    // the column-marching pass where it covers the volume with at least one
-    // column per SM (narrower volumes keep the z-chunked tile pass, whose
-    // tiles fill the GPU)
-    const bool gcol = mode != MODE_MATVEC && mode != MODE_DIAG && !c->general_only && c->pass_sel != 2 &&
-                      ngf_gcol_supported(c->cg) &&
+    // the column-marching passes: the objective wherever it applies (its planes
+    // are dealt evenly to the SMs), the gradient and linearisation where the
+    // volume has at least one column per SM (narrower volumes keep the z-chunked
+    // tile pass, whose tiles fill the GPU)
+    const bool colpass = mode != MODE_MATVEC && mode != MODE_DIAG && !c->general_only && c->pass_sel != 2;
+    const bool gobj = colpass && mode == MODE_OBJ && ngf_gobj_supported(c->cg);
+    const bool gcol = colpass && mode != MODE_OBJ && ngf_gcol_supported(c->cg) &&
                       (c->pass_sel == 1 || c->cg.nb[0] * c->cg.nb[1] >= device_sm_count());
-    if (gcol) {
-        // objective, gradient and linearisation: the column-marching pass
-        auto gfill = [&](auto &g) {
+    if (gobj || gcol) {
+        auto run = [&](auto &g, auto *R, auto *T) {
             g.g = c->cg;
             for (int i = 0; i < 3; ++i) {
                 g.invh[i] = c->tg.invh[i];
                 g.invh_rel[i] = c->tg.invh_rel[i];
             }
             g.eta2 = c->tg.eta2;
+            g.R = R;
+            g.T = T;
             g.u = field;
             g.st_dT = c->lin_dT;
             g.st_a = c->lin_a;
             g.boxes = c->boxA;
             g.dpart = c->dpart;
             g.skip = c->skip;
+            return gobj ? launch_ngf_gobj(g, c->st) : launch_ngf_gcol(mode, g, c->st);
         };
         if (c->dtype == RG_F32) {
             GcolArgs<float> g;
-            gfill(g);
-            g.R = (const float *)c->R;
-            g.T = (const float *)c->T;
-            LAUNCH(pid, launch_ngf_gcol(mode, g, c->st));
+            LAUNCH(pid, run(g, (const float *)c->R, (const float *)c->T));
         } else {
             GcolArgs<__half> g;
-            gfill(g);
-            g.R = (const __half *)c->R;
-            g.T = (const __half *)c->T;
-            LAUNCH(pid, launch_ngf_gcol(mode, g, c->st));
+            LAUNCH(pid, run(g, (const __half *)c->R, (const __half *)c->T));
         }
         c->bcur = &c->bM;
-        c->nD = c->cg.nb[0] * c->cg.nb[1];
+        c->nD = gobj ? ngf_gobj_blocks(c->cg) : c->cg.nb[0] * c->cg.nb[1];
         return RG_OK;
     }
     // objective, gradient and linearisation: the persistent pass where the tile shape allows

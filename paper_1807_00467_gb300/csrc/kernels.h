@@ -46,6 +46,15 @@ bool ngf_gcol_supported(const ColGeom &g);
 cudaError_t launch_ngf_gcol(int mode, const GcolArgs<float> &a, cudaStream_t st);
 cudaError_t launch_ngf_gcol(int mode, const GcolArgs<__half> &a, cudaStream_t st);
 
+// Column-marching objective pass (ngf_gobj.cu): one partial of 1 - r^2 per block
+// (ngf_gobj_blocks, at most kGobjMax); of the arguments g, invh, invh_rel, eta2,
+// R, T, u, dpart and skip are read.
+constexpr int kGobjMax = 152;
+bool ngf_gobj_supported(const ColGeom &g);
+int ngf_gobj_blocks(const ColGeom &g);
+cudaError_t launch_ngf_gobj(const GcolArgs<float> &a, cudaStream_t st);
+cudaError_t launch_ngf_gobj(const GcolArgs<__half> &a, cudaStream_t st);
+
 // Volume change control, Eqs. (7)-(9): per grid cell the 64 bounds d_abc.
 struct VccArgs {
     int m[3];

@@ -1,5 +1,5 @@
-// NGF objective, gradient and Gauss-Newton linearisation (Eq. (1)), the
-// column-marching form: the pass of ngf_grad.cu (trilinear warp of the
+// NGF gradient (with the objective's value) and Gauss-Newton linearisation
+// (Eq. (1)), the column-marching form: the pass of ngf_grad.cu (trilinear warp of the
 // template at y = x + P u, central-difference gradients of R and of the warped
 // template, the per-voxel residual r and 1 - r^2, the adjoint of the central
 // difference and P^T onto the grid nodes) on the column layout of the
@@ -27,7 +27,7 @@
 // lane (hat-weighted lower and upper parts), reduced along x by all threads
 // in the next plane and along y in the plane after, into the column's node
 // box [3][m3][C1 + 1][C0 + 1] (the GN product's boxes; the node pass sums
-// neighbouring columns).  The objective-only mode runs W and C.
+// neighbouring columns).  (The objective alone: ngf_gobj.cu.)
 #include "common.cuh"
 #include "kernels.h"
 
@@ -43,16 +43,16 @@ struct GcSmem {
     int ext, exr, exc, nodes, park, xr, dts, us, total;
 };
 
-__host__ __device__ inline GcSmem gc_smem(const ColGeom &g, bool adj) {
+__host__ __device__ inline GcSmem gc_smem(const ColGeom &g) {
     GcSmem s;
     int off = 0;
     s.ext = off; off += 2 * kEx;                                   // T(y) of plane C, double-buffered
     s.exr = off; off += 2 * kEx;                                   // R of plane C
-    s.exc = off; off += adj ? 2 * kEx : 0;                         // c_y of plane A
+    s.exc = off; off += 2 * kEx;                         // c_y of plane A
     s.nodes = off; off += 4 * ((g.nyt * g.nxt + 31) & ~31) * 4;    // node planes of u, [slot][y][x][xyz_]
-    s.park = off; off += adj ? 2 * kTY * 32 * 6 : 0;               // parked lane parts of 2 node planes
-    s.xr = off; off += adj ? 2 * kTY * (g.C0 + 1) * 3 : 0;         // x-reduced rows of 2 node planes
-    s.dts = off; off += adj ? 2 * 3 * kNT * 2 : 0;                 // per thread: dT/dy of 2 planes
+    s.park = off; off += 2 * kTY * 32 * 6;               // parked lane parts of 2 node planes
+    s.xr = off; off += 2 * kTY * (g.C0 + 1) * 3;         // x-reduced rows of 2 node planes
+    s.dts = off; off += 2 * 3 * kNT * 2;                 // per thread: dT/dy of 2 planes
     s.us = off; off += 2 * 3 * kNT * 2;                             // per thread: P u at 2 node planes
     s.total = off;
     return s;
@@ -129,10 +129,10 @@ __device__ __forceinline__ Place place(float pu, float ih, float ihrel, int i, i
 template <int MODE, typename TImg, int RZ, int RXY>
 __global__ void __launch_bounds__(kNT, 1) ngf_gcol_kernel(const __grid_constant__ GcolArgs<TImg> a) {
     if (a.skip && *a.skip) return;   // uniform: every block reads the same flag
-    constexpr bool ADJ = MODE != MODE_OBJ, STORE = MODE == MODE_GRADLIN;
+    constexpr bool STORE = MODE == MODE_GRADLIN;
     extern __shared__ __align__(16) float smem[];
     const ColGeom &g = a.g;
-    const GcSmem S = gc_smem(g, ADJ);
+    const GcSmem S = gc_smem(g);
 
     const int tid = threadIdx.x, L = tid & 31, w = tid >> 5;
     const int ncols = g.nb[0] * g.nb[1];
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(kNT, 1) ngf_gcol_kernel(const __grid_constant_
 
         {
             float *ex = smem + S.ext;
-            for (int i = tid; i < (ADJ ? 6 : 4) * kEx; i += kNT) ex[i] = 0.f;
+            for (int i = tid; i < 6 * kEx; i += kNT) ex[i] = 0.f;
         }
         __syncthreads();   // node ring filled, exchange rows cleared; the previous column's passes are done
 
@@ -302,8 +302,7 @@ __global__ void __launch_bounds__(kNT, 1) ngf_gcol_kernel(const __grid_constant_
         float2 tm = z2, t0 = z2, rm = z2, r0 = z2;        // T(y) and R at planes pC - 1, pC
         // this thread's dT/dy of planes pW - 2 and pW - 1: [slot = plane parity][component], stride kNT
         float2 *dts = reinterpret_cast<float2 *>(smem + S.dts) + tid;
-        if (ADJ)
-            for (int i = 0; i < 6; ++i) dts[i * kNT] = z2;
+        for (int i = 0; i < 6; ++i) dts[i * kNT] = z2;
         float2 cxp = z2, czm2 = z2, czm1 = z2;             // c of the adjoint at planes pA, pA - 1
         float2 acc0[3] = {z2, z2, z2}, acc1[3] = {z2, z2, z2};
         float ds_e = 0.f, dc_e = 0.f, ds_o = 0.f, dc_o = 0.f;   // Kahan sums of 1 - r^2
@@ -320,7 +319,7 @@ __global__ void __launch_bounds__(kNT, 1) ngf_gcol_kernel(const __grid_constant_
                 const bool cell_start = phW == 0 && s > 0;
                 if (cell_start && node_warp) asm volatile("cp.async.wait_group 1;" ::: "memory");
                 __syncthreads();
-                if (ADJ) {
+                {
                     if (yk >= 0) y_pass(yk);
                     if (xk >= 0) x_pass(xk);
                     yk = xk;
@@ -365,7 +364,7 @@ __global__ void __launch_bounds__(kNT, 1) ngf_gcol_kernel(const __grid_constant_
                     const float2 w0 = fma2(f1, dy0, v00), w1 = fma2(f1, dy1, v01);
                     const float2 dz = sub2(w1, w0);
                     val = fma2(f2, dz, w0);
-                    if (ADJ) {
+                    {
                         const float2 ax0 = fma2(f1, sub2(dx10, dx00), dx00), ax1 = fma2(f1, sub2(dx11, dx01), dx01);
                         // derivative scale 1/h with the step's sign, zero along a clamped axis
                         const float2 sx2 = make_float2(xe.in ? ih0 * (float)xe.st : 0.f, xo.in ? ih0 * (float)xo.st : 0.f);
@@ -416,7 +415,7 @@ __global__ void __launch_bounds__(kNT, 1) ngf_gcol_kernel(const __grid_constant_
                     const bool oz = pC >= 0 && pC < nz;
                     kahan_add(ds_e, dc_e, (own_e && oz && ie) ? dv.x : 0.f);
                     kahan_add(ds_o, dc_o, (own_o && oz && io) ? dv.y : 0.f);
-                    if (ADJ) {
+                    {
                         // a = dr/dg = (f |g|^2 - <f,g> g) / (|f| |g|^3); c = d(1 - r^2)/dg =
                         // -2 <f,g> q / (|f|^2 |g|^4); both times 1/(2h) per axis
                         const float2 q0 = xprod(f0, gg, fg, g0), q1 = xprod(f1, gg, fg, g1);
@@ -438,7 +437,7 @@ __global__ void __launch_bounds__(kNT, 1) ngf_gcol_kernel(const __grid_constant_
                 }
 
                 // ------------------------------------------------ stage A: plane pA = pW - 2
-                if (ADJ) {
+                {
                     const float cxl = __shfl_up_sync(FULL, cxp.y, 1), cxr = __shfl_down_sync(FULL, cxp.x, 1);
                     const int phA = RZ ? (j & (RZ - 1)) : ((pW - 2) & rzm);
                     const float wz1 = RZ ? (phA + 0.5f) / (float)(RZ ? RZ : 1) : (phA + 0.5f) * irz;
@@ -471,7 +470,7 @@ __global__ void __launch_bounds__(kNT, 1) ngf_gcol_kernel(const __grid_constant_
                 rm = r0; r0 = rv;
             }
         }
-        if (ADJ) {   // the pending passes and the top node plane (above the last cell)
+        {   // the pending passes and the top node plane (above the last cell)
             __syncthreads();
             if (yk >= 0) y_pass(yk);
             if (xk >= 0) x_pass(xk);
@@ -500,14 +499,13 @@ __global__ void __launch_bounds__(kNT, 1) ngf_gcol_kernel(const __grid_constant_
 
 bool ngf_gcol_supported(const ColGeom &g) {
     if (g.rho[0] < 2 || g.n[0] % 2 || g.n[0] < 64 || g.n[1] < 20 || g.m[2] > 256 || g.nxt * g.nyt > kNT) return false;
-    return (size_t)gc_smem(g, true).total * sizeof(float) <= 227u * 1024u;
+    return (size_t)gc_smem(g).total * sizeof(float) <= 227u * 1024u;
 }
 
 template <typename TImg>
 static cudaError_t launch_gcol(int mode, const GcolArgs<TImg> &a, cudaStream_t st) {
     if (!ngf_gcol_supported(a.g)) return cudaErrorInvalidValue;
-    const bool adj = mode != MODE_OBJ;
-    const size_t smem = sizeof(float) * (size_t)gc_smem(a.g, adj).total;
+    const size_t smem = sizeof(float) * (size_t)gc_smem(a.g).total;
     const int ncols = a.g.nb[0] * a.g.nb[1];
     const int sms = device_sm_count();
     const int grid = ncols < sms ? ncols : sms;
@@ -521,7 +519,6 @@ static cudaError_t launch_gcol(int mode, const GcolArgs<TImg> &a, cudaStream_t s
 #define NGF_GC(M) (r44 ? (r2 ? run(ngf_gcol_kernel<M, TImg, 2, 4>) : run(ngf_gcol_kernel<M, TImg, 0, 4>)) \
                        : (r2 ? run(ngf_gcol_kernel<M, TImg, 2, 0>) : run(ngf_gcol_kernel<M, TImg, 0, 0>)))
     switch (mode) {
-        case MODE_OBJ: return NGF_GC(MODE_OBJ);
         case MODE_GRAD: return NGF_GC(MODE_GRAD);
         case MODE_GRADLIN:
         case MODE_LIN: return NGF_GC(MODE_GRADLIN);
