@@ -148,6 +148,13 @@ static int check_geom(const rg_image_geom *img, const rg_grid_geom *grid) {
     return RG_OK;
 }
 
+// Row pitch (floats) of the stored linearisation: a TMA tensor's strides are
+// multiples of 16 bytes, so rows are padded to four voxels (dense rows of 182
+// voxels took the general tile kernel's plain loads: product 93 us at
+// 182x150x94, against 39 us for the column kernel).  The padding is never read: the
+// tensors end at n1.
+static long lin_pitch(int n0) { return (n0 + 3) & ~3; }
+
 // Tile shape: TXI x TY voxel columns in x-y (one thread per column, plus a
 // 2-voxel halo: TXI + 4 <= 32 lanes), TZ voxel planes per z chunk.
 //
@@ -202,6 +209,7 @@ static void tile_geom(const rg_image_geom *img, const rg_grid_geom *grid, TileGe
     t.nb[1] = (t.n[1] + t.TY - 1) / t.TY;
     t.nb[2] = (t.n[2] + t.TZ - 1) / t.TZ;
     t.tma = 0;
+    t.lp = (int)lin_pitch(t.n[0]);
     // node planes of the chunk and its 2-plane halo, preloaded once per CTA if they fit in 48 KB
     t.nzt = (t.TZ + 3) / t.rho[2] + 3;
     if ((long)t.nzt * 3 * t.nxt * t.nyt > 12 * 1024) t.nzt = 0;
@@ -245,6 +253,7 @@ static void col_geom(const rg_image_geom *img, const rg_grid_geom *grid, ColGeom
     c.nbz = (c.n[2] + c.TZ - 1) / c.TZ;
     c.box = (c.C0 + 1) * (c.C1 + 1) * (c.TZ / c.rho[2] + 1);
     c.tma = 0;
+    c.lp = (int)lin_pitch(c.n[0]);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -254,9 +263,9 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
 // TMA maps over a stored [3][n3][n2][n1] float field as the 4-D tensor
 // {x, y, z, component}; box {box_x, TY + 4, 1, 3}.  Returns false (and the
 // kernels read with plain loads) when the driver entry point is unavailable or
-// the row pitch is not a multiple of 16 bytes.
+// the volume is narrower than a box.  Rows are lin_pitch floats apart.
 static bool encode_field_map(CUtensorMap *map, const int *n, int TY, float *base, int box_x = kTmaBoxX) {
-    if (n[0] % 4 != 0 || n[0] < box_x || n[1] < TY + 4) return false;
+    if (n[0] < box_x || n[1] < TY + 4) return false;
     static const EncodeTiledFn fn = [] {   // looked up once, also under concurrent callers
         void *f = nullptr;
         cudaDriverEntryPointQueryResult q;
@@ -269,8 +278,8 @@ static bool encode_field_map(CUtensorMap *map, const int *n, int TY, float *base
     }();
     if (!fn) return false;
     const cuuint64_t dims[4] = {(cuuint64_t)n[0], (cuuint64_t)n[1], (cuuint64_t)n[2], 3};
-    const cuuint64_t strides[3] = {(cuuint64_t)n[0] * 4, (cuuint64_t)n[0] * n[1] * 4,
-                                   (cuuint64_t)n[0] * n[1] * n[2] * 4};
+    const cuuint64_t pitch = lin_pitch(n[0]) * 4;
+    const cuuint64_t strides[3] = {pitch, pitch * n[1], pitch * n[1] * n[2]};
     const cuuint32_t box[4] = {(cuuint32_t)box_x, (cuuint32_t)(TY + 4), 1, 3};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -299,9 +308,10 @@ struct Carver {
 };
 
 static void layout(rg_ctx *c, Carver &cv) {
-    const long N = c->N, M = c->M;
-    c->lin_dT = cv.take<float>(3 * N);
-    c->lin_a = cv.take<float>(3 * N);
+    const long M = c->M;
+    const long NL = lin_pitch(c->img.n[0]) * c->img.n[1] * c->img.n[2];
+    c->lin_dT = cv.take<float>(3 * NL);
+    c->lin_a = cv.take<float>(3 * NL);
     c->lin_u = cv.take<float>(3 * M);
     c->boxA = cv.take<float>((size_t)c->boxA_cap);
     c->boxB = cv.take<float>((size_t)c->nB * 3 * c->bB.box);

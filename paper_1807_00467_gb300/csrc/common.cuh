@@ -75,6 +75,7 @@ struct TileGeom {
     int nzt;           // node planes preloaded per CTA (0: two planes streamed as needed)
     int box;           // floats per box per component: (C0+1)(C1+1)(C2+1)
     int tma;           // 1: stream the stored linearisation with TMA (tensor maps valid)
+    int lp;            // row pitch of the stored linearisation, floats
 };
 
 template <typename TImg>
@@ -83,10 +84,10 @@ struct TileArgs {
     const TImg *R;          // reference image
     const TImg *T;          // template image
     const float *u;         // node field interpolated per voxel (u, or v for the matvec)
-    const float *lin_dT;    // stored dT/dy [3][N] (matvec input)
-    const float *lin_a;     // stored dr/dg [3][N], component a scaled by 1 / (2 h_a) (matvec input)
-    float *st_dT;           // linearisation output dT/dy [3][N]
-    float *st_a;            // linearisation output dr/dg [3][N], component a scaled by 1 / (2 h_a)
+    const float *lin_dT;    // stored dT/dy [3][n3][n2][lp] (matvec input)
+    const float *lin_a;     // stored dr/dg [3][n3][n2][lp], component a scaled by 1 / (2 h_a) (matvec input)
+    float *st_dT;           // linearisation output dT/dy [3][n3][n2][lp]
+    float *st_a;            // linearisation output dr/dg [3][n3][n2][lp], component a scaled by 1 / (2 h_a)
     float *boxes;           // per-CTA node partials [cta][3][C2+1][C1+1][C0+1]
     double *dpart;          // per-CTA partial sums of (1 - r^2)
     // Stored linearisation streamed by TMA (GN product and diagonal): tensor
@@ -120,6 +121,7 @@ struct ColGeom {
     int TZ, nbz;       // z planes per chunk (whole cells), chunks (1 but on small volumes)
     int box;           // floats per component of a column's node box: (C0 + 1)(C1 + 1)(TZ / rho_z + 1)
     int tma;           // 1: tensor maps valid
+    int lp;            // row pitch of the stored linearisation, floats
 };
 
 struct ColArgs {

@@ -136,7 +136,8 @@ __global__ void __launch_bounds__(kNT, 1) ngf_gcol_kernel(const __grid_constant_
 
     const int tid = threadIdx.x, L = tid & 31, w = tid >> 5;
     const int ncols = g.nb[0] * g.nb[1];
-    const int nx = g.n[0], ny = g.n[1], nz = g.n[2], sxy = nx * ny, N = sxy * nz;
+    const int nx = g.n[0], ny = g.n[1], nz = g.n[2], sxy = nx * ny;
+    const int lsxy = g.lp * ny, lN = lsxy * nz;   // the stored linearisation: row pitch lp
     const int lrx = g.lrho[0], lry = g.lrho[1], lrz = g.lrho[2];
     const int rx = g.rho[0], half = rx >> 1, rzm = g.rho[2] - 1;
     const float irz = g.irho[2];
@@ -374,10 +375,10 @@ __global__ void __launch_bounds__(kNT, 1) ngf_gcol_kernel(const __grid_constant_
                         dw[1] = mul2(fma2(f2, sub2(dy1, dy0), dy0), sy2);
                         dw[2] = mul2(dz, sz2);
                         if (STORE && own_pair && pair_in && pW >= 0 && pW < nz) {
-                            const long v = (long)pW * sxy + col;
+                            const long v = (long)pW * lsxy + (col + gy * (g.lp - nx));
                             *reinterpret_cast<float2 *>(a.st_dT + v) = dw[0];
-                            *reinterpret_cast<float2 *>(a.st_dT + N + v) = dw[1];
-                            *reinterpret_cast<float2 *>(a.st_dT + 2 * (long)N + v) = dw[2];
+                            *reinterpret_cast<float2 *>(a.st_dT + lN + v) = dw[1];
+                            *reinterpret_cast<float2 *>(a.st_dT + 2 * (long)lN + v) = dw[2];
                         }
                     }
                 }
@@ -428,10 +429,10 @@ __global__ void __launch_bounds__(kNT, 1) ngf_gcol_kernel(const __grid_constant_
                         if (STORE && own_pair && pair_in && oz) {
                             const float2 inv = make_float2(ie ? rsqrtf(ff.x * gg.x) * rgg.x : 0.f,
                                                            io ? rsqrtf(ff.y * gg.y) * rgg.y : 0.f);
-                            const long v = (long)pC * sxy + col;
+                            const long v = (long)pC * lsxy + (col + gy * (g.lp - nx));
                             *reinterpret_cast<float2 *>(a.st_a + v) = mul2(mul2(q0, inv), i2h0);
-                            *reinterpret_cast<float2 *>(a.st_a + N + v) = mul2(mul2(q1, inv), i2h1);
-                            *reinterpret_cast<float2 *>(a.st_a + 2 * (long)N + v) = mul2(mul2(q2, inv), i2h2);
+                            *reinterpret_cast<float2 *>(a.st_a + lN + v) = mul2(mul2(q1, inv), i2h1);
+                            *reinterpret_cast<float2 *>(a.st_a + 2 * (long)lN + v) = mul2(mul2(q2, inv), i2h2);
                         }
                     }
                 }

@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kNT, 1) ngf_grad_kernel(const __grid_constant_
     const int tid = threadIdx.x, L = tid & 31, w = tid >> 5;
     const int TXI = g.TXI, nx = g.n[0], ny = g.n[1], nz = g.n[2];
     const int sxy = nx * ny;
-    const int N = sxy * nz;
+    const long lsxy = (long)g.lp * ny, lN = lsxy * nz;   // the stored linearisation: row pitch lp
     const int ntiles = g.nb[0] * g.nb[1] * g.nb[2];
     const int lrx = g.lrho[0], lry = g.lrho[1], lrz = g.lrho[2];
     const int rzm = g.rho[2] - 1;
@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(kNT, 1) ngf_grad_kernel(const __grid_constant_
         const int gx = x0 - 2 + L, gy = y0 - 2 + w;
         const bool colin = gx >= 0 && gx < nx && gy >= 0 && gy < ny;
         const bool intxy = colin && gx >= 1 && gx <= nx - 2 && gy >= 1 && gy <= ny - 2;
-        const int col = colin ? gy * nx + gx : 0;
+        const int col = colin ? gy * nx + gx : 0, lcol = colin ? gy * g.lp + gx : 0;
         const int cxg = gx >> lrx, cyg = gy >> lry;
         const float fx = ((gx - (cxg << lrx)) + 0.5f) * g.irho[0];
         const float fy = ((gy - (cyg << lry)) + 0.5f) * g.irho[1];
@@ -201,10 +201,10 @@ __global__ void __launch_bounds__(kNT, 1) ngf_grad_kernel(const __grid_constant_
                         dw[1] = in[1] ? fmaf(f[2], dy1 - dy0, dy0) * ih1 * (float)st[1] : 0.f;
                         dw[2] = in[2] ? dz * ih2 * (float)st[2] : 0.f;
                         if (STORE && own_col && colin && pW >= z0 && pW < z0 + TZc) {
-                            const int v = pW * sxy + col;
+                            const long v = pW * lsxy + lcol;
                             a.st_dT[v] = dw[0];
-                            a.st_dT[N + v] = dw[1];
-                            a.st_dT[2 * N + v] = dw[2];
+                            a.st_dT[lN + v] = dw[1];
+                            a.st_dT[2 * lN + v] = dw[2];
                         }
                     }
                 }
@@ -243,10 +243,10 @@ __global__ void __launch_bounds__(kNT, 1) ngf_grad_kernel(const __grid_constant_
                         c0 = sc * q0 * i2h0; c1 = sc * q1 * i2h1; c2 = sc * q2 * i2h2;
                         if (STORE && own && colin && pC >= 0) {
                             const float inv = interior ? rsqrtf(ff * gg) * rgg : 0.f;
-                            const int v = pC * sxy + col;
+                            const long v = pC * lsxy + lcol;
                             a.st_a[v] = q0 * inv * i2h0;   // a = dr/dg, stored with the scale 1 / (2 h)
-                            a.st_a[N + v] = q1 * inv * i2h1;
-                            a.st_a[2 * N + v] = q2 * inv * i2h2;
+                            a.st_a[lN + v] = q1 * inv * i2h1;
+                            a.st_a[2 * lN + v] = q2 * inv * i2h2;
                         }
                     }
                 }

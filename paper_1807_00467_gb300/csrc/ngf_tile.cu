@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(32 * (TY + 4), TY == 8 ? 2 : 1) ngf_tile_kerne
 
     const int tid = threadIdx.x, L = tid & 31, w = tid >> 5;
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-    const long sxy = (long)nx * ny, N = sxy * nz;
+    const long sxy = (long)nx * ny;
     const int TXI = g.TXI;
     const int x0 = blockIdx.x * TXI, y0 = blockIdx.y * TY, z0 = blockIdx.z * g.TZ;
     const int TZc = min(g.TZ, nz - z0);
@@ -148,6 +148,8 @@ __global__ void __launch_bounds__(32 * (TY + 4), TY == 8 ? 2 : 1) ngf_tile_kerne
     const bool inA = L >= 2 && L <= TXI + 1 && w >= 2 && w <= TY + 1;
     const bool intxy = colin && gx >= 1 && gx <= nx - 2 && gy >= 1 && gy <= ny - 2;
     const long col = colin ? (long)gy * nx + gx : 0;
+    // the stored linearisation: row pitch lp
+    const long lsxy = (long)g.lp * ny, lN = lsxy * nz, lcol = colin ? (long)gy * g.lp + gx : 0;
     const int CX = g.C[0];
     const int cta = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
 
@@ -227,13 +229,13 @@ __global__ void __launch_bounds__(32 * (TY + 4), TY == 8 ? 2 : 1) ngf_tile_kerne
     if ((M::matvec || M::diag) && !tma) {
         const int p = z0 - M::HZ;
         if (colin && p >= 0 && p < nz) {
-            const long v = (long)p * sxy + col;
-            dnx[0] = __ldg(a.lin_dT + v); dnx[1] = __ldg(a.lin_dT + N + v); dnx[2] = __ldg(a.lin_dT + 2 * N + v);
-            if (M::diag) { anx[0] = __ldg(a.lin_a + v); anx[1] = __ldg(a.lin_a + N + v); anx[2] = __ldg(a.lin_a + 2 * N + v); }
+            const long v = (long)p * lsxy + lcol;
+            dnx[0] = __ldg(a.lin_dT + v); dnx[1] = __ldg(a.lin_dT + lN + v); dnx[2] = __ldg(a.lin_dT + 2 * lN + v);
+            if (M::diag) { anx[0] = __ldg(a.lin_a + v); anx[1] = __ldg(a.lin_a + lN + v); anx[2] = __ldg(a.lin_a + 2 * lN + v); }
         }
         if (M::matvec && inC && colin && p - 1 >= 0 && p - 1 < nz) {
-            const long v = (long)(p - 1) * sxy + col;
-            anx[0] = __ldg(a.lin_a + v); anx[1] = __ldg(a.lin_a + N + v); anx[2] = __ldg(a.lin_a + 2 * N + v);
+            const long v = (long)(p - 1) * lsxy + lcol;
+            anx[0] = __ldg(a.lin_a + v); anx[1] = __ldg(a.lin_a + lN + v); anx[2] = __ldg(a.lin_a + 2 * lN + v);
         }
     }
     __syncthreads();
@@ -332,14 +334,14 @@ __global__ void __launch_bounds__(32 * (TY + 4), TY == 8 ? 2 : 1) ngf_tile_kerne
             const int p = pW + 1;
             dnx[0] = dnx[1] = dnx[2] = 0.f;
             if (colin && p >= 0 && p < nz) {
-                const long v = (long)p * sxy + col;
-                dnx[0] = __ldg(a.lin_dT + v); dnx[1] = __ldg(a.lin_dT + N + v); dnx[2] = __ldg(a.lin_dT + 2 * N + v);
+                const long v = (long)p * lsxy + lcol;
+                dnx[0] = __ldg(a.lin_dT + v); dnx[1] = __ldg(a.lin_dT + lN + v); dnx[2] = __ldg(a.lin_dT + 2 * lN + v);
             }
             anx[0] = anx[1] = anx[2] = 0.f;
             const int pa = M::matvec ? pW : pW + 1;
             if ((M::diag || inC) && colin && pa >= 0 && pa < nz) {
-                const long v = (long)pa * sxy + col;
-                anx[0] = __ldg(a.lin_a + v); anx[1] = __ldg(a.lin_a + N + v); anx[2] = __ldg(a.lin_a + 2 * N + v);
+                const long v = (long)pa * lsxy + lcol;
+                anx[0] = __ldg(a.lin_a + v); anx[1] = __ldg(a.lin_a + lN + v); anx[2] = __ldg(a.lin_a + 2 * lN + v);
             }
         }
         if (colin && zW && !M::diag) {
@@ -385,10 +387,10 @@ __global__ void __launch_bounds__(32 * (TY + 4), TY == 8 ? 2 : 1) ngf_tile_kerne
                 dn[1] = ins[1] ? fmaf(f[2], dy1 - dy0, dy0) * g.invh[1] * (float)stp[1] : 0.f;
                 dn[2] = ins[2] ? dz * g.invh[2] * (float)stp[2] : 0.f;
                 if (M::store && inA && pW >= z0 && pW < z0 + TZc) {
-                    const long v = (long)pW * sxy + col;
+                    const long v = (long)pW * lsxy + lcol;
                     a.st_dT[v] = dn[0];
-                    a.st_dT[N + v] = dn[1];
-                    a.st_dT[2 * N + v] = dn[2];
+                    a.st_dT[lN + v] = dn[1];
+                    a.st_dT[2 * lN + v] = dn[2];
                 }
             }
         }
@@ -465,17 +467,17 @@ __global__ void __launch_bounds__(32 * (TY + 4), TY == 8 ? 2 : 1) ngf_tile_kerne
                         if (M::store && own) {
                             // a = dr/dg, stored with the central-difference scale 1 / (2 h) per axis
                             const float inv = rsqrtf(ff * gg) * rgg;
-                            const long v = (long)pC * sxy + col;
+                            const long v = (long)pC * lsxy + lcol;
                             a.st_a[v] = q0 * inv * g.inv2h[0];
-                            a.st_a[N + v] = q1 * inv * g.inv2h[1];
-                            a.st_a[2 * N + v] = q2 * inv * g.inv2h[2];
+                            a.st_a[lN + v] = q1 * inv * g.inv2h[1];
+                            a.st_a[2 * lN + v] = q2 * inv * g.inv2h[2];
                         }
                     }
                 } else if (M::store && own && colin) {
-                    const long v = (long)pC * sxy + col;
+                    const long v = (long)pC * lsxy + lcol;
                     a.st_a[v] = 0.f;
-                    a.st_a[N + v] = 0.f;
-                    a.st_a[2 * N + v] = 0.f;
+                    a.st_a[lN + v] = 0.f;
+                    a.st_a[2 * lN + v] = 0.f;
                 }
             }
             if (!M::adj) continue;
