@@ -32,9 +32,12 @@ constexpr int kS = 33;              // labels per axis
 constexpr int kL = kS * kS * kS;    // 35937 labels
 constexpr int kPlane = kS * kS;     // labels per z plane
 constexpr int kW = kS + 3;          // window points per axis: patch (4) + labels (33) - 1
-constexpr int kCvG = 2;             // z labels per cost-volume CTA
-constexpr int kCvT = 224;           // cost-volume threads (2 x 33 rows x 3 runs of 11 labels = 198 busy)
-constexpr int kRun = 11;            // labels per thread along x
+constexpr int kRun = 11, kDy = 3;   // labels per cost-volume thread along x and y
+constexpr int kCvG = 7;             // z labels per cost-volume CTA
+constexpr int kCvR = kS / kRun, kCvD = kS / kDy;   // runs along x, groups along y
+constexpr int kCvT = 256;           // cost-volume threads (3 runs x 7 z labels x 11 y groups = 231 busy)
+constexpr int kWp = kW + 1;         // window row pitch (odd: y groups start in different banks)
+constexpr int kWPlane = kW * kWp;
 constexpr int kCl = 8;              // CTAs per message (one thread-block cluster)
 constexpr int kBpT = 256;           // threads per message CTA
 
@@ -57,65 +60,95 @@ __global__ void features_kernel(int nx, int ny, int nz, const float *img, float 
 }
 
 // ------------------------------------------------------------ cost volume
-// CTA (keypoint k, z labels 2g, 2g + 1): the moving features at the window
-// points k + 2 w - 35 (w = 0..35 per axis) of the kCvG + 3 planes it needs are
-// staged in shared memory; thread (dz, dy, run) accumulates 11 labels along x,
-// reusing each loaded window row for 11 labels x 4 patch columns.
-__global__ void __launch_bounds__(kCvT) cost_volume_kernel(int nx, int ny, int nz, const float4 *__restrict__ ffix,
-                                                           const float4 *__restrict__ fmov, const int *__restrict__ kps,
-                                                           float *__restrict__ D) {
+// CTA (keypoint k, z labels 7 g .. 7 g + 6): the moving features at the window
+// points k + 2 w - 35 (w = 0..35 per axis) of the 10 planes it needs are staged
+// in shared memory (cp.async, the last three planes while the first patch plane
+// is worked on).  A thread accumulates 11 x 3 labels in x and y: a loaded window
+// row of 14 points serves up to 3 y labels x 11 x labels x 4 patch columns.
+// Bound by FP32 issue (5 FMA per label and patch point) once the rows are reused
+// like that: with one y label per thread and 2 z labels per CTA the
+// shared-memory reads bound it (2.68 ms for 3000 keypoints; 2.48 so, floor 1.3
+// at the FMA rate this part sustains; two y labels in two smaller CTAs per SM:
+// 2.80, rows loaded a step ahead: 2.51).  Rows are padded so that the 16-byte reads of eight
+// neighbouring threads (y groups, then z labels: 111 (12 dz + dy) points apart)
+// fall into different banks.
+__global__ void __launch_bounds__(kCvT, 1) cost_volume_kernel(int nx, int ny, int nz, const float4 *__restrict__ ffix,
+                                                              const float4 *__restrict__ fmov,
+                                                              const int *__restrict__ kps, float *__restrict__ D) {
     extern __shared__ float4 sm4[];
-    float4 *win = sm4;                          // [kCvG + 3][kW][kW]
-    float4 *pf = sm4 + (kCvG + 3) * kW * kW;    // [4][4][4] fixed patch
+    float4 *win = sm4;                              // [kCvG + 3][kW][kWp]
+    float4 *pf = sm4 + (kCvG + 3) * kWPlane;        // [4][4][4] fixed patch
     const int ng = (kS + kCvG - 1) / kCvG;
     const int k = blockIdx.x / ng, g = blockIdx.x - k * ng;
     const int kx = kps[3 * k], ky = kps[3 * k + 1], kz = kps[3 * k + 2];
     const int dz0 = g * kCvG;
     const int tid = threadIdx.x;
-    for (int i = tid; i < (kCvG + 3) * kW * kW; i += kCvT) {
-        const int pz = i / (kW * kW), r = i - pz * kW * kW, wy = r / kW, wx = r - wy * kW;
-        const int z = clampi(kz + 2 * (dz0 + pz) - 35, 0, nz - 1);
-        const int y = clampi(ky + 2 * wy - 35, 0, ny - 1), x = clampi(kx + 2 * wx - 35, 0, nx - 1);
-        win[i] = __ldg(fmov + ((long)z * ny + y) * nx + x);
-    }
+    // planes [p0, p1) of the window, one commit group
+    auto stage = [&](int p0, int p1) {
+        for (int i = p0 * kW * kW + tid; i < p1 * kW * kW; i += kCvT) {
+            const int pz = i / (kW * kW), r = i - pz * kW * kW, wy = r / kW, wx = r - wy * kW;
+            const int z = clampi(kz + 2 * (dz0 + pz) - 35, 0, nz - 1);
+            const int y = clampi(ky + 2 * wy - 35, 0, ny - 1), x = clampi(kx + 2 * wx - 35, 0, nx - 1);
+            const uint32_t dst = (uint32_t)__cvta_generic_to_shared(win + pz * kWPlane + wy * kWp + wx);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(fmov + ((long)z * ny + y) * nx + x)
+                         : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    stage(0, kCvG);
+    for (int p = kCvG; p < kCvG + 3; ++p) stage(p, p + 1);
     if (tid < 64) {
         const int px = tid & 3, py = (tid >> 2) & 3, pz = tid >> 4;
         const int z = clampi(kz + 2 * pz - 3, 0, nz - 1), y = clampi(ky + 2 * py - 3, 0, ny - 1);
         const int x = clampi(kx + 2 * px - 3, 0, nx - 1);
         pf[tid] = __ldg(ffix + ((long)z * ny + y) * nx + x);
     }
-    __syncthreads();
-    const int run = tid % 3, dy = (tid / 3) % kS, dzl = tid / (3 * kS);
-    const int dz = dz0 + dzl;
-    if (dzl >= kCvG || dz >= kS) return;
-    const int dx0 = run * kRun;
-    float acc[kRun];
+    const int run = tid / (kCvG * kCvD), rr = tid - run * (kCvG * kCvD), dzl = rr / kCvD, db = rr - dzl * kCvD;
+    const bool busy = run < kCvR && dz0 + dzl < kS;
+    float acc[kDy][kRun];
 #pragma unroll
-    for (int j = 0; j < kRun; ++j) acc[j] = 0.f;
+    for (int d = 0; d < kDy; ++d)
+#pragma unroll
+        for (int j = 0; j < kRun; ++j) acc[d][j] = 0.f;
 #pragma unroll 1
     for (int pz = 0; pz < 4; ++pz) {
-#pragma unroll 1
-        for (int py = 0; py < 4; ++py) {
-            const float4 *row = win + ((dzl + pz) * kW + (dy + py)) * kW + dx0;
+        // planes pz .. pz + kCvG - 1 have landed
+        if (pz == 0) asm volatile("cp.async.wait_group 3;" ::: "memory");
+        else if (pz == 1) asm volatile("cp.async.wait_group 2;" ::: "memory");
+        else if (pz == 2) asm volatile("cp.async.wait_group 1;" ::: "memory");
+        else asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        if (!busy) continue;
+        const float4 *rows = win + (dzl + pz) * kWPlane + kDy * db * kWp + run * kRun;
+        const float4 *f = pf + pz * 16;
+#pragma unroll
+        for (int wy = 0; wy < kDy + 3; ++wy) {
             float4 m[kRun + 3];
 #pragma unroll
-            for (int j = 0; j < kRun + 3; ++j) m[j] = row[j];
-            const float4 *f = pf + (pz * 4 + py) * 4;
+            for (int j = 0; j < kRun + 3; ++j) m[j] = rows[wy * kWp + j];
 #pragma unroll
-            for (int px = 0; px < 4; ++px) {
-                const float4 q = f[px];
+            for (int d = 0; d < kDy; ++d) {
+                const int py = wy - d;   // the patch row of label row kDy db + d on this window row
+                if (py < 0 || py > 3) continue;
 #pragma unroll
-                for (int j = 0; j < kRun; ++j) {
-                    const float4 a = m[j + px];
-                    const float r = fmaf(a.w, q.w, fmaf(a.z, q.z, fmaf(a.y, q.y, a.x * q.x)));
-                    acc[j] = fmaf(r, r, acc[j]);
+                for (int px = 0; px < 4; ++px) {
+                    const float4 q = f[py * 4 + px];
+#pragma unroll
+                    for (int j = 0; j < kRun; ++j) {
+                        const float4 a = m[j + px];
+                        const float r = fmaf(a.w, q.w, fmaf(a.z, q.z, fmaf(a.y, q.y, a.x * q.x)));
+                        acc[d][j] = fmaf(r, r, acc[d][j]);
+                    }
                 }
             }
         }
     }
-    float *out = D + (long)k * kL + ((long)dz * kS + dy) * kS + dx0;
+    if (!busy) return;
+    float *out = D + (long)k * kL + ((long)(dz0 + dzl) * kS + kDy * db) * kS + run * kRun;
 #pragma unroll
-    for (int j = 0; j < kRun; ++j) out[j] = fmaf(-acc[j], 1.f / 64.f, 1.f);
+    for (int d = 0; d < kDy; ++d)
+#pragma unroll
+        for (int j = 0; j < kRun; ++j) out[d * kS + j] = fmaf(-acc[d][j], 1.f / 64.f, 1.f);
 }
 
 // ------------------------------------------------------------ MST (Boruvka)
@@ -779,7 +812,7 @@ cudaError_t run_features(const int *n, const float *img, float eta, float4 *feat
 cudaError_t run_cost(const int *n, const float4 *ffix, const float4 *fmov, int nk, const int *kps, float *D,
                      cudaStream_t st) {
     if (nk <= 0) return cudaSuccess;
-    const size_t smem = sizeof(float4) * ((kCvG + 3) * kW * kW + 64);
+    const size_t smem = sizeof(float4) * ((kCvG + 3) * kWPlane + 64);
     cudaError_t e = allow_max_dynamic_smem(cost_volume_kernel);
     if (e != cudaSuccess) return e;
     const int ng = (kS + kCvG - 1) / kCvG;
