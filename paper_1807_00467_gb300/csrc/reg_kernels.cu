@@ -149,53 +149,66 @@ __global__ void kp_kernel(const KpArgs a) {
     }
 }
 
-// node sums: thread (r, o) for the first sorted keypoint r of a cell and a
+// node sums: warp (r, o) for the first sorted keypoint r of a cell and a
 // corner o of that cell owns node n = cell + o unless a cell n - o' with o' < o
 // holds keypoints; the owner adds, in the order (o'', i), the contributions
 // of every keypoint in the cells n - o'' to out[n] (diag: 2 delta w^2 to all
-// three components; else 2 scale w src_i)
+// three components; else 2 scale w src_i).  The lanes form the terms of 32
+// keypoints at once and add them in order through shuffles: one thread per node
+// followed a chain of dependent loads, two per keypoint (48 us for 3000
+// keypoints along 30 vessels in a 65 x 65 x 33 grid, 10 us so).
 template <bool DIAG>
-__global__ void kp_gather_kernel(const KpArgs a, double two_delta, float *out) {
+__global__ void __launch_bounds__(256) kp_gather_kernel(const KpArgs a, double two_delta, float *out) {
     if (a.skip && *a.skip) return;   // uniform: every block reads the same flag
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int r = t >> 3, o = t & 7;
+    constexpr unsigned FULL = 0xffffffffu;
+    const unsigned t = blockIdx.x * 8u + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31, r = (int)(t >> 3), o = (int)(t & 7u);
     if (r >= a.nk) return;
     const int *sb = a.ix.sb;
-    if (r > 0 && sb[r] == sb[r - 1]) return;
+    const int b = sb[r];
+    if (r > 0 && b == sb[r - 1]) return;
     const int mx = a.m[0], my = a.m[1];
     const long mxy = (long)mx * my, M = mxy * a.m[2];
-    const int b = sb[r];
     const int cz = b / (int)mxy, cy = (b - cz * (int)mxy) / mx, cx = b - cz * (int)mxy - cy * mx;
     const int nx = cx + (o & 1), ny = cy + ((o >> 1) & 1), nz = cz + (o >> 2);
-    // the cell n - o' of corner offset o', or -1 outside the cell grid
-    auto cell_at = [&](int op) {
-        const int x = nx - (op & 1), y = ny - ((op >> 1) & 1), z = nz - (op >> 2);
-        if (x < 0 || y < 0 || z < 0 || x > mx - 2 || y > my - 2 || z > a.m[2] - 2) return -1;
-        return (z * my + y) * mx + x;
-    };
-    for (int op = 0; op < o; ++op) {
-        const int c = cell_at(op);
-        if (c >= 0 && a.ix.soc[c] >= 0) return;
+    // lane op < 8: the first sorted keypoint of cell n - op, -1 if it holds none or lies outside the cell grid
+    int first = -1, cell = -1;
+    if (lane < 8) {
+        const int x = nx - (lane & 1), y = ny - ((lane >> 1) & 1), z = nz - (lane >> 2);
+        if (!(x < 0 || y < 0 || z < 0 || x > mx - 2 || y > my - 2 || z > a.m[2] - 2)) {
+            cell = (z * my + y) * mx + x;
+            first = a.ix.soc[cell];
+        }
     }
+    if (__any_sync(FULL, lane < o && first >= 0)) return;   // a lower corner's warp owns the node
     float acc[3] = {0.f, 0.f, 0.f};
     for (int op = 0; op < 8; ++op) {
-        const int c = cell_at(op);
-        const int s = c >= 0 ? a.ix.soc[c] : -1;
+        const int s = __shfl_sync(FULL, first, op), c = __shfl_sync(FULL, cell, op);
         if (s < 0) continue;
-        for (int q = s; q < a.nk && sb[q] == c; ++q) {
-            const int i = a.ix.perm[q];
-            const float f[3] = {a.ix.frac[3 * i], a.ix.frac[3 * i + 1], a.ix.frac[3 * i + 2]};
-            const float w = kp_weight(op, f);
-            if (DIAG) {
-                const float add = (float)(two_delta * w * w);
-                acc[0] += add; acc[1] += add; acc[2] += add;
-            } else {
-                for (int k = 0; k < 3; ++k) acc[k] += 2.f * a.scale * w * a.ix.src[3 * i + k];
+        for (int q0 = s;; q0 += 32) {
+            const bool in = q0 + lane < a.nk && sb[q0 + lane] == c;   // a prefix of the lanes: the cells are sorted
+            float w = 0.f, v[3] = {0.f, 0.f, 0.f};
+            if (in) {
+                const int i = a.ix.perm[q0 + lane];
+                const float f[3] = {a.ix.frac[3 * i], a.ix.frac[3 * i + 1], a.ix.frac[3 * i + 2]};
+                w = kp_weight(op, f);
+                if (DIAG) {
+                    w = (float)(two_delta * w * w);
+                } else {
+                    w = 2.f * a.scale * w;
+                    for (int k = 0; k < 3; ++k) v[k] = a.ix.src[3 * i + k];
+                }
             }
+            const int n = __popc(__ballot_sync(FULL, in));
+            for (int j = 0; j < n; ++j) {
+                const float wj = __shfl_sync(FULL, w, j);
+                for (int k = 0; k < 3; ++k) acc[k] = DIAG ? acc[k] + wj : fmaf(wj, __shfl_sync(FULL, v[k], j), acc[k]);
+            }
+            if (n < 32) break;
         }
     }
     const long n = (long)nz * mxy + (long)ny * mx + nx;
-    for (int k = 0; k < 3; ++k) out[k * M + n] += acc[k];
+    if (lane < 3) out[lane * M + n] += lane == 0 ? acc[0] : lane == 1 ? acc[1] : acc[2];
 }
 
 cudaError_t launch_kp(const KpArgs &a, cudaStream_t st) {
@@ -205,7 +218,7 @@ cudaError_t launch_kp(const KpArgs &a, cudaStream_t st) {
 
 cudaError_t launch_kp_gather(const KpArgs &a, cudaStream_t st) {
     if (!a.out || a.nk <= 0) return cudaSuccess;
-    kp_gather_kernel<false><<<(8 * a.nk + 255) / 256, 256, 0, st>>>(a, 0.0, a.out);
+    kp_gather_kernel<false><<<a.nk, 256, 0, st>>>(a, 0.0, a.out);
     return cudaGetLastError();
 }
 
@@ -316,7 +329,7 @@ cudaError_t launch_jacobi_diag(int alpha_on, const int *m, const float *ig2, dou
 
 cudaError_t launch_kp_diag(const KpArgs &a, double two_delta, float *diag, cudaStream_t st) {
     if (a.nk <= 0) return cudaSuccess;
-    kp_gather_kernel<true><<<(8 * a.nk + 255) / 256, 256, 0, st>>>(a, two_delta, diag);
+    kp_gather_kernel<true><<<a.nk, 256, 0, st>>>(a, two_delta, diag);
     return cudaGetLastError();
 }
 
