@@ -163,10 +163,15 @@ static long lin_pitch(int n0) { return (n0 + 3) & ~3; }
 // chain while most SMs idle (64x64x48: 24 CTAs of 32 planes on 152 SMs).  The
 // chunk is the number of whole cells that minimises waves x (planes + halo +
 // fixed cost of a chunk, about 4 planes' time); large volumes keep 32 planes.
+// The geometry fixes a result's bits, so it cannot depend on what else runs:
+// where a batch's pairs fill the chip together, halos and fixed costs are work
+// that nothing pays back, so chunks that add more than half to the planes of
+// the 32-plane ones are not taken (24 pairs of 64x64x48, 5 iterations of 20 PCG
+// steps: 27.5 ms in 32-plane chunks, 30.1 with this limit, 36 without it).
 // 152: the SM count of the part, a constant so that a workspace sized on one
 // machine fits the context made on another.
-// 64x64x48 (chunk of 4): ngf_gradient 61 -> 31 us, a Gauss-Newton iteration of
-// 30 PCG steps 2.27 -> 1.84 ms; 182x150x94: Hessian-vector product 355 -> 340 us.
+// 64x64x48 (chunk of 8): ngf_gradient 64 -> 37 us (a chunk of 4: 33 us);
+// 182x150x94: Hessian-vector product 355 -> 340 us.
 static void tile_geom(const rg_image_geom *img, const rg_grid_geom *grid, TileGeom &t, int TY = 16, bool fill = true) {
     for (int a = 0; a < 3; ++a) {
         t.n[a] = img->n[a];
@@ -190,7 +195,9 @@ static void tile_geom(const rg_image_geom *img, const rg_grid_geom *grid, TileGe
         const long nxy = (long)((t.n[0] + t.TXI - 1) / t.TXI) * ((t.n[1] + t.TY - 1) / t.TY);
         long best = LONG_MAX;
         int tz = t.TZ;
+        auto planes = [&](int c) { return t.n[2] + 8L * ((t.n[2] + c - 1) / c); };   // marched per x-y tile, halos and fixed cost
         for (int c = t.TZ; c >= t.rho[2]; c -= t.rho[2]) {   // ties: the larger chunk (fewer boxes)
+            if (2 * planes(c) > 3 * planes(t.TZ)) break;
             const long cost = (nxy * ((t.n[2] + c - 1) / c) + 151) / 152 * (c + 8);
             if (cost < best) {
                 best = cost;
@@ -219,7 +226,10 @@ static void tile_geom(const rg_image_geom *img, const rg_grid_geom *grid, TileGe
 // (TXI = 60 less a remainder so that it is whole cells), every z plane or (fill)
 // chunks of them; node boxes [3][nodes][C1 + 1][C0 + 1] per column and chunk.
 // Chunks, by the rule of tile_geom, where the columns leave SMs idle (one CTA
-// per SM): multiples of 4 planes, so that CTAs can walk several of them.
+// per SM): multiples of 4 planes, so that CTAs can walk several of them, and no
+// more than 1.35 x the planes of whole columns, again for batches (a step of 20
+// PCG iterations at 96x96x48: 2.12 ms whole, 1.46 so, 1.29 without the limit; six
+// such pairs at once, 5 iterations: 14.0, 11.5 and 13.7 ms; 24: 33, 39 and 46).
 static void col_geom(const rg_image_geom *img, const rg_grid_geom *grid, ColGeom &c, bool fill) {
     for (int a = 0; a < 3; ++a) {
         c.n[a] = img->n[a];
@@ -243,6 +253,7 @@ static void col_geom(const rg_image_geom *img, const rg_grid_geom *grid, ColGeom
         const long nxy = (long)c.nb[0] * c.nb[1];
         long best = (nxy + 151) / 152 * (c.n[2] + 8);
         for (int z = c.n[2] / q * q; z >= q; z -= q) {
+            if (100 * (c.n[2] + 8L * ((c.n[2] + z - 1) / z)) > 135 * (c.n[2] + 8L)) break;
             const long cost = (nxy * ((c.n[2] + z - 1) / z) + 151) / 152 * (z + 8);
             if (cost < best) {
                 best = cost;
@@ -999,7 +1010,7 @@ static int pcg(rg_ctx *c, const float *g, float *p, int iters, double *stats) {
 
 // Whether the persistent batched PCG (pcg_batch.cu) can take this context's
 // PCG steps: the column GN-product kernel covers its volume and H has no
-// keypoint term (its node sums use atomics outside the node pass).
+// keypoint term (its node sums are a pass of their own, outside the node pass).
 static bool batch_pcg_ok(const rg_ctx *c) { return !c->general_only && c->nk <= 0 && pcg_batch_supported(c->cp); }
 
 // The operands of one PCG step of the context (the GN product H d into q as
