@@ -121,8 +121,11 @@ typedef struct {
 #define RG_SCHED_AUTOTUNE 4
 /* rg_schedule.flags, register_pyramid_batch only: the PCG steps of every pair
  * whose level the column GN-product kernel covers (volumes at least 68 voxels
- * wide and 20 high, whole grid cells per axis) run in one persistent
- * cooperative kernel per level iteration (up to 24 pairs per launch), whose
+ * wide and 20 high, whole grid cells per axis, two or more voxels per cell
+ * along x and y) run in one persistent cooperative kernel per level iteration
+ * (up to 24 pairs per launch), on levels where these pairs together have at
+ * most two 60 x 16 voxel columns per SM (in z chunks on small volumes; larger
+ * levels keep their launches, which are faster there).  The kernel's
  * CTAs take (pair, tile) items from a work counter, each waiting (bounded;
  * RG_ETIMEOUT when a wait runs out) for the previous phase of its own pair.
  * Same bits per pair as without the flag.  RG_SCHED_HOOK_BARRIER is a test
@@ -387,7 +390,8 @@ int kp_mst(int32_t nk, const int32_t *kps, const float *intensity, double sigma_
  * number of levels; exact min-marginals do not depend on the root); messages
  * are squared-distance min-convolutions over
  * the label grid (axis by axis).  marginals: float [nk][35937].
- * Synchronises the stream once (tree levels). */
+ * Synchronises the stream once, at its end; RG_ETIMEOUT if a bounded wait for
+ * another vertex's message runs out. */
 int kp_bp_marginals(int32_t nk, const float *D, const int32_t *kps, const float *intensity, const int32_t *edges,
                     double sigma_i, double alpha, float *marginals, void *scratch, size_t scratch_bytes,
                     void *cuda_stream);

@@ -1013,6 +1013,12 @@ static int pcg(rg_ctx *c, const float *g, float *p, int iters, double *stats) {
 // keypoint term (its node sums are a pass of their own, outside the node pass).
 static bool batch_pcg_ok(const rg_ctx *c) { return !c->general_only && c->nk <= 0 && pcg_batch_supported(c->cp); }
 
+// The persistent kernel takes a level whose covered pairs together have at most
+// two columns per SM.  Beyond that each phase fills the chip in launches of its
+// own, which keep their own shapes (24 pairs of 320x320x96, 5 iterations of 20
+// PCG steps: 543 ms persistent, 314 ms as launches; 2880 columns).
+static long batch_columns(const rg_ctx *c) { return (long)c->cp.nb[0] * c->cp.nb[1] * c->cp.nbz; }
+
 // The operands of one PCG step of the context (the GN product H d into q as
 // matvec forms it, the vectors of pcg), with s the PCG iterate.
 static void batch_pair(rg_ctx *c, float *s, BatchPair &b) {
@@ -1681,10 +1687,14 @@ extern "C" int register_pyramid_batch(int32_t npairs, const rg_image_geom *img, 
         // pairs whose PCG steps the persistent batched kernel takes (the rest
         // run their whole iteration in their branch)
         std::vector<int> pers;
+        long ncols = 0;
+        for (int p = 0; p < npairs; ++p)
+            if (!halted[p] && batch_pcg_ok(ps[p].cl)) ncols += batch_columns(ps[p].cl);
+        const bool pers_level = persistent && ncols <= 2L * device_sm_count();
         for (int p = 0; p < npairs && cst == RG_OK; ++p) {
             if (halted[p]) continue;
             rg_ctx *cl = ps[p].cl;
-            const bool inp = persistent && batch_pcg_ok(cl);
+            const bool inp = pers_level && batch_pcg_ok(cl);
             if (inp) pers.push_back(p);
             if (cudaStreamWaitEvent(cl->gst, fork, 0) != cudaSuccess) {
                 cst = RG_ECUDA;

@@ -3,12 +3,12 @@
 // one cooperative launch (the Gauss-Newton solve of Sec. II-D3 on the
 // objective of Eq. (11)).
 //
-// One CTA per SM (640 threads, the GN-product kernel's shape) runs every PCG
+// One CTA per SM (320 threads, the GN-product kernel's shape) runs every PCG
 // step k of every volume as five phases:
 //   A  H d pieces: the NGF GN product of every column (gn_product_body), the
-//      VCC product of every cell block (vcc_cell_body, five 128-thread blocks
-//      per item) and the curvature L d of every node tile (curv_body, two
-//      256-thread blocks per item);
+//      VCC product of every cell block (vcc_cell_body, five 64-thread blocks
+//      at once, two cells per thread) and the curvature L d of every node tile (curv_body, one
+//      256-thread block at once);
 //   B  node pass: q = H d and the partials of d . q (node_body);
 //   C  step:   alpha, r' = r - alpha q, Gram-Schmidt coefficient partials;
 //   D  reorth: r_{k+1} = r' - sum_j c_j r_j and the partials of r . z;
