@@ -656,12 +656,17 @@ static int run_tile(rg_ctx *c, int mode, const float *field) {
         return RG_OK;
     }
     c->nD = c->nA;
-    // the column-marching passes: the objective wherever it applies (its planes
-    // are dealt evenly to the SMs), the gradient and linearisation where the
-    // volume has at least one column per SM (narrower volumes keep the z-chunked
-    // tile pass, whose tiles fill the GPU)
+    // the column-marching passes: the objective, whose planes are dealt evenly to
+    // the SMs, with at least 16 planes per SM (below that the two halo planes and
+    // the start of a piece outweigh what its columns save: 24 pairs of 80x64x32 in
+    // one batch 25.8 ms, 23.3 by the tile pass; a step at 96x96x48 alone 1.46 and
+    // 1.45 ms), the gradient and linearisation where the volume has at least one
+    // column per SM (narrower volumes keep the z-chunked tile pass, whose tiles
+    // fill the GPU)
     const bool colpass = mode != MODE_MATVEC && mode != MODE_DIAG && !c->general_only && c->pass_sel != 2;
-    const bool gobj = colpass && mode == MODE_OBJ && ngf_gobj_supported(c->cg);
+    const long obj_planes = (c->cg.n[0] + 61) / 62 * (long)((c->cg.n[1] + 17) / 18) * c->cg.n[2];   // 62 x 18 columns
+    const bool gobj = colpass && mode == MODE_OBJ && ngf_gobj_supported(c->cg) &&
+                      (c->pass_sel == 1 || obj_planes >= 16L * device_sm_count());
     const bool gcol = colpass && mode != MODE_OBJ && ngf_gcol_supported(c->cg) &&
                       (c->pass_sel == 1 || c->cg.nb[0] * c->cg.nb[1] >= device_sm_count());
     if (gobj || gcol) {

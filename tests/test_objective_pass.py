@@ -26,14 +26,16 @@ def test_objective_against_oracle_and_tile_pass(n, m, half):
     ph = small_phantom(n, h, seed=41)
     u = phantom.motion_on_grid(ph, m, scale=0.6)
     ctx = gpu_context(ph, m, half=half)
+    ctx.debug_hook(RG_HOOK_PASS, 1)
     J = ctx.ngf_objective(to_dev(u))
     assert rel(J[0], oracle_problem(ph, m, half=half).objective(u)[0][0]) <= 1e-6
     ctx.debug_hook(RG_HOOK_PASS, 2)
     assert rel(J[0], ctx.ngf_objective(to_dev(u))[0]) <= 1e-7
-    ctx.debug_hook(RG_HOOK_PASS, 0)
+    ctx.debug_hook(RG_HOOK_PASS, 1)
     far = to_dev(u) + 1000.0          # every sample beyond the volume: all clamped
     a = ctx.ngf_objective(far)
     ctx.debug_hook(RG_HOOK_PASS, 2)
     assert rel(a[0], ctx.ngf_objective(far)[0]) <= 1e-7
     same = gpu_context(phantom.Phantom(R=ph.R, T=ph.R, n=ph.n, h=ph.h, amps=ph.amps, centres=ph.centres), m, half=half)
+    same.debug_hook(RG_HOOK_PASS, 1)
     assert float(same.ngf_objective(to_dev(u) * 0.0)[0]) == 0.0
