@@ -192,11 +192,11 @@ __global__ void __launch_bounds__(kNT, 1) pcg_batch_kernel(const __grid_constant
             if (r < A.colOff[np]) {
                 gn_column(P, smem, bars, r - A.colOff[p], pbits);
             } else if (r < A.vccOff[np]) {
-                const int v = tid / kVccT;
+                const int v = tid / kVccT, b0 = (r - A.vccOff[p]) * kVccPer;
                 const int *nb = P.b.vcc.nb;
-                for (int bid = (r - A.vccOff[p]) * kVccPer + v, e = min(bid - v + kVccPer, P.nvcc); bid < e;
-                     bid += kVccRun) {
+                for (int bid = b0 + v, e = min(b0 + kVccPer, P.nvcc); bid < e; bid += kVccRun) {
                     const VBlock b = warp_block(tid % kVccT, bid, nb[0], nb[1], nb[2], 1 + v, kVccT);
+                    if (bid != b0 + v) b.sync();   // the last block's box has been read out of the shared scratch
                     vcck::vcc_cell_body<1, float2>(P.b.vcc, b, reinterpret_cast<vcck::VccSmem<float2> *>(smem)[v]);
                 }
             } else {

@@ -153,7 +153,9 @@ struct VccSmem {
 // VM = 0: gradient of sum psi(d) (+ energy, folds, min / max d);
 // VM = 1: GN product along v; VM = 2: diagonal of the GN matrix.
 // F = float: a block of NC threads, one cell each; F = float2: NC / 2 threads,
-// thread t the cells t and t + NC / 2.
+// thread t the cells t and t + NC / 2.  A caller that runs another block on the
+// same scratch synchronises the threads first: the body ends by reading its box
+// out of it, and begins by clearing the box, each by a mapping of its own.
 template <int VM, typename F>
 __device__ __forceinline__ void vcc_cell_body(const VccArgs &a, const VBlock &vb, VccSmem<F> &sm) {
     constexpr bool GN = VM == 1, DG = VM == 2;
