@@ -662,8 +662,11 @@ static int run_tile(rg_ctx *c, int mode, const float *field) {
     // one batch 25.8 ms, 23.3 by the tile pass; a step at 96x96x48 alone 1.46 and
     // 1.45 ms), the gradient and linearisation where the volume has at least one
     // column per SM (narrower volumes keep the z-chunked tile pass, whose tiles
-    // fill the GPU)
-    const bool colpass = mode != MODE_MATVEC && mode != MODE_DIAG && !c->general_only && c->pass_sel != 2;
+    // fill the GPU).  Both load R's voxels in pairs, so an image that starts on an
+    // odd element (a view into a larger buffer) takes the tile pass, whose loads
+    // are single voxels; R's rows keep the pairs aligned (even widths only).
+    const bool r_pairs = ((uintptr_t)c->R & (c->dtype == RG_F32 ? 7 : 3)) == 0;
+    const bool colpass = mode != MODE_MATVEC && mode != MODE_DIAG && !c->general_only && c->pass_sel != 2 && r_pairs;
     const long obj_planes = (c->cg.n[0] + 61) / 62 * (long)((c->cg.n[1] + 17) / 18) * c->cg.n[2];   // 62 x 18 columns
     const bool gobj = colpass && mode == MODE_OBJ && ngf_gobj_supported(c->cg) &&
                       (c->pass_sel == 1 || obj_planes >= 16L * device_sm_count());
