@@ -161,8 +161,8 @@ cudaError_t launch_pcg_fused(const PcgArgs &a, const float *q, int napart, float
     int nb;
     const Part P = make_part(a.n, &nb);
     auto kernel = pcg_fused_kernel<1>;   // at most kFuseMax blocks: one quad per thread
-    static const cudaError_t big =
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    // the attribute belongs to the current device, so it is set for every launch
+    const cudaError_t big = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (big != cudaSuccess) return big;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nb);
