@@ -485,20 +485,30 @@ __device__ __forceinline__ float min3(float a, float b, float c) {
     return r;
 }
 
+// the larger, NaN when either is
+__device__ __forceinline__ float max_nan(float a, float b) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+
 // One 33-point line of the min-convolution: out[j] = min_i v[i] + lam (2 (i - j))^2
 // (one rounding per candidate), by distance d = |i - j|, both candidates of an output in one three-input
 // minimum.  Every candidate at distance d or more is at least min v + cost(d)
-// (rounding is monotone), so the warp stops at the first d whose bound reaches
-// its lines' largest output: the same values as all 33 candidates, a few
-// distances in place of 32 for most lines.  Called by whole warps.
+// (rounding is monotone, lam >= 0), so the warp stops at the first d whose bound
+// reaches its lines' largest output: the same values as all 33 candidates, a few
+// distances in place of 32 for most lines.  A NaN output makes the largest one
+// NaN, which no bound reaches (any candidate that is a number replaces it), and
+// a negative lam leaves no bound.  Called by whole warps.
 __device__ __forceinline__ void min_conv_line(float (&v)[kS], float lam) {
     float o[kS], lo = v[0], hi = v[0];
 #pragma unroll
     for (int j = 0; j < kS; ++j) {
         o[j] = v[j];   // cost(0) = 0
         lo = fminf(lo, v[j]);
-        hi = fmaxf(hi, v[j]);
+        hi = max_nan(hi, v[j]);
     }
+    if (lam < 0.f) lo = -__int_as_float(0x7f800000);
 #pragma unroll
     for (int d = 1; d < kS; ++d) {
         const float dd = (float)(4 * d * d);
@@ -513,7 +523,7 @@ __device__ __forceinline__ void min_conv_line(float (&v)[kS], float lam) {
         if (d == 1 || d == 2 || d == 4 || d == 8 || d == 16) {   // a tighter bound for the next distances
             hi = o[0];
 #pragma unroll
-            for (int j = 1; j < kS; ++j) hi = fmaxf(hi, o[j]);
+            for (int j = 1; j < kS; ++j) hi = max_nan(hi, o[j]);
         }
     }
 #pragma unroll
