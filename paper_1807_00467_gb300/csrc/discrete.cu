@@ -174,10 +174,10 @@ __global__ void mst_init_kernel(int n, int *comp, int *hook, unsigned long long 
 }
 
 // per vertex (one warp): the lightest edge to another component, then the
-// minimum per component.  An edge weighs at least its length, so a vertex
-// farther than the lightest weight found so far (shared across the warp every
-// 8 candidates) is passed over before its square root and division: the
-// rounds were bound by those (9 M edges a round, 45 us -> 26 us on average at
+// minimum per component.  An edge weighs at least its length (sig > 0; else no
+// vertex is passed over), so a vertex farther than the lightest weight found so
+// far (shared across the warp every 8 candidates) is passed over before its
+// square root and division: the rounds were bound by those (9 M edges a round, 45 us -> 26 us on average at
 // 3000 keypoints).  Once the tree is complete the remaining rounds end at once.
 __global__ void mst_min_edge_kernel(int n, const int *kps, const float *inten, float sig, const int *comp,
                                     unsigned long long *best, const int *nedges) {
@@ -200,7 +200,7 @@ __global__ void mst_min_edge_kernel(int n, const int *kps, const float *inten, f
         // the rounding of the square, the root and the sum stays within the factor 1 + 1e-6
         float w = b == ~0ull ? __int_as_float(0x7f800000) : __uint_as_float((unsigned)(b >> 32));
         for (int o = 16; o > 0; o >>= 1) w = fminf(w, __shfl_xor_sync(0xffffffffu, w, o));
-        far2 = w * w * 1.000001f;
+        if (sig > 0.f) far2 = w * w * 1.000001f;
     }
     for (int o = 16; o > 0; o >>= 1) {
         const unsigned long long t = __shfl_xor_sync(0xffffffffu, b, o);
