@@ -26,7 +26,9 @@
 // a fold is read from the least bound.  On large grids a thread holds two
 // cells, one per half of the packed f32x2 registers (TZ / 2 planes apart, their
 // nodes staged side by side), every operation serving both.  Gradient 137 ->
-// 81 us, GN product 107 -> 98 us at 129 x 129 x 65.  The one-cell form (F =
+// 87 us, GN product 107 -> 98 us at 129 x 129 x 65 (81 us with the energies of
+// four bounds added plainly before the compensated sum: up to 1.4 units in the
+// last place of a cell's energy instead of one).  The one-cell form (F =
 // float: small grids, and the persistent kernel, whose block leaves fewer
 // registers) runs the same operations, each rounded by an explicit intrinsic,
 // so both give the same bits.
@@ -316,7 +318,6 @@ __device__ __forceinline__ void vcc_cell_body(const VccArgs &a, const VBlock &vb
                         axpy(w, E1[aa], W);
                     }
                 } else {
-                    F ps = zero;
 #pragma unroll
                     for (int aa = 0; aa < 4; ++aa) {
                         const F d = dot(E1[aa], X), one = bc_<F>(1.f);
@@ -327,14 +328,13 @@ __device__ __forceinline__ void vcc_cell_body(const VccArgs &a, const VBlock &vb
                         const F r0 = lanes(rcp_pos, d);
                         const F rd = fma_(r0, fma_(d, neg_(r0), one), r0);
                         const F dm = sub_(d, one), q = mul_(dm, rd);
-                        ps = fma_(dm, q, ps);
+                        const F y = fma_(dm, q, neg_(en_c)), t = add_(en, y);   // psi(d)
+                        en_c = sub_(sub_(t, en), y);
+                        en = t;
                         const F w = mul_(q, mul_(add_(d, one), rd));
                         axpy(w, X, G1[aa]);
                         axpy(w, E1[aa], W);
                     }
-                    const F y = sub_(ps, en_c), t = add_(en, y);
-                    en_c = sub_(sub_(t, en), y);
-                    en = t;
                 }
                 const Vec<F> nW = neg_(W);
                 G2 = cross_add_r(E3[c], W, nW, G2);
