@@ -21,9 +21,8 @@
 // (60 us for 129 x 129 x 65 nodes at the ~97 three-operand FMA a clock and SM
 // that this part sustains).  The instructions around them are kept few: the
 // y-edges are taken one at a time in a rolled loop (their gradients parked in
-// shared memory), cells add to the box's nodes in place, one corner at a time
-// over the block, instead of through per-cell slots and an indexed gather, and
-// a fold is read from the least bound.  On large grids a thread holds two
+// shared memory), and cells add to the box's nodes in place, one corner at a time
+// over the block, instead of through per-cell slots and an indexed gather.  On large grids a thread holds two
 // cells, one per half of the packed f32x2 registers (TZ / 2 planes apart, their
 // nodes staged side by side), every operation serving both.  Gradient 137 ->
 // 87 us, GN product 107 -> 98 us at 129 x 129 x 65 (81 us with the energies of
@@ -116,18 +115,25 @@ __device__ __forceinline__ Vec<F> scaled(const Vec<F> &a, float s) {
     const F f = bc_<F>(s);
     return {mul_(a.x, f), mul_(a.y, f), mul_(a.z, f)};
 }
-// 1 / d where d > 0, else 0 (a fold has weight 0)
-__device__ __forceinline__ float rcp_pos(float d) {
+__device__ __forceinline__ float rcp_approx(float d) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
-    return d > 0.f ? r : 0.f;
-}
-
-// the smaller, NaN when either is (a NaN bound counts as a fold)
-__device__ __forceinline__ float min_nan(float a, float b) {
-    float r;
-    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
     return r;
+}
+// w where d > 0, else 0: a fold has weight 0, whatever its other factors are
+__device__ __forceinline__ float if_pos(float d, float w) { return d > 0.f ? w : 0.f; }
+
+// d, or 1 where d is not positive (or NaN): psi(1) = psi'(1) = 0, and the cell has a fold
+__device__ __forceinline__ float unfold(float d, bool (&fold)[1]) {
+    const bool pos = d > 0.f;
+    fold[0] |= !pos;
+    return pos ? d : 1.f;
+}
+__device__ __forceinline__ float2 unfold(float2 d, bool (&fold)[2]) {
+    const bool p0 = d.x > 0.f, p1 = d.y > 0.f;
+    fold[0] |= !p0;
+    fold[1] |= !p1;
+    return make_float2(p0 ? d.x : 1.f, p1 ? d.y : 1.f);
 }
 
 // corner offset (ox + 2 oy + 4 oz) of edge e = p + 2 q of axis `ax` at end `hi`;
@@ -244,7 +250,8 @@ __device__ __forceinline__ void vcc_cell_body(const VccArgs &a, const VBlock &vb
         }
     }
     F en = zero, en_c = zero;                       // Kahan sum of psi(d)
-    F dmn = bc_<F>(3.4e38f), dmx = bc_<F>(-3.4e38f);
+    F dmn = bc_<F>(3.4e38f), dmx = bc_<F>(-3.4e38f);   // of the bounds that are numbers
+    bool fold[CPT] = {};
     if constexpr (DG) {
         F out[8][3];
 #pragma unroll
@@ -257,7 +264,7 @@ __device__ __forceinline__ void vcc_cell_body(const VccArgs &a, const VBlock &vb
                 const Vec<F> X = cross(E2, nE2, E3[c]), gx = scaled(X, ig0), nE3 = neg_(E3[c]);
 #pragma unroll
                 for (int aa = 0; aa < 4; ++aa) {
-                    const F rd = lanes(rcp_pos, dot(E1[aa], X));
+                    const F d = dot(E1[aa], X), rd = lanes(if_pos, d, lanes(rcp_approx, d));
                     const F w = mul_(mul_(rd, rd), rd);   // psi''(d) / 2
                     const Vec<F> nE1 = neg_(E1[aa]);
                     const Vec<F> gy = scaled(cross(E3[c], nE3, E1[aa]), ig1), gz = scaled(cross(E1[aa], nE1, E2), ig2);
@@ -311,21 +318,20 @@ __device__ __forceinline__ void vcc_cell_body(const VccArgs &a, const VBlock &vb
                     const Vec<F> Y = cross_add(D2, nD2, E3[c], cross(E2, nE2, D3[c]));
 #pragma unroll
                     for (int aa = 0; aa < 4; ++aa) {
-                        const F rd = lanes(rcp_pos, dot(E1[aa], X));
+                        const F d = dot(E1[aa], X), rd = lanes(rcp_approx, d);
                         const F dd = dot_add(E1[aa], Y, dot(D1[aa], X));   // grad d . v
-                        const F w = mul_(mul_(rd, rd), mul_(rd, dd));     // psi''(d) (grad d . v) / 2
+                        const F w = lanes(if_pos, d, mul_(mul_(rd, rd), mul_(rd, dd)));   // psi''(d) (grad d . v) / 2
                         axpy(w, X, G1[aa]);
                         axpy(w, E1[aa], W);
                     }
                 } else {
 #pragma unroll
                     for (int aa = 0; aa < 4; ++aa) {
-                        const F d = dot(E1[aa], X), one = bc_<F>(1.f);
-                        dmn = lanes(min_nan, dmn, d);
-                        dmx = lanes([](float p, float q) { return fmaxf(p, q); }, dmx, d);
+                        const F db = dot(E1[aa], X), d = unfold(db, fold), one = bc_<F>(1.f);
+                        dmn = lanes([](float p, float q) { return fminf(p, q); }, dmn, db);
+                        dmx = lanes([](float p, float q) { return fmaxf(p, q); }, dmx, db);
                         // 1 / d, refined to half an ulp; psi = (d - 1)^2 / d and psi' = 1 - 1 / d^2
-                        // vanish with it on a fold
-                        const F r0 = lanes(rcp_pos, d);
+                        const F r0 = lanes(rcp_approx, d);
                         const F rd = fma_(r0, fma_(d, neg_(r0), one), r0);
                         const F dm = sub_(d, one), q = mul_(dm, rd);
                         const F y = fma_(dm, q, neg_(en_c)), t = add_(en, y);   // psi(d)
@@ -378,15 +384,14 @@ __device__ __forceinline__ void vcc_cell_body(const VccArgs &a, const VBlock &vb
         float mn, mxv;
         if constexpr (CPT == 2) {
             e = (valid0 ? (double)en.x - (double)en_c.x : 0.0) + (valid1 ? (double)en.y - (double)en_c.y : 0.0);
-            mn = min_nan(valid0 ? dmn.x : 3.4e38f, valid1 ? dmn.y : 3.4e38f);
+            mn = fminf(valid0 ? dmn.x : 3.4e38f, valid1 ? dmn.y : 3.4e38f);
             mxv = fmaxf(valid0 ? dmx.x : -3.4e38f, valid1 ? dmx.y : -3.4e38f);
         } else {
             e = valid0 ? (double)en - (double)en_c : 0.0;
             mn = valid0 ? dmn : 3.4e38f;
             mxv = valid0 ? dmx : -3.4e38f;
         }
-        // a fold is a bound that is not positive: the least one decides
-        int f = mn > 0.f ? 0 : 1;
+        int f = (valid0 && fold[0]) || (CPT == 2 && valid1 && fold[CPT - 1]) ? 1 : 0;
         for (int off = 16; off > 0; off >>= 1) {
             e += __shfl_xor_sync(FULL, e, off);
             f += __shfl_xor_sync(FULL, f, off);
