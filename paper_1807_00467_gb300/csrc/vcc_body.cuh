@@ -21,17 +21,22 @@
 // (60 us for 129 x 129 x 65 nodes at the ~97 three-operand FMA a clock and SM
 // that this part sustains).  The instructions around them are kept few: the
 // y-edges are taken one at a time in a rolled loop (their gradients parked in
-// shared memory), and cells add to the box's nodes in place, one corner at a time
-// over the block, instead of through per-cell slots and an indexed gather.  On large grids a thread holds two
-// cells, one per half of the packed f32x2 registers (TZ / 2 planes apart, their
-// nodes staged side by side), every operation serving both.  Gradient 137 ->
-// 87 us, GN product 107 -> 98 us at 129 x 129 x 65 (81 us with the energies of
-// four bounds added plainly before the compensated sum: up to 1.4 units in the
-// last place of a cell's energy instead of one).  The one-cell form (F =
-// float: small grids, and the persistent kernel, whose block leaves fewer
-// registers) runs the same operations, each rounded by an explicit intrinsic,
-// so both give the same bits.
+// shared memory), and cells add to the box's nodes in place, one corner at a
+// time over the block, instead of through per-cell slots and an indexed gather.
+// On large grids a thread holds two cells, one per half of the packed f32x2
+// registers (TZ / 2 planes apart, their nodes staged side by side), every
+// operation serving both.  Gradient 137 -> 87 us, GN product 107 -> 98 us at
+// 129 x 129 x 65 (gradient 81 us with the energies of four bounds added plainly
+// before the compensated sum: up to 1.4 units in the last place of a cell's
+// energy instead of one).  The reciprocal of the gradient is the approximate one
+// and a Newton step, correctly rounded for every mantissa while d and 1 / d are
+// normal; a thread with a bound beyond that repeats its cells with __frcp_rn.
+// The one-cell form (F = float: small grids and the diagonal) runs the same
+// operations as the two-cell one (large grids and the persistent kernel), each
+// rounded by an explicit intrinsic, so both give the same bits.
 #pragma once
+
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -300,55 +305,73 @@ __device__ __forceinline__ void vcc_cell_body(const VccArgs &a, const VBlock &vb
         for (int o = 0; o < 8; ++o) scatter(o, out[o][0], out[o][1], out[o][2]);
     } else {
         Vec<F> G1[4], G3[4];
+        // the 64 bounds; any: also bounds whose reciprocals the approximation flushes to 0 or inf
+        auto bounds = [&](auto any) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) G1[e] = G3[e] = Vec<F>{zero, zero, zero};
+            for (int e = 0; e < 4; ++e) G1[e] = G3[e] = Vec<F>{zero, zero, zero};
+            en = en_c = zero;
 #pragma unroll 1
-        for (int b = 0; b < 4; ++b) {
-            const Vec<F> E2 = y_edge(sm.su, b, true), nE2 = neg_(E2);
-            Vec<F> D2, nD2, G2{zero, zero, zero};
-            if constexpr (GN) {
-                D2 = y_edge(sm.sv, b, false);
-                nD2 = neg_(D2);
-            }
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const Vec<F> X = cross(E2, nE2, E3[c]);
-                Vec<F> W{zero, zero, zero};   // sum_a w e1_a
+            for (int b = 0; b < 4; ++b) {
+                const Vec<F> E2 = y_edge(sm.su, b, true), nE2 = neg_(E2);
+                [[maybe_unused]] Vec<F> D2, nD2;
+                Vec<F> G2{zero, zero, zero};
                 if constexpr (GN) {
-                    const Vec<F> Y = cross_add(D2, nD2, E3[c], cross(E2, nE2, D3[c]));
-#pragma unroll
-                    for (int aa = 0; aa < 4; ++aa) {
-                        const F d = dot(E1[aa], X), rd = lanes(rcp_approx, d);
-                        const F dd = dot_add(E1[aa], Y, dot(D1[aa], X));   // grad d . v
-                        const F w = lanes(if_pos, d, mul_(mul_(rd, rd), mul_(rd, dd)));   // psi''(d) (grad d . v) / 2
-                        axpy(w, X, G1[aa]);
-                        axpy(w, E1[aa], W);
-                    }
-                } else {
-#pragma unroll
-                    for (int aa = 0; aa < 4; ++aa) {
-                        const F db = dot(E1[aa], X), d = unfold(db, fold), one = bc_<F>(1.f);
-                        dmn = lanes([](float p, float q) { return fminf(p, q); }, dmn, db);
-                        dmx = lanes([](float p, float q) { return fmaxf(p, q); }, dmx, db);
-                        // 1 / d, refined to half an ulp; psi = (d - 1)^2 / d and psi' = 1 - 1 / d^2
-                        const F r0 = lanes(rcp_approx, d);
-                        const F rd = fma_(r0, fma_(d, neg_(r0), one), r0);
-                        const F dm = sub_(d, one), q = mul_(dm, rd);
-                        const F y = fma_(dm, q, neg_(en_c)), t = add_(en, y);   // psi(d)
-                        en_c = sub_(sub_(t, en), y);
-                        en = t;
-                        const F w = mul_(q, mul_(add_(d, one), rd));
-                        axpy(w, X, G1[aa]);
-                        axpy(w, E1[aa], W);
-                    }
+                    D2 = y_edge(sm.sv, b, false);
+                    nD2 = neg_(D2);
                 }
-                const Vec<F> nW = neg_(W);
-                G2 = cross_add_r(E3[c], W, nW, G2);
-                G3[c] = cross_add_r(W, E2, nE2, G3[c]);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const Vec<F> X = cross(E2, nE2, E3[c]);
+                    Vec<F> W{zero, zero, zero};   // sum_a w e1_a
+                    if constexpr (GN) {
+                        const Vec<F> Y = cross_add(D2, nD2, E3[c], cross(E2, nE2, D3[c]));
+#pragma unroll
+                        for (int aa = 0; aa < 4; ++aa) {
+                            const F d = dot(E1[aa], X), rd = lanes(rcp_approx, d);
+                            const F dd = dot_add(E1[aa], Y, dot(D1[aa], X));   // grad d . v
+                            const F w = lanes(if_pos, d, mul_(mul_(rd, rd), mul_(rd, dd)));   // psi''(d) (grad d . v) / 2
+                            axpy(w, X, G1[aa]);
+                            axpy(w, E1[aa], W);
+                        }
+                    } else {
+#pragma unroll
+                        for (int aa = 0; aa < 4; ++aa) {
+                            const F db = dot(E1[aa], X), d = unfold(db, fold), one = bc_<F>(1.f);
+                            dmn = lanes([](float p, float q) { return fminf(p, q); }, dmn, db);
+                            dmx = lanes([](float p, float q) { return fmaxf(p, q); }, dmx, db);
+                            // 1 / d, correctly rounded (all mantissas tried); psi = (d - 1)^2 / d, psi' = 1 - 1 / d^2
+                            F rd;
+                            if constexpr (decltype(any)::value) {
+                                rd = lanes([](float x) { return __frcp_rn(x); }, d);
+                            } else {
+                                const F r0 = lanes(rcp_approx, d);
+                                rd = fma_(r0, fma_(d, neg_(r0), one), r0);
+                            }
+                            const F dm = sub_(d, one), q = mul_(dm, rd);
+                            const F y = fma_(dm, q, neg_(en_c)), t = add_(en, y);   // psi(d)
+                            en_c = sub_(sub_(t, en), y);
+                            en = t;
+                            const F w = mul_(q, mul_(add_(d, one), rd));
+                            axpy(w, X, G1[aa]);
+                            axpy(w, E1[aa], W);
+                        }
+                    }
+                    const Vec<F> nW = neg_(W);
+                    G2 = cross_add_r(E3[c], W, nW, G2);
+                    G3[c] = cross_add_r(W, E2, nE2, G3[c]);
+                }
+                sm.g2[b * 3][tid] = G2.x;
+                sm.g2[b * 3 + 1][tid] = G2.y;
+                sm.g2[b * 3 + 2][tid] = G2.z;
             }
-            sm.g2[b * 3][tid] = G2.x;
-            sm.g2[b * 3 + 1][tid] = G2.y;
-            sm.g2[b * 3 + 2][tid] = G2.z;
+        };
+        bounds(std::false_type());
+        if constexpr (!GN) {
+            auto beyond = [](float mn, float mx) { return (mn > 0.f && mn < 0x1p-126f) || mx >= 0x1p126f; };
+            bool again;
+            if constexpr (CPT == 2) again = beyond(dmn.x, dmx.x) || beyond(dmn.y, dmx.y);
+            else again = beyond(dmn, dmx);
+            if (again) bounds(std::true_type());   // (all cells with __frcp_rn: 162 against 123 us a call at 129 x 129 x 65)
         }
         // edge gradients onto the cell's corners, scaled by +-1/g of the edge's axis
         // (times 2 for the GN product's halved weights): corner o is an end of one edge per axis
