@@ -391,10 +391,18 @@ int kp_mst(int32_t nk, const int32_t *kps, const float *intensity, double sigma_
  * are squared-distance min-convolutions over
  * the label grid (axis by axis).  marginals: float [nk][35937].
  * Synchronises the stream once, at its end; RG_ETIMEOUT if a bounded wait for
- * another vertex's message runs out. */
+ * another vertex's message runs out (marginals then holds no result: some of
+ * it may have been written). */
 int kp_bp_marginals(int32_t nk, const float *D, const int32_t *kps, const float *intensity, const int32_t *edges,
                     double sigma_i, double alpha, float *marginals, void *scratch, size_t scratch_bytes,
                     void *cuda_stream);
+
+/* Test hook: kp_bp_marginals whose first message is never recorded as
+ * complete, with waits of at most polls (1 .. 2^21): the waits for it run out
+ * and the call returns RG_ETIMEOUT (nk >= 2). */
+int kp_bp_marginals_timeout(int32_t nk, const float *D, const int32_t *kps, const float *intensity,
+                            const int32_t *edges, double sigma_i, double alpha, float *marginals, void *scratch,
+                            size_t scratch_bytes, void *cuda_stream, int32_t polls);
 
 /* Sec. II-C2-4: features, cost volume, MST (intensities of F), marginals and
  * their argmin; symmetric != 0 adds the backward search from x_k + d*_k with
@@ -402,7 +410,8 @@ int kp_bp_marginals(int32_t nk, const float *D, const int32_t *kps, const float 
  * (E_fw(k, d) + E_bw(k, -d)) / 2 (lowest label among equal energies).
  * disp: int32 [nk][3] displacements in voxels (mm).  marginals: NULL, or
  * float [nk][35937] forward marginals followed (symmetric) by [nk][35937]
- * backward ones.  Synchronises the stream. */
+ * backward ones; the array is worked in, so after an error (RG_ETIMEOUT as in
+ * kp_bp_marginals, RG_ECUDA) it holds no result.  Synchronises the stream. */
 int kp_match(const int32_t *n, const float *F, const float *M, int32_t nk, const int32_t *kps, const kp_params *p,
              int32_t symmetric, int32_t *disp, float *marginals, void *workspace, size_t ws_bytes,
              void *cuda_stream);

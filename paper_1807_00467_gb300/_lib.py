@@ -46,7 +46,8 @@ EXPORTS = [
     "regularizer_apply", "gn_pcg_solve", "gn_solve", "rg_pyramid_workspace_size", "register_pyramid",
     "rg_restrict_image", "rg_prolong_grid", "rg_last_error", "rg_version", "rg_profile", "rg_profile_read",
     "rg_launch_count", "ngf_distance_noalloc", "rg_set_tile", "rg_autotune", "kp_workspace_size", "kp_scratch_size",
-    "kp_ngf_features", "kp_cost_volume", "kp_mst", "kp_bp_marginals", "kp_match", "kp_launch_count",
+    "kp_ngf_features", "kp_cost_volume", "kp_mst", "kp_bp_marginals", "kp_bp_marginals_timeout", "kp_match",
+    "kp_launch_count",
     "kp_forstner_workspace_size", "kp_forstner", "register_pyramid_batch", "rg_sync", "rg_debug_hook",
 ]
 
@@ -84,6 +85,7 @@ def load():
         "kp_cost_volume": ([C.POINTER(i32), vp, vp, i32, vp, vp, vp], C.c_int),
         "kp_mst": ([i32, vp, vp, C.c_double, vp, vp, sz, vp], C.c_int),
         "kp_bp_marginals": ([i32, vp, vp, vp, vp, C.c_double, C.c_double, vp, vp, sz, vp], C.c_int),
+        "kp_bp_marginals_timeout": ([i32, vp, vp, vp, vp, C.c_double, C.c_double, vp, vp, sz, vp, i32], C.c_int),
         "kp_match": ([C.POINTER(i32), vp, vp, i32, vp, vp, i32, vp, vp, vp, sz, vp], C.c_int),
         "kp_launch_count": ([], C.c_int64),
         "kp_forstner_workspace_size": ([C.POINTER(i32), C.POINTER(sz)], C.c_int),

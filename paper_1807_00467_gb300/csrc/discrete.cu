@@ -542,14 +542,16 @@ struct BpArgs {
     unsigned *next;        // work counter
     unsigned *done;        // [n] CTAs of the vertex's cluster that have finished: kCl after the up message, 2 kCl with the marginal
     int *err;              // set to 2 when a wait runs out
+    int polls;             // polls before a wait gives up
+    int withhold;          // test hook: the first item's completion is never recorded
 };
 
 constexpr int kBpClusters = 38;          // clusters of 8 CTAs, two CTAs per SM
 constexpr int kBpPolls = 1 << 21;        // polls before a wait gives up (about two seconds)
 
 // Bounded wait for a completion count; after one wait has run out the others end too.
-__device__ __forceinline__ void bp_wait(const unsigned *p, unsigned need, int *err) {
-    for (int i = 0; i < kBpPolls; ++i) {
+__device__ __forceinline__ void bp_wait(const unsigned *p, unsigned need, int *err, int polls) {
+    for (int i = 0; i < polls; ++i) {
         unsigned v;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
         if (v >= need) return;
@@ -594,9 +596,9 @@ __global__ void __launch_bounds__(kBpT, 2) bp_kernel(const BpArgs a) {
             for (int c = 0; c < kCl; ++c) *cl.map_shared_rank(&s_item[slot], c) = it;
         }
     };
-    auto finish = [&](int k, unsigned add) {   // this CTA's stores of vertex k are complete
+    auto finish = [&](int item, int k, unsigned add) {   // this CTA's stores of vertex k are complete
         __syncthreads();
-        if (tid == 0) {
+        if (tid == 0 && !(a.withhold && item == 0)) {
             __threadfence();
             asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(a.done + k), "r"(add) : "memory");
         }
@@ -617,7 +619,7 @@ __global__ void __launch_bounds__(kBpT, 2) bp_kernel(const BpArgs a) {
 #pragma unroll
             for (int i = 0; i < kPer; ++i) h[i] = tid + i * kBpT < nown ? __ldg(src + tid + i * kBpT) : 0.f;
             const int c0 = a.child_off[k], c1 = a.child_off[k + 1];
-            for (int c = c0 + tid; c < c1; c += kBpT) bp_wait(a.done + a.child[c], kCl, a.err);
+            for (int c = c0 + tid; c < c1; c += kBpT) bp_wait(a.done + a.child[c], kCl, a.err, a.polls);
             __syncthreads();
             for (int c = c0; c < c1; ++c) {
                 const float *u = a.up + (long)a.child[c] * kL + pb;
@@ -630,7 +632,7 @@ __global__ void __launch_bounds__(kBpT, 2) bp_kernel(const BpArgs a) {
             for (int i = 0; i < kPer; ++i)
                 if (tid + i * kBpT < nown) mk[tid + i * kBpT] = h[i];
         } else {
-            if (tid == 0) bp_wait(a.done + q, 2 * kCl, a.err);
+            if (tid == 0) bp_wait(a.done + q, 2 * kCl, a.err, a.polls);
             __syncthreads();
             const float *src = a.marg + (long)q * kL + pb, *u = a.up + (long)k * kL + pb;
 #pragma unroll
@@ -640,7 +642,7 @@ __global__ void __launch_bounds__(kBpT, 2) bp_kernel(const BpArgs a) {
                 if (tid + i * kBpT < nown) h[i] -= __ldcg(u + tid + i * kBpT);
         }
         if (q < 0) {   // the root: its marginal is complete
-            finish(k, 2);
+            finish(item, k, 2);
             cl.sync();
             continue;
         }
@@ -689,7 +691,7 @@ __global__ void __launch_bounds__(kBpT, 2) bp_kernel(const BpArgs a) {
             }
             if (pass < 2) __syncthreads();
         }
-        finish(k, 1);
+        finish(item, k, 1);
     }
     cl.sync();   // no CTA leaves while another may still read its planes or write its mailbox
 }
@@ -847,7 +849,7 @@ cudaError_t run_mst(int n, const int *kps, const float *inten, float sig, KpWs &
 
 // Tree from the sorted MST edges, then both passes in one launch.
 int run_bp(int n, const float *D, const int *kps, const float *inten, float sig, float alpha, KpWs &w, float *marg,
-           cudaStream_t st) {
+           cudaStream_t st, int polls = kBpPolls, bool withhold = false) {
     const int root = 0;   // start of the sweeps that find the tree's centre
     if (allow_max_dynamic_smem(tree_kernel) != cudaSuccess) return RG_ECUDA;
     tree_kernel<<<1, 1024, tree_smem(n), st>>>(n, root, w.edges, w.deg, w.off, w.adj, w.order, w.level_off, w.nlevels,
@@ -871,6 +873,8 @@ int run_bp(int n, const float *D, const int *kps, const float *inten, float sig,
     a.next = w.next;
     a.done = w.done;
     a.err = w.err;
+    a.polls = polls;
+    a.withhold = withhold;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kCl * std::min(n, kBpClusters));
     cfg.blockDim = dim3(kBpT);
@@ -958,9 +962,9 @@ extern "C" int kp_mst(int32_t nk, const int32_t *kps, const float *intensity, do
     return read_flag(w, st);
 }
 
-extern "C" int kp_bp_marginals(int32_t nk, const float *D, const int32_t *kps, const float *intensity,
-                               const int32_t *edges, double sigma_i, double alpha, float *marginals, void *ws,
-                               size_t ws_bytes, void *stream) {
+static int bp_marginals(int32_t nk, const float *D, const int32_t *kps, const float *intensity, const int32_t *edges,
+                        double sigma_i, double alpha, float *marginals, void *ws, size_t ws_bytes, void *stream,
+                        int polls, bool withhold) {
     KpWs w;
     if (!D || !kps || !intensity || !edges || !marginals || kp_scratch(nk, ws, ws_bytes, w) != RG_OK)
         return RG_EINVAL;
@@ -969,8 +973,21 @@ extern "C" int kp_bp_marginals(int32_t nk, const float *D, const int32_t *kps, c
         return RG_ECUDA;
     flag_kernel<<<1, 1, 0, st>>>(w.err);
     counted();
-    const int s = run_bp(nk, D, kps, intensity, (float)sigma_i, (float)alpha, w, marginals, st);
+    const int s = run_bp(nk, D, kps, intensity, (float)sigma_i, (float)alpha, w, marginals, st, polls, withhold);
     return s ? s : read_flag(w, st);
+}
+
+extern "C" int kp_bp_marginals(int32_t nk, const float *D, const int32_t *kps, const float *intensity,
+                               const int32_t *edges, double sigma_i, double alpha, float *marginals, void *ws,
+                               size_t ws_bytes, void *stream) {
+    return bp_marginals(nk, D, kps, intensity, edges, sigma_i, alpha, marginals, ws, ws_bytes, stream, kBpPolls, false);
+}
+
+extern "C" int kp_bp_marginals_timeout(int32_t nk, const float *D, const int32_t *kps, const float *intensity,
+                                       const int32_t *edges, double sigma_i, double alpha, float *marginals, void *ws,
+                                       size_t ws_bytes, void *stream, int32_t polls) {
+    if (polls < 1 || polls > kBpPolls) return RG_EINVAL;
+    return bp_marginals(nk, D, kps, intensity, edges, sigma_i, alpha, marginals, ws, ws_bytes, stream, polls, true);
 }
 
 extern "C" int kp_match(const int32_t *n, const float *F, const float *M, int32_t nk, const int32_t *kps,
