@@ -124,8 +124,8 @@ typedef struct {
  * wide and 20 high, whole grid cells per axis, two or more voxels per cell
  * along x and y) run in one persistent cooperative kernel per level iteration
  * (up to 24 pairs per launch), on levels where these pairs together have at
- * most two 60 x 16 voxel columns per SM (in z chunks on small volumes; larger
- * levels keep their launches, which are faster there).  The kernel's
+ * most seven 60 x 16 voxel columns (in z chunks on small volumes) per eight SMs;
+ * larger levels keep their launches, which are faster at every size.  The kernel's
  * CTAs take (pair, tile) items from a work counter, each waiting (bounded;
  * RG_ETIMEOUT when a wait runs out) for the previous phase of its own pair.
  * Same bits per pair as without the flag.  RG_SCHED_HOOK_BARRIER is a test

@@ -62,8 +62,9 @@ def register_batch_graph(pairs, params, levels, gn_iters, pcg_iters, ls_max=10, 
     one CUDA graph per level advancing every pair's Gauss-Newton iteration
     (register_pyramid_batch); no host threads.  persistent: the PCG steps of
     the pairs whose level the column GN-product kernel covers run in one
-    persistent cooperative kernel per iteration, on levels of at most two
-    columns per SM (RG_SCHED_PERSISTENT; same bits); hook_barrier: test hook, that kernel's grid barriers run out
+    persistent cooperative kernel per iteration, on levels of at most seven
+    columns per eight SMs (RG_SCHED_PERSISTENT; same bits, slower than without);
+    hook_barrier: test hook, that kernel's grid barriers run out
     (RG_ETIMEOUT).  Returns (displacements, reports, seconds, code): code is
     RG_OK, or the halting status (RG_EFOLD, RG_ENONFINITE) of the
     lowest-numbered pair whose schedule halted; such a pair keeps its start

@@ -1022,9 +1022,12 @@ static int pcg(rg_ctx *c, const float *g, float *p, int iters, double *stats) {
 static bool batch_pcg_ok(const rg_ctx *c) { return !c->general_only && c->nk <= 0 && pcg_batch_supported(c->cp); }
 
 // The persistent kernel takes a level whose covered pairs together have at most
-// two columns per SM.  Beyond that each phase fills the chip in launches of its
-// own, which keep their own shapes (24 pairs of 320x320x96, 5 iterations of 20
-// PCG steps: 543 ms persistent, 314 ms as launches; 2880 columns).
+// seven columns per eight SMs.  The level's launches are faster at every size (one
+// pair of 80x64x32, 5 iterations of 20 PCG steps: 6.4 ms against 16.0; 4 pairs of
+// 128x128x48: 11.8 against 23.9), so the kernel keeps only the levels where the
+// product's CTA shape (10 warps) costs its other phases nothing: against CTAs of
+// 20 warps, 16.0 / 16.4 ms at 16 columns, 19.1 / 19.1 at 128, 18.4 / 18.0 at 144
+// and 22.7 / 21.1 at 192.
 static long batch_columns(const rg_ctx *c) { return (long)c->cp.nb[0] * c->cp.nb[1] * c->cp.nbz; }
 
 // The operands of one PCG step of the context (the GN product H d into q as
@@ -1698,7 +1701,7 @@ extern "C" int register_pyramid_batch(int32_t npairs, const rg_image_geom *img, 
         long ncols = 0;
         for (int p = 0; p < npairs; ++p)
             if (!halted[p] && batch_pcg_ok(ps[p].cl)) ncols += batch_columns(ps[p].cl);
-        const bool pers_level = persistent && ncols <= 2L * device_sm_count();
+        const bool pers_level = persistent && 8 * ncols <= 7L * device_sm_count();
         for (int p = 0; p < npairs && cst == RG_OK; ++p) {
             if (halted[p]) continue;
             rg_ctx *cl = ps[p].cl;
