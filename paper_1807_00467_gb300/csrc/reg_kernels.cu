@@ -149,38 +149,51 @@ __global__ void kp_kernel(const KpArgs a) {
     }
 }
 
-// node sums: warp (r, o) for the first sorted keypoint r of a cell and a
-// corner o of that cell owns node n = cell + o unless a cell n - o' with o' < o
-// holds keypoints; the owner adds, in the order (o'', i), the contributions
-// of every keypoint in the cells n - o'' to out[n] (diag: 2 delta w^2 to all
-// three components; else 2 scale w src_i).  The lanes form the terms of 32
-// keypoints at once and add them in order through shuffles: one thread per node
-// followed a chain of dependent loads, two per keypoint (48 us for 3000
-// keypoints along 30 vessels in a 65 x 65 x 33 grid, 10 us so).
-template <bool DIAG>
-__global__ void __launch_bounds__(256) kp_gather_kernel(const KpArgs a, double two_delta, float *out) {
-    if (a.skip && *a.skip) return;   // uniform: every block reads the same flag
-    constexpr unsigned FULL = 0xffffffffu;
-    const unsigned t = blockIdx.x * 8u + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31, r = (int)(t >> 3), o = (int)(t & 7u);
-    if (r >= a.nk) return;
-    const int *sb = a.ix.sb;
-    const int b = sb[r];
-    if (r > 0 && b == sb[r - 1]) return;
+// node sums: the first sorted keypoint r of a cell and a corner o of that cell
+// own node n = cell + o unless a cell n - o' with o' < o holds keypoints; the
+// owner adds, in the order (o'', i), the contributions of every keypoint in the
+// cells n - o'' to out[n] (diag: 2 delta w^2 to all three components; else
+// 2 scale w src_i).
+
+// lane op < 8: the first sorted keypoint of cell n - op (and the cell) of the
+// node n of (r, o), -1 if it holds none or lies outside the cell grid
+__device__ __forceinline__ long kp_node(const KpArgs &a, int b, int o, int op, int &cell, int &first) {
     const int mx = a.m[0], my = a.m[1];
-    const long mxy = (long)mx * my, M = mxy * a.m[2];
+    const long mxy = (long)mx * my;
     const int cz = b / (int)mxy, cy = (b - cz * (int)mxy) / mx, cx = b - cz * (int)mxy - cy * mx;
     const int nx = cx + (o & 1), ny = cy + ((o >> 1) & 1), nz = cz + (o >> 2);
-    // lane op < 8: the first sorted keypoint of cell n - op, -1 if it holds none or lies outside the cell grid
-    int first = -1, cell = -1;
-    if (lane < 8) {
-        const int x = nx - (lane & 1), y = ny - ((lane >> 1) & 1), z = nz - (lane >> 2);
-        if (!(x < 0 || y < 0 || z < 0 || x > mx - 2 || y > my - 2 || z > a.m[2] - 2)) {
-            cell = (z * my + y) * mx + x;
-            first = a.ix.soc[cell];
-        }
+    const int x = nx - (op & 1), y = ny - ((op >> 1) & 1), z = nz - (op >> 2);
+    cell = first = -1;
+    if (op < 8 && !(x < 0 || y < 0 || z < 0 || x > mx - 2 || y > my - 2 || z > a.m[2] - 2)) {
+        cell = (z * my + y) * mx + x;
+        first = a.ix.soc[cell];
     }
-    if (__any_sync(FULL, lane < o && first >= 0)) return;   // a lower corner's warp owns the node
+    return (long)nz * mxy + (long)ny * mx + nx;
+}
+
+// a keypoint's term of a node, w times src (DIAG: w alone)
+template <bool DIAG>
+__device__ __forceinline__ float kp_term(const KpArgs &a, double two_delta, int q, int op, float (&v)[3]) {
+    const int i = a.ix.perm[q];
+    const float f[3] = {a.ix.frac[3 * i], a.ix.frac[3 * i + 1], a.ix.frac[3 * i + 2]};
+    const float w = kp_weight(op, f);
+    if constexpr (DIAG) {
+        return (float)(two_delta * w * w);
+    } else {
+        for (int k = 0; k < 3; ++k) v[k] = a.ix.src[3 * i + k];
+        return 2.f * a.scale * w;
+    }
+}
+
+// the sum of the node of (r, o) by a whole warp: the lanes form the terms of 32
+// keypoints at once and add them in order through shuffles
+template <bool DIAG>
+__device__ __forceinline__ void kp_warp_sum(const KpArgs &a, double two_delta, int r, int o, float *out) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, *sb = a.ix.sb;
+    int cell, first;
+    const long n = kp_node(a, sb[r], o, lane, cell, first);
+    if (__any_sync(FULL, lane < o && first >= 0)) return;   // a lower corner owns the node
     float acc[3] = {0.f, 0.f, 0.f};
     for (int op = 0; op < 8; ++op) {
         const int s = __shfl_sync(FULL, first, op), c = __shfl_sync(FULL, cell, op);
@@ -188,27 +201,74 @@ __global__ void __launch_bounds__(256) kp_gather_kernel(const KpArgs a, double t
         for (int q0 = s;; q0 += 32) {
             const bool in = q0 + lane < a.nk && sb[q0 + lane] == c;   // a prefix of the lanes: the cells are sorted
             float w = 0.f, v[3] = {0.f, 0.f, 0.f};
-            if (in) {
-                const int i = a.ix.perm[q0 + lane];
-                const float f[3] = {a.ix.frac[3 * i], a.ix.frac[3 * i + 1], a.ix.frac[3 * i + 2]};
-                w = kp_weight(op, f);
-                if (DIAG) {
-                    w = (float)(two_delta * w * w);
-                } else {
-                    w = 2.f * a.scale * w;
-                    for (int k = 0; k < 3; ++k) v[k] = a.ix.src[3 * i + k];
-                }
-            }
-            const int n = __popc(__ballot_sync(FULL, in));
-            for (int j = 0; j < n; ++j) {
+            if (in) w = kp_term<DIAG>(a, two_delta, q0 + lane, op, v);
+            const int cnt = __popc(__ballot_sync(FULL, in));
+            for (int j = 0; j < cnt; ++j) {
                 const float wj = __shfl_sync(FULL, w, j);
                 for (int k = 0; k < 3; ++k) acc[k] = DIAG ? acc[k] + wj : fmaf(wj, __shfl_sync(FULL, v[k], j), acc[k]);
             }
-            if (n < 32) break;
+            if (cnt < 32) break;
         }
     }
-    const long n = (long)nz * mxy + (long)ny * mx + nx;
+    const long M = (long)a.m[0] * a.m[1] * a.m[2];
     if (lane < 3) out[lane * M + n] += lane == 0 ? acc[0] : lane == 1 ? acc[1] : acc[2];
+}
+
+// A warp takes rw keypoints r of one corner.  rw = 1: it sums the node.  Else
+// each lane below rw sums its node itself while no cell of it holds more than
+// kLight keypoints, and the warp together sums the others one after the other.
+// One thread per node (light or not) follows a chain of two dependent loads per
+// keypoint, one warp per node makes eight warps of every keypoint, of which most
+// find nothing to do.  The call, of which ~20 us are the other kernels, in a 65 x
+// 65 x 17 grid, by thread / by warp / so: 3000 keypoints along 30 vessels 45 / 30
+// / 32 us, 100000 spread evenly 69 / 155 / 62 us, 100000 along 30 vessels 675 /
+// 102 / 87 us.  rw leaves about 12000 warps, 80 per SM.
+constexpr int kLight = 8;
+template <bool DIAG>
+__global__ void __launch_bounds__(256) kp_gather_kernel(const KpArgs a, int rw, double two_delta, float *out) {
+    if (a.skip && *a.skip) return;   // uniform: every block reads the same flag
+    const unsigned wid = blockIdx.x * 8u + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31, o = (int)(wid & 7u), r0 = (int)(wid >> 3) * rw, r = r0 + lane, *sb = a.ix.sb;
+    const bool cell_start = lane < rw && r < a.nk && (r == 0 || sb[r] != sb[r - 1]);
+    bool heavy = cell_start;
+    if (rw > 1 && cell_start) {
+        int cell[8], first[8];
+        long n = 0;
+        bool own = true;
+        heavy = false;
+#pragma unroll
+        for (int op = 0; op < 8; ++op) {
+            n = kp_node(a, sb[r], o, op, cell[op], first[op]);
+            own = own && !(op < o && first[op] >= 0);
+        }
+#pragma unroll
+        for (int op = 0; op < 8; ++op) {
+            const int q = first[op] + kLight;
+            heavy = heavy || (own && first[op] >= 0 && q < a.nk && sb[q] == cell[op]);
+        }
+        if (own && !heavy) {
+            float acc[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+            for (int op = 0; op < 8; ++op)
+                for (int q = first[op]; q >= 0 && q < a.nk && sb[q] == cell[op]; ++q) {
+                    float v[3];
+                    const float w = kp_term<DIAG>(a, two_delta, q, op, v);
+                    for (int k = 0; k < 3; ++k) acc[k] = DIAG ? acc[k] + w : fmaf(w, v[k], acc[k]);
+                }
+            const long M = (long)a.m[0] * a.m[1] * a.m[2];
+            for (int k = 0; k < 3; ++k) out[k * M + n] += acc[k];
+        }
+    }
+    for (unsigned todo = __ballot_sync(0xffffffffu, heavy); todo; todo &= todo - 1)
+        kp_warp_sum<DIAG>(a, two_delta, r0 + __ffs(todo) - 1, o, out);
+}
+
+template <bool DIAG>
+static cudaError_t launch_gather(const KpArgs &a, double two_delta, float *out, cudaStream_t st) {
+    int rw = 1;
+    while (rw < 32 && a.nk > 1536L * rw) rw *= 2;
+    kp_gather_kernel<DIAG><<<(a.nk + rw - 1) / rw, 256, 0, st>>>(a, rw, two_delta, out);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_kp(const KpArgs &a, cudaStream_t st) {
@@ -218,8 +278,7 @@ cudaError_t launch_kp(const KpArgs &a, cudaStream_t st) {
 
 cudaError_t launch_kp_gather(const KpArgs &a, cudaStream_t st) {
     if (!a.out || a.nk <= 0) return cudaSuccess;
-    kp_gather_kernel<false><<<a.nk, 256, 0, st>>>(a, 0.0, a.out);
-    return cudaGetLastError();
+    return launch_gather<false>(a, 0.0, a.out, st);
 }
 
 // ------------------------------------------------------------------ terms
@@ -329,8 +388,7 @@ cudaError_t launch_jacobi_diag(int alpha_on, const int *m, const float *ig2, dou
 
 cudaError_t launch_kp_diag(const KpArgs &a, double two_delta, float *diag, cudaStream_t st) {
     if (a.nk <= 0) return cudaSuccess;
-    kp_gather_kernel<true><<<a.nk, 256, 0, st>>>(a, two_delta, diag);
-    return cudaGetLastError();
+    return launch_gather<true>(a, two_delta, diag, st);
 }
 
 // reciprocal of the preconditioner diagonal; entries that are not positive
