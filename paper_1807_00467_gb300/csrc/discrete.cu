@@ -38,6 +38,7 @@ constexpr int kCvR = kS / kRun, kCvD = kS / kDy;   // runs along x, groups along
 constexpr int kCvT = 256;           // cost-volume threads (3 runs x 7 z labels x 11 y groups = 231 busy)
 constexpr int kWp = kW + 1;         // window row pitch (odd: y groups start in different banks)
 constexpr int kWPlane = kW * kWp;
+constexpr int kFewG = 2, kFewT = 224;   // z labels and threads (2 x 33 rows x 3 runs = 198 busy) per CTA for few keypoints
 constexpr int kCl = 8;              // CTAs per message (one thread-block cluster)
 constexpr int kBpT = 256;           // threads per message CTA
 
@@ -149,6 +150,64 @@ __global__ void __launch_bounds__(kCvT, 1) cost_volume_kernel(int nx, int ny, in
     for (int d = 0; d < kDy; ++d)
 #pragma unroll
         for (int j = 0; j < kRun; ++j) out[d * kS + j] = fmaf(-acc[d][j], 1.f / 64.f, 1.f);
+}
+
+// The cost volume of few keypoints: CTAs of two z labels and one y label per
+// thread, shorter and more of them per keypoint.  A label's patch points are
+// added in the same order as above (same bits).
+__global__ void __launch_bounds__(kFewT) cost_volume_few_kernel(int nx, int ny, int nz, const float4 *__restrict__ ffix,
+                                                                const float4 *__restrict__ fmov,
+                                                                const int *__restrict__ kps, float *__restrict__ D) {
+    extern __shared__ float4 sm4[];
+    float4 *win = sm4;                          // [kFewG + 3][kW][kW]
+    float4 *pf = sm4 + (kFewG + 3) * kW * kW;   // [4][4][4] fixed patch
+    const int ng = (kS + kFewG - 1) / kFewG;
+    const int k = blockIdx.x / ng, g = blockIdx.x - k * ng;
+    const int kx = kps[3 * k], ky = kps[3 * k + 1], kz = kps[3 * k + 2];
+    const int dz0 = g * kFewG;
+    const int tid = threadIdx.x;
+    for (int i = tid; i < (kFewG + 3) * kW * kW; i += kFewT) {
+        const int pz = i / (kW * kW), r = i - pz * kW * kW, wy = r / kW, wx = r - wy * kW;
+        const int z = clampi(kz + 2 * (dz0 + pz) - 35, 0, nz - 1);
+        const int y = clampi(ky + 2 * wy - 35, 0, ny - 1), x = clampi(kx + 2 * wx - 35, 0, nx - 1);
+        win[i] = __ldg(fmov + ((long)z * ny + y) * nx + x);
+    }
+    if (tid < 64) {
+        const int px = tid & 3, py = (tid >> 2) & 3, pz = tid >> 4;
+        const int z = clampi(kz + 2 * pz - 3, 0, nz - 1), y = clampi(ky + 2 * py - 3, 0, ny - 1);
+        const int x = clampi(kx + 2 * px - 3, 0, nx - 1);
+        pf[tid] = __ldg(ffix + ((long)z * ny + y) * nx + x);
+    }
+    __syncthreads();
+    const int run = tid % kCvR, dy = (tid / kCvR) % kS, dzl = tid / (kCvR * kS), dz = dz0 + dzl;
+    if (dzl >= kFewG || dz >= kS) return;
+    float acc[kRun];
+#pragma unroll
+    for (int j = 0; j < kRun; ++j) acc[j] = 0.f;
+#pragma unroll 1
+    for (int pz = 0; pz < 4; ++pz) {
+#pragma unroll 1
+        for (int py = 0; py < 4; ++py) {
+            const float4 *row = win + ((dzl + pz) * kW + (dy + py)) * kW + run * kRun;
+            float4 m[kRun + 3];
+#pragma unroll
+            for (int j = 0; j < kRun + 3; ++j) m[j] = row[j];
+            const float4 *f = pf + (pz * 4 + py) * 4;
+#pragma unroll
+            for (int px = 0; px < 4; ++px) {
+                const float4 q = f[px];
+#pragma unroll
+                for (int j = 0; j < kRun; ++j) {
+                    const float4 a = m[j + px];
+                    const float r = fmaf(a.w, q.w, fmaf(a.z, q.z, fmaf(a.y, q.y, a.x * q.x)));
+                    acc[j] = fmaf(r, r, acc[j]);
+                }
+            }
+        }
+    }
+    float *out = D + (long)k * kL + ((long)dz * kS + dy) * kS + run * kRun;
+#pragma unroll
+    for (int j = 0; j < kRun; ++j) out[j] = fmaf(-acc[j], 1.f / 64.f, 1.f);
 }
 
 // ------------------------------------------------------------ MST (Boruvka)
@@ -824,13 +883,21 @@ cudaError_t run_features(const int *n, const float *img, float eta, float4 *feat
 cudaError_t run_cost(const int *n, const float4 *ffix, const float4 *fmov, int nk, const int *kps, float *D,
                      cudaStream_t st) {
     if (nk <= 0) return cudaSuccess;
-    const size_t smem = sizeof(float4) * ((kCvG + 3) * kWPlane + 64);
-    cudaError_t e = allow_max_dynamic_smem(cost_volume_kernel);
-    if (e != cudaSuccess) return e;
-    const int ng = (kS + kCvG - 1) / kCvG;
-    cost_volume_kernel<<<nk * ng, kCvT, smem, st>>>(n[0], n[1], n[2], ffix, fmov, kps, D);
+    auto run = [&](auto kernel, int G, int threads, size_t points) {
+        cudaError_t e = allow_max_dynamic_smem(kernel);
+        if (e != cudaSuccess) return e;
+        kernel<<<nk * ((kS + G - 1) / G), threads, sizeof(float4) * (points + 64), st>>>(n[0], n[1], n[2], ffix, fmov, kps, D);
+        return cudaGetLastError();
+    };
+    // The wide form's five CTAs per keypoint run one per SM in whole waves of 26 us,
+    // so it is taken from ten waves on: us for 1, 8, 46, 100, 200 keypoints 29, 31,
+    // 67, 106, 195 against 19, 19, 53, 101, 187; at 300 272 / 272, at 500 438 / 443,
+    // at 3000 2496 / 2575.
+    const cudaError_t e = 5L * nk >= 10L * device_sm_count()
+                              ? run(cost_volume_kernel, kCvG, kCvT, (kCvG + 3) * kWPlane)
+                              : run(cost_volume_few_kernel, kFewG, kFewT, (kFewG + 3) * kW * kW);
     counted();
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t run_mst(int n, const int *kps, const float *inten, float sig, KpWs &w, cudaStream_t st) {
