@@ -161,13 +161,17 @@ static long lin_pitch(int n0) { return (n0 + 3) & ~3; }
 // z chunk (fill): a CTA marches its chunk's planes and a 2-plane halo on either
 // side one after the other, so a volume with few x-y tiles is bound by that
 // chain while most SMs idle (64x64x48: 24 CTAs of 32 planes on 152 SMs).  The
-// chunk is the number of whole cells that minimises waves x (planes + halo +
-// fixed cost of a chunk, about 4 planes' time); large volumes keep 32 planes.
+// chunk is the number of whole cells that minimises the longest SM's sum of
+// (planes + halo + fixed cost of a chunk, about 4 planes' time) over its tiles,
+// dealt in turn, the shorter last chunks included; large volumes keep 32 planes.
 // The geometry fixes a result's bits, so it cannot depend on what else runs:
 // where a batch's pairs fill the chip together, halos and fixed costs are work
 // that nothing pays back, so chunks that add more than half to the planes of
 // the 32-plane ones are not taken (24 pairs of 64x64x48, 5 iterations of 20 PCG
-// steps: 27.5 ms in 32-plane chunks, 30.1 with this limit, 36 without it).
+// steps: 27.5 ms in 32-plane chunks, 30.1 with this limit, 36 without it), nor
+// are those that promise less than a twentieth (256x128x64 with cells of 2x1x2
+// voxels, 14 planes for 20, a promise of 3%: objective 95 -> 103 us, gradient
+// 154 -> 167).
 // 152: the SM count of the part, a constant so that a workspace sized on one
 // machine fits the context made on another.
 // 64x64x48 (chunk of 8): ngf_gradient 64 -> 37 us (a chunk of 4: 33 us);
@@ -193,13 +197,24 @@ static void tile_geom(const rg_image_geom *img, const rg_grid_geom *grid, TileGe
         t.TZ -= t.rho[2];
     if (fill) {
         const long nxy = (long)((t.n[0] + t.TXI - 1) / t.TXI) * ((t.n[1] + t.TY - 1) / t.TY);
-        long best = LONG_MAX;
-        int tz = t.TZ;
         auto planes = [&](int c) { return t.n[2] + 8L * ((t.n[2] + c - 1) / c); };   // marched per x-y tile, halos and fixed cost
-        for (int c = t.TZ; c >= t.rho[2]; c -= t.rho[2]) {   // ties: the larger chunk (fewer boxes)
+        auto longest = [&](int c) {   // of 152 SMs: the full chunks' tiles come first, then the last ones'
+            const long nz = (t.n[2] + c - 1) / c, full = nxy * (nz - 1), all = nxy * nz;
+            const int last = t.n[2] - (int)(nz - 1) * c;
+            long m = 0;
+            for (long sm = 0; sm < 152 && sm < all; ++sm) {
+                const long f = sm < full ? (full - sm + 151) / 152 : 0, a = (all - sm + 151) / 152;
+                m = std::max(m, f * (c + 8) + (a - f) * (last + 8));
+            }
+            return m;
+        };
+        const long whole = longest(t.TZ);
+        long best = whole;
+        int tz = t.TZ;
+        for (int c = t.TZ - t.rho[2]; c >= t.rho[2]; c -= t.rho[2]) {   // ties: the larger chunk (fewer boxes)
             if (2 * planes(c) > 3 * planes(t.TZ)) break;
-            const long cost = (nxy * ((t.n[2] + c - 1) / c) + 151) / 152 * (c + 8);
-            if (cost < best) {
+            const long cost = longest(c);
+            if (cost < best && 20 * cost < 19 * whole) {
                 best = cost;
                 tz = c;
             }
