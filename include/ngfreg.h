@@ -327,8 +327,10 @@ int rg_sync(rg_ctx *ctx);
  * before such a wait gives up (default 2^20).  RG_HOOK_PASS (value 0, 1, 2):
  * the objective / gradient / linearisation pass chosen by the volume's size
  * (0, the default: the column-marching pass for the objective when its 62 x 18
- * voxel columns have at least 16 planes per SM, and for the gradient and
- * linearisation when there is at least one column of 60 x 16 voxels per SM), always the column-marching pass where it
+ * voxel columns have at least 16 planes per SM, and for the objective, gradient
+ * and linearisation when there is at least one column of 60 x 16 voxels per SM;
+ * in both cases R must start on an even element), always the column-marching
+ * pass where it
  * applies (1), or always the tile pass (2); the results agree within rounding. */
 #define RG_HOOK_NO_TMA 1
 #define RG_HOOK_POLL_LIMIT 2

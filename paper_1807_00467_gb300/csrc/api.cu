@@ -675,18 +675,19 @@ static int run_tile(rg_ctx *c, int mode, const float *field) {
     // the SMs, with at least 16 planes per SM (below that the two halo planes and
     // the start of a piece outweigh what its columns save: 24 pairs of 80x64x32 in
     // one batch 25.8 ms, 23.3 by the tile pass; a step at 96x96x48 alone 1.46 and
-    // 1.45 ms), the gradient and linearisation where the volume has at least one
-    // column per SM (narrower volumes keep the z-chunked tile pass, whose tiles
-    // fill the GPU).  Both load R's voxels in pairs, so an image that starts on an
+    // 1.45 ms) or, in thin slabs, a whole column per SM (512x512x8: 41 us, tile pass
+    // 56, FP16 images 64), the gradient and linearisation where the volume has one
+    // 60 x 16 voxel column per SM (narrower volumes keep the z-chunked tile pass,
+    // whose tiles fill the GPU).  Both load R's voxels in pairs, so an image that starts on an
     // odd element (a view into a larger buffer) takes the tile pass, whose loads
     // are single voxels; R's rows keep the pairs aligned (even widths only).
     const bool r_pairs = ((uintptr_t)c->R & (c->dtype == RG_F32 ? 7 : 3)) == 0;
     const bool colpass = mode != MODE_MATVEC && mode != MODE_DIAG && !c->general_only && c->pass_sel != 2 && r_pairs;
     const long obj_planes = (c->cg.n[0] + 61) / 62 * (long)((c->cg.n[1] + 17) / 18) * c->cg.n[2];   // 62 x 18 columns
+    const bool col_per_sm = c->cg.nb[0] * c->cg.nb[1] >= device_sm_count();
     const bool gobj = colpass && mode == MODE_OBJ && ngf_gobj_supported(c->cg) &&
-                      (c->pass_sel == 1 || obj_planes >= 16L * device_sm_count());
-    const bool gcol = colpass && mode != MODE_OBJ && ngf_gcol_supported(c->cg) &&
-                      (c->pass_sel == 1 || c->cg.nb[0] * c->cg.nb[1] >= device_sm_count());
+                      (c->pass_sel == 1 || col_per_sm || obj_planes >= 16L * device_sm_count());
+    const bool gcol = colpass && mode != MODE_OBJ && ngf_gcol_supported(c->cg) && (c->pass_sel == 1 || col_per_sm);
     if (gobj || gcol) {
         auto run = [&](auto &g, auto *R, auto *T) {
             g.g = c->cg;

@@ -29,3 +29,19 @@ def test_objective_against_oracle_and_tile_pass(n, m, half):
         assert rel(J, tile) <= 1e-7
         same_bits.append(J == tile)
     assert not all(same_bits)
+
+
+def test_thin_slab_takes_columns():
+    """A slab of few planes with a column per SM: the pass chosen by size is the column pass (its bits)."""
+    import torch
+    from paper_1807_00467_gb300 import api
+    n, m = (512, 512, 8), (129, 129, 5)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    R, T = (200.0 * torch.rand(n[::-1], generator=g, device="cuda") for _ in range(2))
+    ctx = api.Context(R, T, (1.0, 1.0, 2.0), m, api.make_params(), pcg_max=1)
+    u = to_dev(phantom.random_grid_field(m, seed=9))
+    J = {}
+    for hook in (0, 1, 2):
+        ctx.debug_hook(RG_HOOK_PASS, hook)
+        J[hook] = float(ctx.ngf_objective(u)[0])
+    assert J[0] == J[1] and rel(J[1], J[2]) <= 1e-7 and J[1] != J[2]
