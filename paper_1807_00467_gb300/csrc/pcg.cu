@@ -130,16 +130,20 @@ __global__ void __launch_bounds__(kVT, 2) pcg_dir_kernel(Part P, PcgScalars *sc,
 // launches of 6 blocks spent much of their ~30 us on launch, drain and
 // re-reading r, M^-1 and the scalars: 24 us fused at 11 k floats.  Up to 16
 // blocks: longer vectors need more than a cluster's SMs for their history.
+// Groups of six residuals and 64 registers, so that two blocks share an SM: the
+// clusters of a batch's pairs compete for whole SMs (24 pairs of 96x96x48, 5
+// iterations of 20 PCG steps: 40.6 -> 39.3 ms, 39.7 as three launches; groups of
+// eight in one block an SM: the same for a lone small solve).
 template <int Q>
-__global__ void __launch_bounds__(kVT) pcg_fused_kernel(Part P, PcgScalars *sc, const double *apart, int napart,
+__global__ void __launch_bounds__(kVT, 2) pcg_fused_kernel(Part P, PcgScalars *sc, const double *apart, int napart,
                                                      const float *q, const float *minv, float *Rh, long stride, int k,
                                                      double *part, double *rzh, double *rzpart, float *d, float *s) {
     __shared__ PcgSmem sm;
     const VBlock b = cuda_block_1d();
     cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
-    pcg_step_body<Q>(P, sc, apart, napart, q, minv, Rh, stride, k, part, b, sm);
+    pcg_step_body<Q, 1, 6>(P, sc, apart, napart, q, minv, Rh, stride, k, part, b, sm);
     cl.sync();
-    pcg_reorth_body<Q>(P, sc, minv, Rh, stride, k, rzh, part, rzpart, b, sm);
+    pcg_reorth_body<Q, 1, 6>(P, sc, minv, Rh, stride, k, rzh, part, rzpart, b, sm);
     cl.sync();
     pcg_dir_body(P, sc, minv, Rh + (long)(k + 1) * stride, d, s, k, rzh, rzpart, b, sm);
 }

@@ -123,14 +123,14 @@ struct PcgSmem {
 // ---------------------------------------------------------------------------
 // alpha = r.z / d.q (stop on a non-positive curvature d.q or a vanishing r.z);
 // r_{k+1} = r_k - alpha q; then the partials of (M^-1 r_{k+1}) . r_j, j = 0..k
-template <int Q = 0, int S = 1>
+template <int Q = 0, int S = 1, int G = hist_group<Q>()>
 __device__ __forceinline__ void pcg_step_body(const Part &P, PcgScalars *sc, const double *apart, int napart,
                                               const float *q, const float *minv, float *Rh, long stride, int k,
                                               double *part, const VBlock &b, PcgSmem &sm) {
     double (&wp)[kHist][kVW] = sm.wp;
     double *red = sm.red;
     const int nb = b.nblk, lane = b.tid & 31;
-    constexpr int NQ = Q > 0 ? Q : kQmax, G = hist_group<Q>();
+    constexpr int NQ = Q > 0 ? Q : kQmax;
     // a short vector's operands are loaded before the scalars are formed
     float4 x[Q > 0 ? G : 1][NQ];
     auto load_group = [&](int j0) {
@@ -225,7 +225,7 @@ __device__ __forceinline__ void pcg_step_body(const Part &P, PcgScalars *sc, con
 // ---------------------------------------------------------------------------
 // c_j = (M^-1 r_{k+1}) . r_j / (r_j . z_j);  r_{k+1} -= sum_j c_j r_j;  then the
 // partials of r.z with z = M^-1 r_{k+1}
-template <int Q = 0, int S = 1>
+template <int Q = 0, int S = 1, int G = hist_group<Q>()>
 __device__ __forceinline__ void pcg_reorth_body(const Part &P, const PcgScalars *sc, const float *minv, float *Rh,
                                                 long stride, int k, const double *rzh, const double *cpart,
                                                 double *rzpart, const VBlock &b, PcgSmem &sm) {
@@ -233,7 +233,7 @@ __device__ __forceinline__ void pcg_reorth_body(const Part &P, const PcgScalars 
     double *red = sm.red;
     const int nb = b.nblk, lane = b.tid & 31, warp = b.tid >> 5;
     float *r = Rh + (long)(k + 1) * stride;
-    constexpr int NQ = Q > 0 ? Q : kQmax, G = hist_group<Q>();
+    constexpr int NQ = Q > 0 ? Q : kQmax;
     float4 x[Q > 0 ? G : 1][NQ];
     auto load_group = [&](int j0) {
 #pragma unroll
