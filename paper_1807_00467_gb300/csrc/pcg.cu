@@ -132,8 +132,8 @@ __global__ void __launch_bounds__(kVT, 2) pcg_dir_kernel(Part P, PcgScalars *sc,
 // blocks: longer vectors need more than a cluster's SMs for their history.
 // Groups of six residuals and 64 registers, so that two blocks share an SM: the
 // clusters of a batch's pairs compete for whole SMs (24 pairs of 96x96x48, 5
-// iterations of 20 PCG steps: 40.6 -> 39.3 ms, 39.7 as three launches; groups of
-// eight in one block an SM: the same for a lone small solve).
+// iterations of 20 PCG steps: 40.6 ms with groups of eight and one block an SM,
+// 39.3 so; a lone small solve takes the same time).
 template <int Q>
 __global__ void __launch_bounds__(kVT, 2) pcg_fused_kernel(Part P, PcgScalars *sc, const double *apart, int napart,
                                                      const float *q, const float *minv, float *Rh, long stride, int k,

@@ -25,11 +25,11 @@ __global__ void __launch_bounds__(NC / vcck::VccSmem<F>::kLanes, VM == 1 || size
 cudaError_t launch_vcc_cells(const VccArgs &a, cudaStream_t st) {
     dim3 grid(a.nb[0], a.nb[1], a.nb[2]);
     // Two cells per thread from more than one wave of one-cell blocks on (4 per
-    // SM): gradient 81 against 100 us and GN product 98 against 101 us at
-    // 129 x 129 x 65 nodes (8192 blocks), 38 / 46 and 45 / 47 us at 97 x 97 x 49
-    // (3456); below, one cell per thread has the shorter chain: 6.1 against
-    // 7.7 us at 17 x 17 x 13 (24 blocks), 7.7 / 8.1 us at 33 x 33 x 33 (256),
-    // equal at 576.  Both forms give the same bits.
+    // SM): gradient 88 against 105 us and GN product 97 against 103 us at
+    // 129 x 129 x 65 nodes (8192 blocks), 43 / 49 and 46 / 48 us at 97 x 97 x 49
+    // (3456); below, one cell per thread has the shorter chain: 8.4 against
+    // 10.5 us at 17 x 17 x 13 (24 blocks), 10.5 / 10.9 us at 33 x 33 x 33 (256).
+    // Both forms give the same bits.
     const bool two = (long)a.nb[0] * a.nb[1] * a.nb[2] > 4L * device_sm_count();
     if (a.diag) vcc_cell_kernel<2, float><<<grid, NC, 0, st>>>(a);
     else if (a.v && two) vcc_cell_kernel<1, float2><<<grid, NC / 2, 0, st>>>(a);

@@ -25,8 +25,8 @@
 // time over the block, instead of through per-cell slots and an indexed gather.
 // On large grids a thread holds two cells, one per half of the packed f32x2
 // registers (TZ / 2 planes apart, their nodes staged side by side), every
-// operation serving both.  Gradient 137 -> 87 us, GN product 107 -> 98 us at
-// 129 x 129 x 65 (gradient 81 us with the energies of four bounds added plainly
+// operation serving both.  Gradient 137 -> 88 us, GN product 107 -> 97 us at
+// 129 x 129 x 65 (gradient 82 us with the energies of four bounds added plainly
 // before the compensated sum: up to 1.4 units in the last place of a cell's
 // energy instead of one).  The reciprocal of the gradient is the approximate one
 // and a Newton step, correctly rounded for every mantissa while d and 1 / d are
@@ -128,17 +128,13 @@ __device__ __forceinline__ float rcp_approx(float d) {
 // w where d > 0, else 0: a fold has weight 0, whatever its other factors are
 __device__ __forceinline__ float if_pos(float d, float w) { return d > 0.f ? w : 0.f; }
 
-// d, or 1 where d is not positive (or NaN): psi(1) = psi'(1) = 0, and the cell has a fold
-__device__ __forceinline__ float unfold(float d, bool (&fold)[1]) {
-    const bool pos = d > 0.f;
-    fold[0] |= !pos;
-    return pos ? d : 1.f;
-}
-__device__ __forceinline__ float2 unfold(float2 d, bool (&fold)[2]) {
-    const bool p0 = d.x > 0.f, p1 = d.y > 0.f;
-    fold[0] |= !p0;
-    fold[1] |= !p1;
-    return make_float2(p0 ? d.x : 1.f, p1 ? d.y : 1.f);
+// d, or 1 where d is not positive (or NaN): psi(1) = psi'(1) = 0
+__device__ __forceinline__ float unfold(float d) { return d > 0.f ? d : 1.f; }
+// the smaller, NaN when either is
+__device__ __forceinline__ float min_nan(float a, float b) {
+    float r;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
 }
 
 // corner offset (ox + 2 oy + 4 oz) of edge e = p + 2 q of axis `ax` at end `hi`;
@@ -254,7 +250,7 @@ __device__ __forceinline__ void vcc_cell_body(const VccArgs &a, const VBlock &vb
             }
         }
     }
-    F en = zero, en_c = zero;                       // Kahan sum of psi(d)
+    F en = zero, en_c = zero;                       // Kahan sum of -psi(d), its next correction
     F dmn = bc_<F>(3.4e38f), dmx = bc_<F>(-3.4e38f);   // of the bounds that are numbers
     bool fold[CPT] = {};
     if constexpr (DG) {
@@ -305,11 +301,15 @@ __device__ __forceinline__ void vcc_cell_body(const VccArgs &a, const VBlock &vb
         for (int o = 0; o < 8; ++o) scatter(o, out[o][0], out[o][1], out[o][2]);
     } else {
         Vec<F> G1[4], G3[4];
-        // the 64 bounds; any: also bounds whose reciprocals the approximation flushes to 0 or inf
+        // The 64 bounds; any: also bounds whose reciprocals the approximation flushes
+        // to 0 or inf, and the least of bounds with NaN among them.  The gradient's
+        // sums are of -psi and -psi' (packed operations have no free negation).
         auto bounds = [&](auto any) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) G1[e] = G3[e] = Vec<F>{zero, zero, zero};
             en = en_c = zero;
+            dmn = bc_<F>(3.4e38f);
+            dmx = bc_<F>(-3.4e38f);
 #pragma unroll 1
             for (int b = 0; b < 4; ++b) {
                 const Vec<F> E2 = y_edge(sm.su, b, true), nE2 = neg_(E2);
@@ -336,22 +336,23 @@ __device__ __forceinline__ void vcc_cell_body(const VccArgs &a, const VBlock &vb
                     } else {
 #pragma unroll
                         for (int aa = 0; aa < 4; ++aa) {
-                            const F db = dot(E1[aa], X), d = unfold(db, fold), one = bc_<F>(1.f);
-                            dmn = lanes([](float p, float q) { return fminf(p, q); }, dmn, db);
+                            const F db = dot(E1[aa], X), d = lanes(unfold, db), one = bc_<F>(1.f);
+                            if constexpr (decltype(any)::value) dmn = lanes([](float p, float q) { return fminf(p, q); }, dmn, db);
+                            else dmn = lanes(min_nan, dmn, db);
                             dmx = lanes([](float p, float q) { return fmaxf(p, q); }, dmx, db);
-                            // 1 / d, correctly rounded (all mantissas tried); psi = (d - 1)^2 / d, psi' = 1 - 1 / d^2
-                            F rd;
+                            // nr = -1 / d, correctly rounded (all mantissas tried); psi = (d - 1)^2 / d, psi' = 1 - 1 / d^2
+                            F nr;
                             if constexpr (decltype(any)::value) {
-                                rd = lanes([](float x) { return __frcp_rn(x); }, d);
+                                nr = lanes([](float x) { return -__frcp_rn(x); }, d);
                             } else {
-                                const F r0 = lanes(rcp_approx, d);
-                                rd = fma_(r0, fma_(d, neg_(r0), one), r0);
+                                const F r0 = lanes([](float x) { return rcp_approx(-x); }, d);
+                                nr = fma_(r0, fma_(d, r0, one), r0);
                             }
-                            const F dm = sub_(d, one), q = mul_(dm, rd);
-                            const F y = fma_(dm, q, neg_(en_c)), t = add_(en, y);   // psi(d)
-                            en_c = sub_(sub_(t, en), y);
+                            const F nm = sub_(one, d), q = mul_(nm, nr);
+                            const F y = fma_(nm, q, en_c), t = add_(en, y);   // -psi(d)
+                            en_c = add_(sub_(en, t), y);
                             en = t;
-                            const F w = mul_(q, mul_(add_(d, one), rd));
+                            const F w = mul_(q, mul_(add_(d, one), nr));
                             axpy(w, X, G1[aa]);
                             axpy(w, E1[aa], W);
                         }
@@ -367,15 +368,23 @@ __device__ __forceinline__ void vcc_cell_body(const VccArgs &a, const VBlock &vb
         };
         bounds(std::false_type());
         if constexpr (!GN) {
-            auto beyond = [](float mn, float mx) { return (mn > 0.f && mn < 0x1p-126f) || mx >= 0x1p126f; };
+            // a fold is a bound that is not positive, or NaN: the least one tells
+            auto beyond = [](float mn, float mx) { return !(mn >= 0x1p-126f || mn <= 0.f) || mx >= 0x1p126f; };
             bool again;
-            if constexpr (CPT == 2) again = beyond(dmn.x, dmx.x) || beyond(dmn.y, dmx.y);
-            else again = beyond(dmn, dmx);
+            if constexpr (CPT == 2) {
+                fold[0] = !(dmn.x > 0.f);
+                fold[1] = !(dmn.y > 0.f);
+                again = beyond(dmn.x, dmx.x) || beyond(dmn.y, dmx.y);
+            } else {
+                fold[0] = !(dmn > 0.f);
+                again = beyond(dmn, dmx);
+            }
             if (again) bounds(std::true_type());   // (all cells with __frcp_rn: 162 against 123 us a call at 129 x 129 x 65)
         }
         // edge gradients onto the cell's corners, scaled by +-1/g of the edge's axis
-        // (times 2 for the GN product's halved weights): corner o is an end of one edge per axis
-        const float h = GN ? 2.f : 1.f, h0 = ig0 * h, h1 = ig1 * h, h2 = ig2 * h;
+        // (times 2 for the GN product's halved weights, -1 for the gradient's negated
+        // ones): corner o is an end of one edge per axis
+        const float h = GN ? 2.f : -1.f, h0 = ig0 * h, h1 = ig1 * h, h2 = ig2 * h;
         Vec<F> G2[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) G2[e] = Vec<F>{sm.g2[e * 3][tid], sm.g2[e * 3 + 1][tid], sm.g2[e * 3 + 2][tid]};
@@ -406,11 +415,11 @@ __device__ __forceinline__ void vcc_cell_body(const VccArgs &a, const VBlock &vb
         double e;
         float mn, mxv;
         if constexpr (CPT == 2) {
-            e = (valid0 ? (double)en.x - (double)en_c.x : 0.0) + (valid1 ? (double)en.y - (double)en_c.y : 0.0);
+            e = -((valid0 ? (double)en.x + (double)en_c.x : 0.0) + (valid1 ? (double)en.y + (double)en_c.y : 0.0));
             mn = fminf(valid0 ? dmn.x : 3.4e38f, valid1 ? dmn.y : 3.4e38f);
             mxv = fmaxf(valid0 ? dmx.x : -3.4e38f, valid1 ? dmx.y : -3.4e38f);
         } else {
-            e = valid0 ? (double)en - (double)en_c : 0.0;
+            e = valid0 ? -((double)en + (double)en_c) : 0.0;
             mn = valid0 ? dmn : 3.4e38f;
             mxv = valid0 ? dmx : -3.4e38f;
         }
