@@ -220,9 +220,10 @@ __device__ __forceinline__ void kp_warp_sum(const KpArgs &a, double two_delta, i
 // One thread per node (light or not) follows a chain of two dependent loads per
 // keypoint, one warp per node makes eight warps of every keypoint, of which most
 // find nothing to do.  The call, of which ~20 us are the other kernels, in a 65 x
-// 65 x 17 grid, by thread / by warp / so: 3000 keypoints along 30 vessels 45 / 30
-// / 32 us, 100000 spread evenly 69 / 155 / 62 us, 100000 along 30 vessels 675 /
-// 102 / 87 us.  rw leaves about 12000 warps, 80 per SM.
+// 65 x 17 grid, by thread / by warp / so: 100000 spread evenly 69 / 155 / 62 us,
+// 100000 along 30 vessels 675 / 102 / 87 us.  Up to 3072 keypoints a warp each
+// (3000 along 30 vessels: 45 by thread, 30 so, 32 with two a warp); above, rw
+// leaves 6000 to 12000 warps, up to 80 per SM.
 constexpr int kLight = 8;
 template <bool DIAG>
 __global__ void __launch_bounds__(256) kp_gather_kernel(const KpArgs a, int rw, double two_delta, float *out) {
@@ -266,7 +267,7 @@ __global__ void __launch_bounds__(256) kp_gather_kernel(const KpArgs a, int rw, 
 template <bool DIAG>
 static cudaError_t launch_gather(const KpArgs &a, double two_delta, float *out, cudaStream_t st) {
     int rw = 1;
-    while (rw < 32 && a.nk > 1536L * rw) rw *= 2;
+    while (rw < 32 && a.nk > (rw == 1 ? 3072L : 1536L * rw)) rw *= 2;
     kp_gather_kernel<DIAG><<<(a.nk + rw - 1) / rw, 256, 0, st>>>(a, rw, two_delta, out);
     return cudaGetLastError();
 }

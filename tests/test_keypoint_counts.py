@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 N, M = (128, 128, 64), (33, 33, 17)
 
 
-@pytest.mark.parametrize("nk", [1, 33, 1536, 1537, 6200, 12500, 24600, 50001])      # 1, 1, 1, 2, 8, 16, 32, 32 per warp
+@pytest.mark.parametrize("nk", [1, 33, 1537, 3072, 3073, 6200, 12500, 24600, 50001])      # 1, 1, 1, 1, 4, 8, 16, 32, 32 per warp
 def test_node_sums_are_exact(nk):
     import torch
     rng = np.random.default_rng(nk)
