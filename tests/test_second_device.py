@@ -78,6 +78,8 @@ print("solved")
 
 
 def test_wide_clusters_on_both_devices(tmp_path):
+    from paper_1807_00467_gb300 import build
+    build.build()
     include = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
     if not shutil.which("gcc") or not os.path.isdir(include):
         pytest.skip("needs gcc and the CUDA headers")
